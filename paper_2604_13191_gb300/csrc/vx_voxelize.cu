@@ -173,7 +173,6 @@ vx_status window_reduce(vx_context* ctx, bool fiber, uint32_t np, uint32_t nseg,
     seg.mass = (float*)(so + (size_t)nseg * 88);
     seg.key = k1;
     seg.nonzero = v1;
-    const unsigned rblocks = (unsigned)std::min<size_t>((nseg + RED_WARPS - 1) / RED_WARPS, (size_t)vx::kSMs * 32);
     VX_CUDA_TRY(cudaMemsetAsync(misc + 6, 0, 4, s));
     if (fiber) {
         // resident blocks (7 per SM) taking voxels from a counter
@@ -181,7 +180,9 @@ vx_status window_reduce(vx_context* ctx, bool fiber, uint32_t np, uint32_t nseg,
         VX_LAUNCH(ctx, ST_REDUCE_FIBERS, s, k_reduce_fibers<<<fblocks, RED_WARPS * 32, 0, s>>>(
                                                 k0, v0, starts, misc + 2, r0, r1, r2, seg, bx, by, bz, misc + 6));
     } else {
-        VX_LAUNCH(ctx, ST_REDUCE_TRIS, s, k_reduce_tris<<<rblocks, RED_WARPS * 32, 0, s>>>(
+        // resident blocks (5 per SM)
+        const unsigned tblocks = (unsigned)std::min<size_t>((nseg + RED_WARPS - 1) / RED_WARPS, (size_t)vx::kSMs * 5);
+        VX_LAUNCH(ctx, ST_REDUCE_TRIS, s, k_reduce_tris<<<tblocks, RED_WARPS * 32, 0, s>>>(
                                               k0, v0, starts, misc + 2, r0, r1, r2, seg, bx, by, bz, misc + 6));
     }
     VX_CUDA_TRY(cudaGetLastError());
