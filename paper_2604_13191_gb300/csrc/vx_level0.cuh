@@ -162,24 +162,6 @@ __device__ __forceinline__ AxisTerms axis_terms(float a, float b, int k) {
     return t;
 }
 
-// Per-axis bounds over a union of sub-cell intervals [lo, hi] on one axis:
-//   gap  <= the step-1 gap of every sub-cell inside (FP subtraction is monotone)
-//   farA >= the step-2 distance of endpoint a to every sub-cell inside, likewise farB.
-struct AxisBound {
-    float g2, fa2, fb2;
-};
-__device__ __forceinline__ AxisBound axis_bound(float a, float b, float lo, float hi) {
-    const float mn = fminf(a, b), mx = fmaxf(a, b);
-    const float g = gap3(lo, hi, mn, mx);
-    const float fa = fmaxf(hi - a, a - lo);
-    const float fb = fmaxf(hi - b, b - lo);
-    AxisBound r;
-    r.g2 = g * g;
-    r.fa2 = fa * fa;
-    r.fb2 = fb * fb;
-    return r;
-}
-
 // Per-warp pool of step-3 work of one voxel: (capsule slot, sub-cell) tasks left undecided
 // by steps 1-2 of the batch's capsules, those capsules, and the voxel's mask while the pool
 // is evaluated.  Tasks of many capsules are evaluated 32 at a time, so that the exact
@@ -194,14 +176,16 @@ struct CapsuleLocal {
 // lane): squared gap of the segment's extent, squared distances of the endpoints.
 struct CapsuleX {
     float4 g2[2], ea2[2], eb2[2];
-    float4 bx;                     // the voxel's x interval [0, 1]: gap^2, far_a^2, far_b^2
+};
+struct CapsuleSlot {
+    CapsuleLocal c;
+    CapsuleX x;
 };
 struct CapsuleTasks {
-    uint16_t task[CT_TASKS];       // batch slot << 9 | sub-cell id
-    uint32_t mask[16];             // 512-bit mask, word w = lanes 2w (low half) and 2w+1
+    CapsuleSlot slot[32];          // the batch's capsules (by lane)
     float q[32 * 7];               // w mu and w mu T(t) of up to 32 pairs (pair-major, stride 7)
-    CapsuleLocal batch[32];        // the batch's capsules (by lane)
-    CapsuleX xt[32];               // their x-axis terms
+    uint32_t mask[16];             // 512-bit mask, word w = lanes 2w (low half) and 2w+1
+    uint16_t task[CT_TASKS];       // batch slot << 9 | sub-cell id
 };
 
 __device__ __forceinline__ CapsuleX capsule_x(float a, float b) {
@@ -220,73 +204,86 @@ __device__ __forceinline__ CapsuleX capsule_x(float a, float b) {
     x.ea2[1] = make_float4(ea[4], ea[5], ea[6], ea[7]);
     x.eb2[0] = make_float4(eb[0], eb[1], eb[2], eb[3]);
     x.eb2[1] = make_float4(eb[4], eb[5], eb[6], eb[7]);
-    const AxisBound bx = axis_bound(a, b, 0.0f, 1.0f);
-    x.bx = make_float4(bx.g2, bx.fa2, bx.fb2, 0.0f);
     return x;
 }
 
-// Steps 1-2 of the capsule test for the 16 sub-cells of one lane (sx = 0..7,
-// sy = sy0 + (0|1), sz); bit b = sx + 8 (sy - sy0), so lane L holds bits 16L .. 16L+15 of
-// the voxel's 512-bit mask (bit id sx + 8 sy + 64 sz).  Bits already set in `have` are
-// skipped (OR is idempotent).  Returns `have` plus the bits step 1-2 decide set; `und`
-// receives the sub-cells left for step 3.
+// Steps 1-2 of the capsule test for one row of 8 sub-cells (sx = 0..7 at sy; tz: the z terms of
+// its slab).  `set` receives the sub-cells that step 2 decides set, `open` those that pass step 1.
 // Both steps compare the x term with what r^2 leaves after the y and z terms:
 //   step 1 fails  when  g_x^2 > r^2 - (g_y^2 + g_z^2),
 //   step 2 passes when  e_x^2 <= r^2 - (e_y^2 + e_z^2)  for endpoint a or b,
-// so a row's 8 sub-cells compare 8 x terms with one budget each.
-// A group of sub-cells (the lane's 16, or one row of 8) is decided at once when its per-axis
-// gap bounds fail step 1, or an endpoint's far bounds pass step 2: FP addition and
-// subtraction are monotone, so every sub-cell inside then fails (passes) too, and the group
-// result equals the per-sub-cell definition bit for bit.
-__device__ __forceinline__ uint32_t capsule_steps12(const CapsuleLocal& c, const CapsuleX& X, int sy0, int sz,
-                                                    uint32_t have, uint32_t& und) {
-    uint32_t bits = have;
-    und = 0;
-    if (have == 0xffffu) return bits;
-    const float a[3] = {c.a_rr.x, c.a_rr.y, c.a_rr.z}, b[3] = {c.b_reta.x, c.b_reta.y, c.b_reta.z};
-    const float rr = c.a_rr.w;
-    const float zlo = (float)sz * 0.125f, zhi = (float)(sz + 1) * 0.125f;
-    const AxisBound bz = axis_bound(a[2], b[2], zlo, zhi);
-    const float4 bxv = X.bx;
-    const AxisBound bx = {bxv.x, bxv.y, bxv.z};
-    const AxisBound bb = axis_bound(a[1], b[1], (float)sy0 * 0.125f, (float)(sy0 + 2) * 0.125f);
-    if (bx.g2 > rr - (bb.g2 + bz.g2)) return bits;                       // all 16 fail step 1
-    if (bx.fa2 <= rr - (bb.fa2 + bz.fa2) || bx.fb2 <= rr - (bb.fb2 + bz.fb2)) return 0xffffu;
-    const AxisTerms tz = axis_terms(a[2], b[2], sz);
+// so a row's 8 sub-cells compare 8 x terms with one budget each.  (e >= g on every axis, an
+// endpoint being no closer to a sub-cell than the segment's extent, and the operations are
+// monotone, so a set sub-cell is open too.)
+__device__ __forceinline__ void capsule_row(const CapsuleSlot& cs, const AxisTerms& tz, int sy, uint32_t& set,
+                                            uint32_t& open) {
+    const AxisTerms ty = axis_terms(cs.c.a_rr.y, cs.c.b_reta.y, sy);
+    const float rr = cs.c.a_rr.w;
+    const float TG = rr - (ty.g2 + tz.g2);
+    const float TA = rr - (ty.ea2 + tz.ea2);
+    const float TB = rr - (ty.eb2 + tz.eb2);
+    const CapsuleX& X = cs.x;
+    const float4 g0 = X.g2[0], g1 = X.g2[1], a0 = X.ea2[0], a1 = X.ea2[1], b0 = X.eb2[0], b1 = X.eb2[1];
+    const float xg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+    const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+    const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+    set = 0;
+    open = 0;
+#pragma unroll
+    for (int sx = 0; sx < 8; ++sx) {
+        set |= ((xa[sx] <= TA) || (xb[sx] <= TB) ? 1u : 0u) << sx;
+        open |= (xg[sx] <= TG ? 1u : 0u) << sx;
+    }
+}
+
+// The unset sub-cells of one lane's two rows: the centres of the first and last of each row.
+struct UnsetRows {
+    float lo[2], hi[2];
+};
+__device__ __forceinline__ UnsetRows unset_rows(uint32_t chunk) {
+    UnsetRows r;
 #pragma unroll
     for (int yi = 0; yi < 2; ++yi) {
-        const uint32_t rowmask = 0xffu << (8 * yi);
-        if ((bits & rowmask) == rowmask) continue;
-        const float ylo = (float)(sy0 + yi) * 0.125f, yhi = (float)(sy0 + yi + 1) * 0.125f;
-        const AxisBound by = axis_bound(a[1], b[1], ylo, yhi);
-        if (bx.g2 > rr - (by.g2 + bz.g2)) continue;
-        if (bx.fa2 <= rr - (by.fa2 + bz.fa2) || bx.fb2 <= rr - (by.fb2 + bz.fb2)) {
-            bits |= rowmask;
-            continue;
-        }
-        const AxisTerms ty = axis_terms(a[1], b[1], sy0 + yi);
-        const float TG = rr - (ty.g2 + tz.g2);
-        const float TA = rr - (ty.ea2 + tz.ea2);
-        const float TB = rr - (ty.eb2 + tz.eb2);
-        const float4 g0 = X.g2[0], g1 = X.g2[1], a0 = X.ea2[0], a1 = X.ea2[1], b0 = X.eb2[0], b1 = X.eb2[1];
-        const float xg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-        const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-        // per sub-cell: set when an endpoint passes step 2, open (step 3) when it passes
-        // step 1 only.  e >= g on every axis (an endpoint is no closer to a sub-cell than the
-        // segment's extent) and the operations are monotone, so a set sub-cell is open too;
-        // bits set before are dropped from `und` at the end.
-        uint32_t row_set = 0, row_open = 0;
-#pragma unroll
-        for (int sx = 0; sx < 8; ++sx) {
-            row_set |= ((xa[sx] <= TA) || (xb[sx] <= TB) ? 1u : 0u) << sx;
-            row_open |= (xg[sx] <= TG ? 1u : 0u) << sx;
-        }
-        bits |= row_set << (8 * yi);
-        und |= row_open << (8 * yi);
+        const uint32_t u = ~(chunk >> (8 * yi)) & 0xffu;   // (no meaning when the row is full)
+        r.lo[yi] = (float)(__ffs(u) - 1) * 0.125f + 0.0625f;
+        r.hi[yi] = (float)(31 - __clz(u)) * 0.125f + 0.0625f;
     }
-    und &= ~bits;
-    return bits;
+    return r;
+}
+
+// True unless the capsule is separated, by more than r + eta, from the box around the sub-cells
+// centred at x = lo..hi of the row (y, z): none of them can then be set (see
+// capsule_cell_separated).  The separation is taken along v, from the centre of the end
+// sub-cell that faces the capsule to the nearest point of its axis; the box reaches away from
+// that centre by half a sub-cell, and along x to the row's other end.  Any v gives a bound, so
+// neither the choice of the end nor the rounding of v matters; a NaN leaves the row open.
+__device__ __forceinline__ bool row_reached(const CapsuleLocal& c, float Az, float lo, float hi, float y) {
+    const float e = hi - lo;
+    const bool left = c.a_rr.x + c.b_reta.x < lo + hi;
+    const float Ax = c.a_rr.x - (left ? lo : hi), Ay = c.a_rr.y - y;
+    const float dx = c.d_idd.x, dy = c.d_idd.y, dz = c.d_idd.z;
+    const float tc = __saturatef(-c.d_idd.w * __fmaf_rn(Ax, dx, __fmaf_rn(Ay, dy, Az * dz)));
+    const float vx = __fmaf_rn(tc, dx, Ax), vy = __fmaf_rn(tc, dy, Ay), vz = __fmaf_rn(tc, dz, Az);
+    const float sa = __fmaf_rn(vx, Ax, __fmaf_rn(vy, Ay, vz * Az));
+    const float sb = __fmaf_rn(vx, dx, __fmaf_rn(vy, dy, __fmaf_rn(vz, dz, sa)));
+    const float beyond = fmaxf((left ? e : -e) * vx, 0.0f);
+    const float sep = fminf(sa, sb) - __fmaf_rn(0.0625f, (fabsf(vx) + fabsf(vy)) + fabsf(vz), beyond);
+    const float vv = __fmaf_rn(vx, vx, __fmaf_rn(vy, vy, vz * vz));
+    return !(sep * fabsf(sep) > (c.b_reta.w * c.b_reta.w) * vv);
+}
+
+// True when an endpoint of the capsule is within r of every point of the voxel: step 2 then
+// passes for each of its sub-cells (the far bounds are no smaller than a sub-cell's endpoint
+// distance on any axis, and the operations are monotone).
+__device__ __forceinline__ bool capsule_covers(const float* a, const float* b, float rr) {
+    float fa2[3], fb2[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float fa = fmaxf(1.0f - a[i], a[i] - 0.0f), fb = fmaxf(1.0f - b[i], b[i] - 0.0f);
+        fa2[i] = fa * fa;
+        fb2[i] = fb * fb;
+    }
+    return fa2[0] <= rr - (fa2[1] + fa2[2]) || fb2[0] <= rr - (fb2[1] + fb2[2]);
 }
 
 // Local capsule of endpoints a, b (voxel-local grid units) and radius r.  eta bounds, with
@@ -356,7 +353,7 @@ __device__ __forceinline__ uint32_t capsule_step3_pool(CapsuleTasks& ct, int nta
         if (t < ntask) {
             task = ct.task[t];
             const int id = (int)(task & 511u);
-            keep = !(ct.mask[id >> 5] & (1u << (id & 31))) && !capsule_cell_separated(ct.batch[task >> 9], id);
+            keep = !(ct.mask[id >> 5] & (1u << (id & 31))) && !capsule_cell_separated(ct.slot[task >> 9].c, id);
         }
         const uint32_t kept = __ballot_sync(0xffffffffu, keep);
         __syncwarp();   // the chunk is read before any lane writes (writes land at or below it)
@@ -369,7 +366,7 @@ __device__ __forceinline__ uint32_t capsule_step3_pool(CapsuleTasks& ct, int nta
         const int id = (int)(task & 511u);
         const uint32_t bit = 1u << (id & 31);
         if (ct.mask[id >> 5] & bit) continue;
-        const CapsuleLocal& c = ct.batch[task >> 9];
+        const CapsuleLocal& c = ct.slot[task >> 9].c;
         const int sx = id & 7, sy = (id >> 3) & 7, zz = id >> 6;
         if (seg_box_min(c.a_rr.x, c.a_rr.y, c.a_rr.z, c.d_idd.x, c.d_idd.y, c.d_idd.z, (float)sx * 0.125f,
                         (float)sy * 0.125f, (float)zz * 0.125f, 0.125f) <= c.a_rr.w)
@@ -742,23 +739,6 @@ __global__ void k_prep_fibers(const float4* __restrict__ ctrl, int64_t num_ctrl,
     rb[p] = B;
 }
 
-// The tangent terms of each capsule's moment, T = (t_x^2, t_y^2, t_z^2, t_x t_y, t_x t_z,
-// t_y t_z) with t = (B - A) / |B - A| (zero for a degenerate segment), as two float4 per
-// primitive (the last two lanes zero).  These are the operations the reduce applied to every
-// candidate pair; they depend on the primitive only, so they run once per primitive.
-__global__ void k_tangent_terms(const float4* __restrict__ ra, const float4* __restrict__ rb, uint32_t np,
-                                float4* __restrict__ rt) {
-    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    const float4 A = ra[p], B = rb[p];
-    const float dg[3] = {B.x - A.x, B.y - A.y, B.z - A.z};
-    const float dn = sqrtf((dg[0] * dg[0] + dg[1] * dg[1]) + dg[2] * dg[2]);
-    float t[3] = {0.0f, 0.0f, 0.0f};
-    if (dn > 0.0f) { t[0] = dg[0] / dn; t[1] = dg[1] / dn; t[2] = dg[2] / dn; }
-    rt[2 * (size_t)p] = make_float4(t[0] * t[0], t[1] * t[1], t[2] * t[2], t[0] * t[1]);
-    rt[2 * (size_t)p + 1] = make_float4(t[0] * t[2], t[1] * t[2], 0.0f, 0.0f);
-}
-
 // tri records: (U0, w), (U1, 0), (U2, 0)
 __global__ void k_prep_tris(const float4* __restrict__ tv, const float* __restrict__ weights, uint32_t np, GridDev g,
                             float4* __restrict__ r0, float4* __restrict__ r1, float4* __restrict__ r2,
@@ -980,200 +960,246 @@ __device__ __forceinline__ void write_mask(SegOut out, uint32_t seg, uint32_t ke
     }
 }
 
-// The same with the voxel's sums, spread over lanes 0..6 (lane c: component c).
-__device__ __forceinline__ void write_seg7(SegOut out, uint32_t seg, uint32_t key, uint32_t chunk, float accc) {
-    const int lane = threadIdx.x & 31;
-    write_mask(out, seg, key, chunk);
-    if (lane == 0) out.mass[seg] = accc;
-    else if (lane < 7) out.moment[(size_t)seg * 6 + lane - 1] = accc;
+// The measure and moment terms of capsule A-B (grid units) in the voxel that has it at a-b: w mu
+// and w mu T(t), t = (B - A) / |B - A| (zero for a degenerate segment), into q[0..6].
+__device__ __forceinline__ void capsule_moments(float4 A, float4 B, const float* a, const float* b, float* q) {
+    const float mu = capsule_measure(a, b, A.w);
+    const float dg[3] = {B.x - A.x, B.y - A.y, B.z - A.z};
+    const float dn = sqrtf((dg[0] * dg[0] + dg[1] * dg[1]) + dg[2] * dg[2]);
+    float t[3] = {0.0f, 0.0f, 0.0f};
+    if (dn > 0.0f) { t[0] = dg[0] / dn; t[1] = dg[1] / dn; t[2] = dg[2] / dn; }
+    const float c = B.w * mu;
+    q[0] = c;
+    q[1] = c * (t[0] * t[0]);
+    q[2] = c * (t[1] * t[1]);
+    q[3] = c * (t[2] * t[2]);
+    q[4] = c * (t[0] * t[1]);
+    q[5] = c * (t[0] * t[2]);
+    q[6] = c * (t[1] * t[2]);
 }
 
-// Batch slot `lane` of a voxel at (fx, fy, fz): capsule p's local record, the x terms of its
-// steps 1-2 and its w mu, w mu T(t) moment terms, in the warp's shared state.  Returns the
-// key that orders the mask tests: capsules whose axis passes deepest into the voxel first
-// (they set the most bits, so later capsules find more lanes already full).  The mask is an
-// OR, so the order does not change it.
-__device__ __forceinline__ uint32_t capsule_slot_setup(CapsuleTasks& ct, int lane, uint32_t p, float fx, float fy,
-                                                       float fz, const float4* __restrict__ ra,
-                                                       const float4* __restrict__ rb,
-                                                       const float4* __restrict__ rt) {
-    const float4 A = ra[p], B = rb[p];
-    float a[3] = {A.x - fx, A.y - fy, A.z - fz};
-    float b[3] = {B.x - fx, B.y - fy, B.z - fz};
-    const CapsuleLocal cl = capsule_local(a, b, A.w);
-    ct.batch[lane] = cl;
-    ct.xt[lane] = capsule_x(a[0], b[0]);
-    uint32_t okey;
-    {
-        // squared distance from the voxel centre to the axis, minus r^2 (an ordering key only:
-        // any rounding of it leaves the outputs unchanged)
-        const float e[3] = {cl.d_idd.x, cl.d_idd.y, cl.d_idd.z};
-        const float w[3] = {0.5f - a[0], 0.5f - a[1], 0.5f - a[2]};
-        float tt = ((w[0] * e[0] + w[1] * e[1]) + w[2] * e[2]) * cl.d_idd.w;
-        tt = fminf(fmaxf(tt, 0.0f), 1.0f);
-        const float dx = w[0] - tt * e[0], dy = w[1] - tt * e[1], dz = w[2] - tt * e[2];
-        const float v = ((dx * dx + dy * dy) + dz * dz) - A.w * A.w;
-        uint32_t bits = __float_as_uint(v);
-        bits ^= (bits >> 31) ? 0xffffffffu : 0x80000000u;   // order-preserving as unsigned
-        okey = (min(bits, 0xffffffbfu) & 0xffffffe0u) | (uint32_t)lane;   // below the empty lanes
-    }
-    const float mu = capsule_measure(a, b, A.w);
-    // w mu and w mu T(t), T the primitive's tangent terms (k_tangent_terms)
-    const float4 T0 = rt[2 * (size_t)p], T1 = rt[2 * (size_t)p + 1];
-    const float c = B.w * mu;
-    float* q = ct.q + lane * 7;
-    q[0] = c;
-    q[1] = c * T0.x;
-    q[2] = c * T0.y;
-    q[3] = c * T0.z;
-    q[4] = c * T0.w;
-    q[5] = c * T1.x;
-    q[6] = c * T1.y;
-    return okey;
+// The key that orders the mask tests of a voxel's capsules: those whose axis passes deepest into
+// the voxel first (they set the most bits, so later capsules find more rows full or out of
+// reach).  The mask is an OR, so neither the order nor any rounding of the key changes it.
+__device__ __forceinline__ uint32_t capsule_order(const CapsuleLocal& cl) {
+    const float e[3] = {cl.d_idd.x, cl.d_idd.y, cl.d_idd.z};
+    const float w[3] = {0.5f - cl.a_rr.x, 0.5f - cl.a_rr.y, 0.5f - cl.a_rr.z};
+    float tt = ((w[0] * e[0] + w[1] * e[1]) + w[2] * e[2]) * cl.d_idd.w;
+    tt = fminf(fmaxf(tt, 0.0f), 1.0f);
+    const float dx = w[0] - tt * e[0], dy = w[1] - tt * e[1], dz = w[2] - tt * e[2];
+    const float v = ((dx * dx + dy * dy) + dz * dz) - cl.a_rr.w;
+    const uint32_t bits = __float_as_uint(v);
+    return bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);   // order-preserving as unsigned
 }
 
 // Steps 1-3 of the `cnt` capsules of one voxel whose ordering keys sit at lanes src0,
-// src0 + dir, ... of `okey` (the batch slot is a key's low 5 bits), on top of the lane's
-// 16-bit chunk of the mask.  The pooled step-3 tasks refer to this batch's slots, so they
-// are evaluated before the function returns.
-__device__ __forceinline__ uint32_t voxel_mask(CapsuleTasks& ct, uint32_t okey, uint32_t cnt, int src0, int dir,
-                                               int sy0, int sz, uint32_t chunk, bool& full) {
+// src0 + 1, ... of `okey` (the batch slot is a key's low 5 bits), on top of the lane's 16-bit
+// chunk of the mask (lane L: rows sy0, sy0 + 1 of slab sz).  A row whose unset sub-cells are all
+// out of the capsule's reach is passed over; most capsules reach no such row in the whole
+// voxel.  The pooled step-3 tasks refer to this batch's slots, so they are evaluated before the
+// function returns.
+__device__ __forceinline__ uint32_t voxel_mask(CapsuleTasks& ct, uint32_t okey, uint32_t cnt, int src0, int sy0, int sz,
+                                               uint32_t chunk, bool& full) {
     const int lane = threadIdx.x & 31;
+    const float y0 = (float)sy0 * 0.125f + 0.0625f, zc = (float)sz * 0.125f + 0.0625f;
+    UnsetRows ur = unset_rows(chunk);
     int ntask = 0;
     for (uint32_t j = 0; j < cnt; ++j) {
         if (full) break;
-        const int slot = (int)(__shfl_sync(0xffffffffu, okey, src0 + dir * (int)j) & 31u);
-        uint32_t und;
-        chunk = capsule_steps12(ct.batch[slot], ct.xt[slot], sy0, sz, chunk, und);
-        // pool the undecided sub-cells as step-3 tasks of this capsule
-        if (__any_sync(0xffffffffu, und != 0u)) {
-            const uint32_t n = __popc(und);
-            uint32_t off = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, off, o);
-                if (lane >= o) off += t;
-            }
-            const int total = (int)__shfl_sync(0xffffffffu, off, 31);
-            if (ntask + total > CT_TASKS) {
+        const int slot = (int)(__shfl_sync(0xffffffffu, okey, src0 + (int)j) & 31u);
+        const CapsuleSlot& cs = ct.slot[slot];
+        const float Az = cs.c.a_rr.z - zc;
+        const bool p0 = (chunk & 0xffu) != 0xffu && row_reached(cs.c, Az, ur.lo[0], ur.hi[0], y0);
+        const bool p1 = (chunk & 0xff00u) != 0xff00u && row_reached(cs.c, Az, ur.lo[1], ur.hi[1], y0 + 0.125f);
+        if (!__any_sync(0xffffffffu, p0 || p1)) continue;
+        const AxisTerms tz = axis_terms(cs.c.a_rr.z, cs.c.b_reta.z, sz);
+        uint32_t set = 0, open = 0;
+        if (__any_sync(0xffffffffu, p0)) {
+            uint32_t rs, ro;
+            capsule_row(cs, tz, sy0, rs, ro);
+            if (p0) { set = rs; open = ro; }
+        }
+        if (__any_sync(0xffffffffu, p1)) {
+            uint32_t rs, ro;
+            capsule_row(cs, tz, sy0 + 1, rs, ro);
+            if (p1) { set |= rs << 8; open |= ro << 8; }
+        }
+        const uint32_t before = chunk;
+        chunk |= set;
+        // pool the undecided sub-cells as step-3 tasks of this capsule, one per lane and turn
+        uint32_t und = open & ~chunk;
+        for (uint32_t bal; (bal = __ballot_sync(0xffffffffu, und != 0u)) != 0u;) {
+            if (ntask + 32 > CT_TASKS) {
+                __syncwarp();
                 chunk = capsule_step3_pool(ct, ntask, chunk);
                 ntask = 0;
+                und &= ~chunk;
+                continue;
             }
-            uint32_t pos = (uint32_t)ntask + off - n;
-            uint32_t u = und;
-            while (u) {
-                const int bpos = __ffs(u) - 1;
-                u &= u - 1;
-                ct.task[pos++] = (uint16_t)((slot << 9) | (16 * lane + bpos));
+            if (und) {
+                const int bpos = __ffs(und) - 1;
+                und &= und - 1;
+                ct.task[ntask + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((slot << 9) | (16 * lane + bpos));
             }
-            ntask += total;
-            __syncwarp();
+            ntask += __popc(bal);
         }
-        full = __all_sync(0xffffffffu, chunk == 0xffffu);
+        if (__any_sync(0xffffffffu, chunk != before)) {
+            ur = unset_rows(chunk);
+            full = __all_sync(0xffffffffu, chunk == 0xffffu);
+        }
     }
+    __syncwarp();
     if (ntask > 0 && !full) chunk = capsule_step3_pool(ct, ntask, chunk);
     return chunk;
 }
 
-// Voxel origin (grid units) of a window-relative Morton key.
-__device__ __forceinline__ void voxel_origin(uint32_t key, int bx, int by, int bz, float& fx, float& fy, float& fz) {
-    fx = (float)((int)vx_compact1by2(key) + bx);
-    fy = (float)((int)vx_compact1by2(key >> 1) + by);
-    fz = (float)((int)vx_compact1by2(key >> 2) + bz);
-}
-
-// Warp per candidate voxel, four voxels per step.  The step's voxels form groups of
-// consecutive voxels whose capsules fit one batch (at most 32 together), and one setup serves
-// a group: lane l takes the group's l-th capsule (the capsules of consecutive voxels are
-// consecutive in the sorted pairs), the sums of voxel u run on lanes 7u .. 7u+6, and one
-// ordering sort with the voxel above the distance key leaves each voxel's capsules together,
-// in voxel order; then the mask steps run voxel by voxel.  A voxel of more than 32 capsules
-// is a group of its own and runs in batches of 32.  The setup, the mask steps and the output
-// each have one call site, so that the kernel holds one copy of them.
+// Warp per candidate voxel, up to eight voxels per step (fewer when the grid's warps would
+// otherwise run out of voxels).  The step's voxels form groups of consecutive voxels whose
+// capsules fit one batch (at most 32 together), and one setup serves a group: lane l takes the
+// group's l-th pair.
+//   - A capsule whose axis misses the voxel has measure 0 (few cross it: a capsule is a candidate
+//     of every voxel that its radius reaches), so the measures and the sums run over the
+//     others only.  Adding the zeros would not change an FP32 sum.
+//   - A voxel with a capsule that covers it whole is full, and needs no mask steps.
+//   - The rest are ordered by one sort of the batch with the voxel above the distance key, which
+//     leaves each voxel's capsules together, and their mask steps run voxel by voxel.
+// A voxel of more than 32 capsules is a group of its own and runs in batches of 32.  The setup
+// and the mask steps each have one call site, so that the kernel holds one copy of them.
 __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint32_t* __restrict__ keys,
                                                                   const uint32_t* __restrict__ prims,
                                                                   const uint32_t* __restrict__ starts,
                                                                   const uint32_t* __restrict__ nseg_p,
                                                                   const float4* __restrict__ ra,
-                                                                  const float4* __restrict__ rb,
-                                                                  const float4* __restrict__ rt, SegOut out,
-                                                                  int bx, int by, int bz,
-                                                                  uint32_t* __restrict__ next) {
-    constexpr uint32_t STEP = 4;   // voxels per warp step (a group's voxel index takes 2 bits)
+                                                                  const float4* __restrict__ rb, SegOut out, int bx,
+                                                                  int by, int bz, uint32_t* __restrict__ next) {
+    constexpr uint32_t STEP = 8;   // voxels per warp step (a group's voxel index takes 3 bits)
     const int lane = threadIdx.x & 31;
     const uint32_t nseg = *nseg_p;
     const int sz = lane >> 2, sy0 = (lane & 3) * 2;
-    const uint32_t warps = gridDim.x * RED_WARPS;
     __shared__ CapsuleTasks pool[RED_WARPS];
     CapsuleTasks& ct = pool[threadIdx.x >> 5];
-    // voxels are taken STEP at a time from the counter `next` when it is given (a grid of
-    // resident blocks), else in a fixed grid stride
-    auto take = [&]() -> uint32_t {
-        uint32_t v = 0;
-        if (lane == 0) v = atomicAdd(next, STEP);
-        return __shfl_sync(0xffffffffu, v, 0);
-    };
-    for (uint32_t s0 = next ? take() : STEP * (blockIdx.x * RED_WARPS + (threadIdx.x >> 5)); s0 < nseg;
-         s0 = next ? take() : s0 + STEP * warps) {
-        const uint32_t s_end = min(s0 + STEP, nseg);
-        for (uint32_t g = s0; g < s_end;) {
-            // the group [g, g + m): consecutive voxels of at most 32 capsules together, or one voxel
-            const uint32_t gbeg = starts[g];
-            uint32_t m = 1, gend = starts[g + 1];
-            while (g + m < s_end) {
-                const uint32_t nx = starts[g + m + 1];
-                if (nx - gbeg > 32u) break;
-                gend = nx;
-                ++m;
-            }
+    const uint32_t step = max(1u, min(STEP, nseg / (gridDim.x * RED_WARPS)));
+    for (;;) {
+        uint32_t s0 = 0;
+        if (lane == 0) s0 = atomicAdd(next, step);
+        s0 = __shfl_sync(0xffffffffu, s0, 0);
+        if (s0 >= nseg) break;
+        const uint32_t nv = min(step, nseg - s0);
+        // lane i holds the first pair of voxel s0 + i (lane nv the end of the last one)
+        const uint32_t st = starts[s0 + min((uint32_t)lane, nv)];
+        for (uint32_t g = 0; g < nv;) {
+            const uint32_t gbeg = __shfl_sync(0xffffffffu, st, g);
+            // the group [g, g + m): as many voxels as end within 32 pairs, at least one
+            const uint32_t fit = __ballot_sync(0xffffffffu, (uint32_t)lane > g && (uint32_t)lane <= nv && st - gbeg <= 32u);
+            const uint32_t m = max(1u, (uint32_t)__popc(fit));
+            const uint32_t gend = __shfl_sync(0xffffffffu, st, g + m);
             uint32_t chunk = 0;
             bool full = false;
-            float accc = 0.0f;   // lane 7u + c: component c of voxel u's sums
+            float accc = 0.0f;   // one voxel's sums, lane c < 7: component c
             for (uint32_t base = gbeg; base < gend; base += 32) {
                 const uint32_t cnt = min(32u, gend - base);
-                // the lane's voxel in the group, and its origin
-                uint32_t v = 0;
-                for (uint32_t t = 1; t < m; ++t) v += (base + (uint32_t)lane >= starts[g + t]) ? 1u : 0u;
-                float fx, fy, fz;
-                voxel_origin(keys[starts[g + v]], bx, by, bz, fx, fy, fz);
-                __syncwarp();   // the previous batch's sums have read ct.q
-                uint32_t okey = 0xffffffe0u | (uint32_t)lane;
+                // the lane's voxel in the group and that voxel's lanes [vb, ve)
+                uint32_t v = 0, vb = 0, ve = cnt;
+                for (uint32_t t = 1; t < m; ++t) {
+                    const uint32_t e = __shfl_sync(0xffffffffu, st, g + t) - base;
+                    if ((uint32_t)lane >= e) { v = t; vb = e; }
+                    else ve = min(ve, e);
+                }
+                __syncwarp();   // the previous batch's sums and masks have read the shared state
+                uint32_t key = 0, okey = 0xffffffe0u | (uint32_t)lane;
+                bool covers = false, sums = false;
+                float a[3], b[3];
+                float4 A = make_float4(0, 0, 0, 0), B = A;
                 if ((uint32_t)lane < cnt) {
-                    okey = capsule_slot_setup(ct, lane, prims[base + lane], fx, fy, fz, ra, rb, rt);
-                    // the voxel above the distance key (still below the empty lanes' keys)
-                    if (m > 1) okey = (v << 30) | ((okey >> 2) & 0x3fffffc0u) | (uint32_t)lane;
-                }
-                __syncwarp();
-                // sums in primitive order, one component per lane (the same sequence of FP32
-                // additions as a single running sum per component); all voxels at once
-                if ((uint32_t)lane < 7u * m) {
-                    const uint32_t u = (uint32_t)lane / 7u;
-                    const uint32_t ub = m > 1 ? starts[g + u] - base : 0u;
-                    const uint32_t un = m > 1 ? starts[g + u + 1] - starts[g + u] : cnt;
-                    const float* q = ct.q + ub * 7 + ((uint32_t)lane - 7u * u);
-                    for (uint32_t j = 0; j < un; ++j) accc = accc + q[j * 7];
-                }
-                // bitonic sort of the keys (unique: the lane is the low 5 bits); after the
-                // stage of width k, lanes 0..k-1 hold their keys in ascending order, so the sort
-                // stops once k covers the batch
+                    key = keys[base + lane];
+                    const uint32_t p = prims[base + lane];
+                    A = ra[p];
+                    B = rb[p];
+                    const float f[3] = {(float)((int)vx_compact1by2(key) + bx), (float)((int)vx_compact1by2(key >> 1) + by),
+                                        (float)((int)vx_compact1by2(key >> 2) + bz)};
+                    a[0] = A.x - f[0]; a[1] = A.y - f[1]; a[2] = A.z - f[2];
+                    b[0] = B.x - f[0]; b[1] = B.y - f[1]; b[2] = B.z - f[2];
+                    covers = capsule_covers(a, b, A.w * A.w);
+                    // with both ends beyond one face the clip is empty: one of its parameters is
+                    // at least 1 (or at most 0) after rounding too, since |b - a| is then no
+                    // larger than the distance of the farther end to that face
+                    bool out_ = false;
 #pragma unroll
-                for (int k = 2; k <= 32; k <<= 1) {
+                    for (int i = 0; i < 3; ++i) out_ = out_ || (a[i] < 0.0f && b[i] < 0.0f) || (a[i] > 1.0f && b[i] > 1.0f);
+                    // (an infinite B - A has no tangent: its terms are not finite and are kept)
+                    out_ = out_ && fmax3(fabsf(B.x - A.x), fabsf(B.y - A.y), fabsf(B.z - A.z)) < INFINITY;
+                    if (!out_) {
+                        float* q = ct.q + lane * 7;
+                        capsule_moments(A, B, a, b, q);
 #pragma unroll
-                    for (int jj = k >> 1; jj > 0; jj >>= 1) {
-                        const uint32_t other = __shfl_xor_sync(0xffffffffu, okey, jj);
-                        const bool keep_min = ((lane & k) == 0) == ((lane & jj) == 0);
-                        okey = keep_min ? min(okey, other) : max(okey, other);
+                        for (int c = 0; c < 7; ++c) sums = sums || q[c] != 0.0f;
                     }
-                    if ((uint32_t)k >= cnt) break;
                 }
-                // the mask steps, voxel by voxel; a voxel's outputs once its last batch is in
+                const uint32_t summed = __ballot_sync(0xffffffffu, sums);
+                const uint32_t cover = __ballot_sync(0xffffffffu, covers);
+                const uint32_t vlanes = (ve > 31u ? 0xffffffffu : (1u << ve) - 1u) & ~((1u << vb) - 1u);
+                const bool live = (uint32_t)lane < cnt && (cover & vlanes) == 0u;
+                __syncwarp();
+                // sums in primitive order, one component of one voxel per lane (the same sequence
+                // of FP32 additions as a single running sum per component)
+                if (m > 1) {
+                    for (uint32_t it0 = 0; it0 < 7u * m; it0 += 32) {
+                        const uint32_t it = it0 + (uint32_t)lane, u = min(it / 7u, m - 1u), c = it - 7u * u;
+                        const uint32_t ub = __shfl_sync(0xffffffffu, st, g + u) - base;
+                        const uint32_t ue = __shfl_sync(0xffffffffu, st, g + u + 1) - base;
+                        if (it < 7u * m) {
+                            float acc = 0.0f;
+                            for (uint32_t w = summed & (ue > 31u ? 0xffffffffu : (1u << ue) - 1u) & ~((1u << ub) - 1u); w;
+                                 w &= w - 1u)
+                                acc = acc + ct.q[(__ffs(w) - 1) * 7 + c];
+                            if (c == 0) out.mass[s0 + g + u] = acc;
+                            else out.moment[(size_t)(s0 + g + u) * 6 + c - 1] = acc;
+                        }
+                    }
+                } else if (lane < 7) {
+                    for (uint32_t w = summed; w; w &= w - 1u) accc = accc + ct.q[(__ffs(w) - 1) * 7 + lane];
+                }
+                // the mask steps' slots and their order, for the voxels that need them
+                if (__any_sync(0xffffffffu, live && !full)) {
+                    if (live) {
+                        const CapsuleLocal cl = capsule_local(a, b, A.w);
+                        ct.slot[lane].c = cl;
+                        ct.slot[lane].x = capsule_x(a[0], b[0]);
+                        okey = capsule_order(cl);
+                    }
+                    // the voxel in the top bits (every key of a lane in use below the others')
+                    if ((uint32_t)lane < cnt) okey = (v << 29) | (min(okey >> 3, 0x1fffffbfu) & 0x1fffffe0u) | (uint32_t)lane;
+                    __syncwarp();
+                    // bitonic sort of the keys (unique: the lane is the low 5 bits); after the
+                    // stage of width k, lanes 0..k-1 hold their keys in ascending order, so the sort
+                    // stops once k covers the batch
+#pragma unroll
+                    for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+                        for (int jj = k >> 1; jj > 0; jj >>= 1) {
+                            const uint32_t other = __shfl_xor_sync(0xffffffffu, okey, jj);
+                            const bool keep_min = ((lane & k) == 0) == ((lane & jj) == 0);
+                            okey = keep_min ? min(okey, other) : max(okey, other);
+                        }
+                        if ((uint32_t)k >= cnt) break;
+                    }
+                }
+                // voxel by voxel; a voxel's outputs once its last batch is in
                 for (uint32_t u = 0; u < m; ++u) {
-                    const uint32_t ub = m > 1 ? starts[g + u] - base : 0u;
-                    const uint32_t un = m > 1 ? starts[g + u + 1] - starts[g + u] : cnt;
-                    chunk = voxel_mask(ct, okey, un, (int)ub, 1, sy0, sz, chunk, full);
+                    const uint32_t ub = m > 1 ? __shfl_sync(0xffffffffu, st, g + u) - base : 0u;
+                    const uint32_t ue = m > 1 ? __shfl_sync(0xffffffffu, st, g + u + 1) - base : cnt;
+                    const uint32_t lanes = (ue > 31u ? 0xffffffffu : (1u << ue) - 1u) & ~((1u << ub) - 1u);
+                    if (cover & lanes) {
+                        chunk = 0xffffu;
+                        full = true;
+                    }
+                    if (!full) chunk = voxel_mask(ct, okey, ue - ub, (int)ub, sy0, sz, chunk, full);
                     if (m > 1 || base + cnt >= gend) {
-                        write_seg7(out, g + u, keys[starts[g + u]], chunk,
-                                   __shfl_down_sync(0xffffffffu, accc, 7 * u));
+                        write_mask(out, s0 + g + u, __shfl_sync(0xffffffffu, key, ub), chunk);
+                        if (m == 1 && lane < 7) {
+                            if (lane == 0) out.mass[s0 + g] = accc;
+                            else out.moment[(size_t)(s0 + g) * 6 + lane - 1] = accc;
+                        }
                         chunk = 0;
                         full = false;
                     }
