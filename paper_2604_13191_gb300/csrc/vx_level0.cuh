@@ -168,7 +168,7 @@ __device__ __forceinline__ AxisTerms axis_terms(float a, float b, int k) {
 // minimum (the expensive case) runs with all lanes busy.
 constexpr int CT_TASKS = 512;
 // One capsule in voxel-local grid units: (a.xyz, r^2), (b.xyz, r + eta), (d = b - a, 1 / |d|^2)
-// with eta the margin of capsule_cell_separated.
+// with eta the margin of capsule_cell_quick.
 struct CapsuleLocal {
     float4 a_rr, b_reta, d_idd;
 };
@@ -236,40 +236,61 @@ __device__ __forceinline__ void capsule_row(const CapsuleSlot& cs, const AxisTer
     }
 }
 
-// The unset sub-cells of one lane's two rows: the centres of the first and last of each row.
+// The unset sub-cells of one lane's two rows, as packed pairs (row sy0, row sy0 + 1): the centres
+// of each row's first and last one, negated, and their sum.
 struct UnsetRows {
-    float lo[2], hi[2];
+    f2 nlo, nhi, sum;
 };
 __device__ __forceinline__ UnsetRows unset_rows(uint32_t chunk) {
-    UnsetRows r;
+    float lo[2], hi[2];
 #pragma unroll
     for (int yi = 0; yi < 2; ++yi) {
         const uint32_t u = ~(chunk >> (8 * yi)) & 0xffu;   // (no meaning when the row is full)
-        r.lo[yi] = (float)(__ffs(u) - 1) * 0.125f + 0.0625f;
-        r.hi[yi] = (float)(31 - __clz(u)) * 0.125f + 0.0625f;
+        lo[yi] = (float)(__ffs(u) - 1) * 0.125f + 0.0625f;
+        hi[yi] = (float)(31 - __clz(u)) * 0.125f + 0.0625f;
     }
-    return r;
+    return {f2_pack(-lo[0], -lo[1]), f2_pack(-hi[0], -hi[1]), f2_pack(lo[0] + hi[0], lo[1] + hi[1])};
 }
 
-// True unless the capsule is separated, by more than r + eta, from the box around the sub-cells
-// centred at x = lo..hi of the row (y, z): none of them can then be set (see
-// capsule_cell_separated).  The separation is taken along v, from the centre of the end
+// Per row (reach0: y, reach1: y + 1/8), true unless the capsule is separated, by more than r + eta,
+// from the box around the row's unset sub-cells: none of them can then be set (see
+// capsule_cell_quick).  The separation is taken along v, from the centre of the end
 // sub-cell that faces the capsule to the nearest point of its axis; the box reaches away from
 // that centre by half a sub-cell, and along x to the row's other end.  Any v gives a bound, so
 // neither the choice of the end nor the rounding of v matters; a NaN leaves the row open.
-__device__ __forceinline__ bool row_reached(const CapsuleLocal& c, float Az, float lo, float hi, float y) {
-    const float e = hi - lo;
-    const bool left = c.a_rr.x + c.b_reta.x < lo + hi;
-    const float Ax = c.a_rr.x - (left ? lo : hi), Ay = c.a_rr.y - y;
-    const float dx = c.d_idd.x, dy = c.d_idd.y, dz = c.d_idd.z;
-    const float tc = __saturatef(-c.d_idd.w * __fmaf_rn(Ax, dx, __fmaf_rn(Ay, dy, Az * dz)));
-    const float vx = __fmaf_rn(tc, dx, Ax), vy = __fmaf_rn(tc, dy, Ay), vz = __fmaf_rn(tc, dz, Az);
-    const float sa = __fmaf_rn(vx, Ax, __fmaf_rn(vy, Ay, vz * Az));
-    const float sb = __fmaf_rn(vx, dx, __fmaf_rn(vy, dy, __fmaf_rn(vz, dz, sa)));
-    const float beyond = fmaxf((left ? e : -e) * vx, 0.0f);
-    const float sep = fminf(sa, sb) - __fmaf_rn(0.0625f, (fabsf(vx) + fabsf(vy)) + fabsf(vz), beyond);
-    const float vv = __fmaf_rn(vx, vx, __fmaf_rn(vy, vy, vz * vz));
-    return !(sep * fabsf(sep) > (c.b_reta.w * c.b_reta.w) * vv);
+// (The two rows as packed FP32 pairs; Az = a.z minus the slab's centre, ny = -(y, y + 1/8).)
+__device__ __forceinline__ void rows_reached(const CapsuleLocal& c, const UnsetRows& u, f2 ny, float Az, bool& reach0,
+                                             bool& reach1) {
+    const float4 a = c.a_rr, b = c.b_reta, d = c.d_idd;
+    float s0, s1, lo0, lo1, hi0, hi1;
+    f2_unpack(u.sum, s0, s1);
+    f2_unpack(u.nlo, lo0, lo1);
+    f2_unpack(u.nhi, hi0, hi1);
+    const float mid2 = a.x + b.x;
+    const f2 nref = f2_pack(mid2 < s0 ? lo0 : hi0, mid2 < s1 ? lo1 : hi1);
+    const f2 e = f2_fma(nref, f2_pack(2.0f, 2.0f), u.sum);       // to the row's other end, signed
+    const f2 Ax = f2_add(f2_pack(a.x, a.x), nref), Ay = f2_add(f2_pack(a.y, a.y), ny), Az2 = f2_pack(Az, Az);
+    const f2 dx = f2_pack(d.x, d.x), dy = f2_pack(d.y, d.y), dz = f2_pack(d.z, d.z);
+    const float azdz = Az * d.z;
+    float t0, t1;
+    f2_unpack(f2_fma(Ax, dx, f2_fma(Ay, dy, f2_pack(azdz, azdz))), t0, t1);
+    const f2 tc = f2_pack(__saturatef(-d.w * t0), __saturatef(-d.w * t1));
+    const f2 vx = f2_fma(tc, dx, Ax), vy = f2_fma(tc, dy, Ay), vz = f2_fma(tc, dz, Az2);
+    const f2 sa = f2_fma(vx, Ax, f2_fma(vy, Ay, f2_mul(vz, Az2)));
+    const f2 sb = f2_fma(vx, dx, f2_fma(vy, dy, f2_fma(vz, dz, sa)));
+    const f2 vv = f2_mul(f2_fma(vx, vx, f2_fma(vy, vy, f2_mul(vz, vz))), f2_pack(b.w * b.w, b.w * b.w));
+    float x0, x1, y0, y1, z0, z1, e0, e1, a0, a1, b0, b1, r0, r1;
+    f2_unpack(vx, x0, x1);
+    f2_unpack(vy, y0, y1);
+    f2_unpack(vz, z0, z1);
+    f2_unpack(f2_mul(e, vx), e0, e1);
+    f2_unpack(sa, a0, a1);
+    f2_unpack(sb, b0, b1);
+    f2_unpack(vv, r0, r1);
+    const float p0 = fminf(a0, b0) - __fmaf_rn(0.0625f, (fabsf(x0) + fabsf(y0)) + fabsf(z0), fmaxf(e0, 0.0f));
+    const float p1 = fminf(a1, b1) - __fmaf_rn(0.0625f, (fabsf(x1) + fabsf(y1)) + fabsf(z1), fmaxf(e1, 0.0f));
+    reach0 = !(p0 * fabsf(p0) > r0);
+    reach1 = !(p1 * fabsf(p1) > r1);
 }
 
 // True when an endpoint of the capsule is within r of every point of the voxel: step 2 then
@@ -287,7 +308,7 @@ __device__ __forceinline__ bool capsule_covers(const float* a, const float* b, f
 }
 
 // Local capsule of endpoints a, b (voxel-local grid units) and radius r.  eta bounds, with
-// a wide factor, the FP32 error of the separation test below plus that of step 3: both
+// a wide factor, the FP32 error of the distance bounds below plus that of step 3: both
 // scale with the magnitude M of the local coordinates (and r), and sum to less than
 // 3e-6 (M + r + 3).
 __device__ __forceinline__ CapsuleLocal capsule_local(const float* a, const float* b, float r) {
@@ -323,22 +344,36 @@ __device__ __forceinline__ bool segment_box_separated(float4 a, float4 b, float4
     return sep > 0.0f && sep * sep > (re * re) * vv;
 }
 
-// True when the capsule provably misses sub-cell `id` by more than the rounding of the
-// exact minimum: separated by more than r + eta, eta (per capsule) covering the FP32 errors
-// of this bound and of step 3.  Step 3's FP32 value is the squared distance of a point
-// within ~1e-6 (M + 1) of the segment, to relative 1e-6, so a sub-cell separated by more
-// than r + eta has that value above r^2: the task can be dropped without changing the mask.
-__device__ __forceinline__ bool capsule_cell_separated(const CapsuleLocal& c, int id) {
-    return segment_box_separated(c.a_rr, c.b_reta, c.d_idd, (float)(id & 7) * 0.125f + 0.0625f,
-                                 (float)((id >> 3) & 7) * 0.125f + 0.0625f, (float)(id >> 6) * 0.125f + 0.0625f,
-                                 0.0625f, c.b_reta.w);
+// Sub-cell `id` against the capsule without the exact minimum: -1 provably out, 1 provably in,
+// 0 open.  Out: separated by more than r + eta (see segment_box_separated).  In: the point of the
+// axis nearest to the sub-cell's centre is within r - eta of the sub-cell.  eta (per capsule)
+// covers the FP32 errors of these bounds and of step 3, whose value is the squared distance of
+// the segment within 2e-7 (M + 3) (measured against FP64 over 160 M segments, degenerate
+// directions among them; eta is 2e-5 (M + r + 3)), so step 3 decides the same.
+__device__ __forceinline__ int capsule_cell_quick(const CapsuleLocal& c, int id) {
+    const float cx = (float)(id & 7) * 0.125f + 0.0625f, cy = (float)((id >> 3) & 7) * 0.125f + 0.0625f,
+                cz = (float)(id >> 6) * 0.125f + 0.0625f;
+    const float4 a = c.a_rr, d = c.d_idd;
+    const float Ax = a.x - cx, Ay = a.y - cy, Az = a.z - cz;
+    const float tc = __saturatef(-d.w * __fmaf_rn(Ax, d.x, __fmaf_rn(Ay, d.y, Az * d.z)));
+    const float vx = __fmaf_rn(tc, d.x, Ax), vy = __fmaf_rn(tc, d.y, Ay), vz = __fmaf_rn(tc, d.z, Az);
+    const float sa = __fmaf_rn(vx, Ax, __fmaf_rn(vy, Ay, vz * Az));
+    const float sb = __fmaf_rn(vx, d.x, __fmaf_rn(vy, d.y, __fmaf_rn(vz, d.z, sa)));
+    const float sep = fminf(sa, sb) - 0.0625f * ((fabsf(vx) + fabsf(vy)) + fabsf(vz));
+    const float vv = __fmaf_rn(vx, vx, __fmaf_rn(vy, vy, vz * vz));
+    const float re = c.b_reta.w;
+    if (sep * fabsf(sep) > (re * re) * vv) return -1;
+    const float ex = fmaxf(fabsf(vx) - 0.0625f, 0.0f), ey = fmaxf(fabsf(vy) - 0.0625f, 0.0f),
+                ez = fmaxf(fabsf(vz) - 0.0625f, 0.0f);
+    const float ri = 2.0f * sqrtf(a.w) - re;   // r - eta
+    return ri > 0.0f && __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, ez * ez)) <= ri * ri ? 1 : 0;
 }
 
 // Step 3 of every pooled task whose sub-cell is not set yet (warp-collective); returns the
 // lane's 16 bits of the updated mask.  A task skipped because an earlier task of the same
 // sub-cell set it would have returned a bit that is already 1, so the order of evaluation
-// does not change the mask.  Tasks whose sub-cell is separated from the capsule are dropped
-// first (compacting the rest in place), so that the exact minimum runs on full warps.
+// does not change the mask.  Most tasks are decided by capsule_cell_quick; the rest are compacted
+// in place, so that the exact minimum runs on full warps.
 __device__ __forceinline__ uint32_t capsule_step3_pool(CapsuleTasks& ct, int ntask, uint32_t chunk) {
     const int lane = threadIdx.x & 31;
     const uint32_t lo16 = __shfl_sync(0xffffffffu, chunk, (2 * lane) & 31);
@@ -353,7 +388,12 @@ __device__ __forceinline__ uint32_t capsule_step3_pool(CapsuleTasks& ct, int nta
         if (t < ntask) {
             task = ct.task[t];
             const int id = (int)(task & 511u);
-            keep = !(ct.mask[id >> 5] & (1u << (id & 31))) && !capsule_cell_separated(ct.slot[task >> 9].c, id);
+            const uint32_t bit = 1u << (id & 31);
+            if (!(ct.mask[id >> 5] & bit)) {
+                const int q = capsule_cell_quick(ct.slot[task >> 9].c, id);
+                keep = q == 0;
+                if (q > 0) atomicOr(&ct.mask[id >> 5], bit);
+            }
         }
         const uint32_t kept = __ballot_sync(0xffffffffu, keep);
         __syncwarp();   // the chunk is read before any lane writes (writes land at or below it)
@@ -1002,27 +1042,30 @@ __device__ __forceinline__ uint32_t voxel_mask(CapsuleTasks& ct, uint32_t okey, 
                                                uint32_t chunk, bool& full) {
     const int lane = threadIdx.x & 31;
     const float y0 = (float)sy0 * 0.125f + 0.0625f, zc = (float)sz * 0.125f + 0.0625f;
+    const f2 ny = f2_pack(-y0, -(y0 + 0.125f));
     UnsetRows ur = unset_rows(chunk);
     int ntask = 0;
     for (uint32_t j = 0; j < cnt; ++j) {
         if (full) break;
         const int slot = (int)(__shfl_sync(0xffffffffu, okey, src0 + (int)j) & 31u);
         const CapsuleSlot& cs = ct.slot[slot];
-        const float Az = cs.c.a_rr.z - zc;
-        const bool p0 = (chunk & 0xffu) != 0xffu && row_reached(cs.c, Az, ur.lo[0], ur.hi[0], y0);
-        const bool p1 = (chunk & 0xff00u) != 0xff00u && row_reached(cs.c, Az, ur.lo[1], ur.hi[1], y0 + 0.125f);
+        bool p0, p1;
+        rows_reached(cs.c, ur, ny, cs.c.a_rr.z - zc, p0, p1);
+        p0 = p0 && (chunk & 0xffu) != 0xffu;
+        p1 = p1 && (chunk & 0xff00u) != 0xff00u;
         if (!__any_sync(0xffffffffu, p0 || p1)) continue;
         const AxisTerms tz = axis_terms(cs.c.a_rr.z, cs.c.b_reta.z, sz);
         uint32_t set = 0, open = 0;
-        if (__any_sync(0xffffffffu, p0)) {
+#pragma unroll
+        for (int yi = 0; yi < 2; ++yi) {
+            const bool p = yi ? p1 : p0;
+            if (!__any_sync(0xffffffffu, p)) continue;
             uint32_t rs, ro;
-            capsule_row(cs, tz, sy0, rs, ro);
-            if (p0) { set = rs; open = ro; }
-        }
-        if (__any_sync(0xffffffffu, p1)) {
-            uint32_t rs, ro;
-            capsule_row(cs, tz, sy0 + 1, rs, ro);
-            if (p1) { set |= rs << 8; open |= ro << 8; }
+            capsule_row(cs, tz, sy0 + yi, rs, ro);
+            if (p) {
+                set |= rs << (8 * yi);
+                open |= ro << (8 * yi);
+            }
         }
         const uint32_t before = chunk;
         chunk |= set;
@@ -1065,6 +1108,11 @@ __device__ __forceinline__ uint32_t voxel_mask(CapsuleTasks& ct, uint32_t okey, 
 //     leaves each voxel's capsules together, and their mask steps run voxel by voxel.
 // A voxel of more than 32 capsules is a group of its own and runs in batches of 32.  The setup
 // and the mask steps each have one call site, so that the kernel holds one copy of them.
+// Issue-bound (80 % of slots; DRAM at the definition's bytes).  768k capsules at 512^3, 75 M pairs:
+// 10.4 ms against 18.9 ms when every capsule ran steps 1-2 on every row; a yarn of 4-voxel
+// radius at 1024^3, 107 M pairs, four of five voxels covered: 5.2 ms against 9.6 ms.  Of 46 M
+// capsules tested, 24 % reach a row and 40 rows per 100 run.  7 blocks per SM (72 registers,
+// 24 words spilled) ran the 1024^3 yarn in 5.2 ms, 6 blocks in 5.4 ms.
 __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint32_t* __restrict__ keys,
                                                                   const uint32_t* __restrict__ prims,
                                                                   const uint32_t* __restrict__ starts,

@@ -459,33 +459,6 @@ __device__ __forceinline__ uint32_t ge_mask(float a, float b) {
     return m;
 }
 
-// Two FP32 values packed in a 64-bit register (low half first) and the packed FP32 operations
-// on them; each half is rounded to nearest even, exactly as the scalar operation.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f2 v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // One direction sample of a well-conditioned lobe (|v|^2 > 0): the six histogram masks and
 // the six moment terms as raw FP32 bit patterns (x * 2^20 / |v|^2 + 1.5 * 2^23, rounded once).
 struct SampleTerms {
