@@ -262,9 +262,8 @@ VX_API vx_status vx_voxelize_lod_windowed(vx_context* ctx, const vx_primitives* 
  *     weight (n the unit normal; the clipped polygon's edges on voxel planes carry the
  *     derivative of the area).
  * Sub-cell occupancy and the key set are piecewise constant and carry no gradient.
- * Candidate pairs are recomputed, not stored, window by window as in vx_voxelize (windows
- * at most 1024 voxels wide and one pass of pairs each); every window adds its terms to the
- * per-primitive FP64 gradients.
+ * The voxels that a segment's axis or a triangle passes through are found again from the
+ * primitives (nothing of the forward is stored), over the whole grid in one pass.
  *   prims: the forward's primitives; grid: the forward's grid (resolution <= 2048).
  *   keys0 (device) [num_voxels0]: level-0 keys of the forward (sorted).
  *   grad_mass, grad_moment: HOST arrays of num_levels+1 device pointers; level l has
@@ -287,7 +286,7 @@ VX_API vx_status vx_backward(vx_context* ctx, const vx_primitives* prims, const 
  * The arguments and results are those of vx_backward with prims->kind == VX_FIBERS (no
  * context: nothing is allocated, not even through an allocator); triangles return
  * VX_ERR_UNSUPPORTED.  There is no counterpart in the paper.
- * Scratch: one fixed array of about 39 MB inside the library (a file-scope device
+ * Scratch: one fixed array of about 21 MB inside the library (a file-scope device
  * array), which every GPU that loads the library holds until the process exits.
  * Limits: at most 65,536 segments, 8,192 fibers, 262,144 level-0 voxels and 2,097,152
  * candidate (voxel, segment) pairs; larger inputs return VX_ERR_CAPACITY.  The pair limit

@@ -71,3 +71,76 @@ def test_capsule_masks_at_the_boundaries(n_fibers, pts, R, radius, step, snap):
                        weights=torch.from_numpy(w.weights).to(DEV))
     _same_level0(got, oracle.voxelize(w))
     ctx.close()
+
+
+def _adjoint_case(kind, seed, R, levels, n, **kw):
+    rng = np.random.default_rng(seed)
+    ctx = vx.Context(DEV)
+    if kind == "fibers":
+        ctrl, off, grid = synth.random_segments(n, kw.get("pts", 12), R, seed=seed, radius=kw["radius"], step=kw["step"])
+        geom = dict(ctrl=torch.from_numpy(ctrl).to(DEV), fiber_offsets=torch.from_numpy(off).to(DEV))
+        count = synth.fiber_segment_count(off)
+    else:
+        tris, grid = synth.random_triangles(n, R, seed=seed, size=kw["size"])
+        geom = dict(tri_verts=torch.from_numpy(tris).to(DEV))
+        count = n
+    geom["weights"] = torch.from_numpy(rng.uniform(0.5, 2.0, count).astype(np.float32)).to(DEV)
+    keys = ctx.voxelize(grid, **geom).keys.clone()
+    gm, gM = [], []
+    for l in range(levels + 1):
+        v = int(torch.unique_consecutive(keys >> (3 * l)).numel())
+        gm.append(torch.from_numpy(rng.uniform(-1, 1, v).astype(np.float32)).to(DEV))
+        gM.append(torch.from_numpy(rng.uniform(-1, 1, (v, 6)).astype(np.float32)).to(DEV))
+    return ctx, grid, geom, keys, gm, gM
+
+
+@pytest.mark.parametrize("kind,n,R,levels,kw", [
+    ("fibers", 1, 8, 0, dict(pts=2, radius=(0.4, 0.4), step=(0.6, 0.6))),
+    ("fibers", 3, 256, 5, dict(pts=3, radius=(0.3, 0.5), step=(90.0, 140.0))),    # few and long
+    ("fibers", 40, 64, 6, dict(pts=30, radius=(0.2, 2.0), step=(0.05, 6.0))),
+    ("fibers", 900, 32, 3, dict(pts=100, radius=(0.1, 0.4), step=(0.02, 0.6))),   # a segment per lane
+    ("triangles", 1, 8, 0, dict(size=(0.6, 0.6))),
+    ("triangles", 6, 128, 4, dict(size=(30.0, 50.0))),                            # few and large
+    ("triangles", 3000, 32, 5, dict(size=(0.1, 2.0))),
+])
+def test_adjoint_walks_every_voxel(kind, n, R, levels, kw):
+    """The gradient with respect to the weights is each primitive's own loss, so it is computed
+    again from the forward pass of that primitive alone: sum over its voxels and the levels'
+    gradients of their ancestors.  A voxel that the walk misses would show as a missing term.
+    Tolerance: masses of up to a few hundred FP32 terms (1e-5) of the sum of magnitudes."""
+    ctx, grid, geom, keys, gm, gM = _adjoint_case(kind, 7 + n, R, levels, n, **kw)
+    g_geom, g_w = ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **geom)
+    assert bool(torch.isfinite(g_geom).all())
+    gm0 = torch.zeros(keys.shape[0], dtype=torch.float64, device=DEV)
+    gM0 = torch.zeros(keys.shape[0], 6, dtype=torch.float64, device=DEV)
+    for l in range(levels + 1):
+        at = torch.unique_consecutive(keys >> (3 * l), return_inverse=True)[1]
+        gm0 += gm[l].double()[at]
+        gM0 += gM[l].double()[at]
+    count = g_w.shape[0]
+    pick = range(count) if count <= 40 else np.random.default_rng(1).choice(count, 40, replace=False)
+    for p in pick:
+        p = int(p)
+        if kind == "fibers":
+            off = geom["fiber_offsets"]
+            pts = kw["pts"]
+            c = (p // (pts - 1)) * pts + p % (pts - 1)
+            one = dict(ctrl=geom["ctrl"][c:c + 2].contiguous(), fiber_offsets=off.new_tensor([0, 2]))
+        else:
+            one = dict(tri_verts=geom["tri_verts"][p:p + 1].contiguous())
+        lv = ctx.voxelize(grid, **one)
+        at = torch.searchsorted(keys, lv.keys)
+        assert bool((keys[at] == lv.keys).all())
+        terms = lv.mass.double() * gm0[at] + (lv.moment.double() * gM0[at]).sum(1)
+        size = float((lv.mass.double() * gm0[at].abs() + (lv.moment.double() * gM0[at]).abs().sum(1)).sum())
+        assert abs(float(g_w[p]) - float(terms.sum())) <= 1e-5 * size + 1e-7, p
+    # the pair limit refuses what it refused: one voxel of more pairs than a pass may hold
+    ctx.set_max_pairs_per_pass(10 ** 9)
+    again = ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **geom)
+    assert torch.equal(again[0], g_geom) and torch.equal(again[1], g_w)
+    if count > 1000:
+        ctx.set_max_pairs_per_pass(1)
+        with pytest.raises(vx.VxError) as e:
+            ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **geom)
+        assert e.value.status == 3
+    ctx.close()
