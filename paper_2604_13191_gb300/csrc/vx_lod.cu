@@ -389,7 +389,7 @@ inline unsigned lod_reduce_grid(size_t np) {
 // S'^(1/2) of a symmetric 3x3 matrix (packed xx,yy,zz,xy,xz,yz) by cyclic Jacobi (at most 6
 // sweeps; a rotation is skipped when its off-diagonal is zero or negligible).  Returns
 // true when the square root is well conditioned: smallest singular value above 1e-4 of the
-// largest, and the largest above 1e-15.  S' = S + 1e-6 tr(S) I bounds the ratio below by
+// largest, and the largest in 1e-6 .. 1e6 (about 1 for a lobe of unit trace).  S' = S + 1e-6 tr(S) I bounds the ratio below by
 // ~1e-3 for any S with tr(S) > 0; the rounding of the FP32 Jacobi (orthogonality of the
 // rotations, the product R u) is ~1e-6 of the largest value, so for every unit u the FP32
 // v = R u then has |v| > 1e-4 sg_max (1 - 1e-2) and |v|^2 > 0.
@@ -449,7 +449,7 @@ __device__ bool sqrtm3(const float* S, float* Rm) {
         for (int j = 0; j < 3; ++j)
             Rm[3 * i + j] = ((V[i][0] * sg[0]) * V[j][0] + (V[i][1] * sg[1]) * V[j][1]) + (V[i][2] * sg[2]) * V[j][2];
     const float smax = fmaxf(fmaxf(sg[0], sg[1]), sg[2]), smin = fminf(fminf(sg[0], sg[1]), sg[2]);
-    return smax > 1e-15f && smin > 1e-4f * smax;
+    return smax > 1e-6f && smax < 1e6f && smin > 1e-4f * smax;
 }
 
 // a >= b as an integer mask (all ones or zero; zero when either is NaN)
@@ -498,8 +498,30 @@ __device__ __forceinline__ int rint_prod(float x, float s) {
     return __float_as_int(__fmaf_rn(x, s, 12582912.0f)) - 0x4B400000;
 }
 
+// 1 / n per half, correctly rounded, for n of magnitude 2^-100 .. 2^100: the hardware's approximation
+// (within 1 ulp) and one Newton step with fused multiply-adds, x' = x + x (1 - n x), which
+// Markstein (IBM J. Res. Dev. 34, 1990) shows to round correctly from such a start but for
+// isolated mantissas; compared with __frcp_rn on every mantissa at 137 exponents of that range, it
+// is the same throughout.  No slow path, so the sample loop holds no branch.
+__device__ __forceinline__ f2 f2_rcp(f2 n) {
+    float a, b, x, y;
+    f2_unpack(n, a, b);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(a));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
+    const f2 r = f2_pack(x, y);
+    return f2_fma(r, f2_fma(f2_pack(-a, -b), r, f2_pack(1.0f, 1.0f)), r);
+}
+
+// q / d for integers |q| <= d, given r = 1 / d correctly rounded: the product's remainder, exact in
+// a fused multiply-add, corrects it to the correctly rounded quotient (Markstein, as above).
+__device__ __forceinline__ double div_by(double q, double d, double r) {
+    const double y = q * r;
+    return fma(fma(-y, d, q), r, y);
+}
+
 // Histogram and sample second moment of lobe S, computed cooperatively by G warps
-// (G = 1: one warp; G > 1: the whole block, `red` is G * 13 words of shared memory).
+// (G = 1: one warp; G > 1: the whole block, `red` is 2 * G * 13 words of shared memory, `turn` says
+// which half: a half is written again only after the barrier of the call in between).
 // Every count and sum is an integer, so the result is independent of G and of the order
 // in which the threads visit the samples.  Threads tid < 6 receive the result.
 // The part of a lobe's statistics one thread keeps: component `tid` of the histogram and
@@ -509,8 +531,11 @@ struct LobeOwn {
     float mh;
 };
 
+// The direction table's last word tells whether every |u|^2 lies in [1/4, 4] (unit directions, as
+// the interface asks): the samples' |v|^2 then stay within f2_rcp's range.
 template <int G>
-__device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, int N, long long* red) {
+__device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, int N, bool unit, double inv_n,
+                               long long* red, int turn) {
     const float tr = (S[0] + S[1]) + S[2];
     const float eps = 1e-6f * tr;
     const float Sp[6] = {S[0] + eps, S[1] + eps, S[2] + eps, S[3], S[4], S[5]};
@@ -521,7 +546,7 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
     int cnt = 0;
     const int tid = (G == 1) ? (threadIdx.x & 31) : (int)threadIdx.x;
     constexpr int STRIDE = 32 * G;
-    if (wellcond && N <= STRIDE * 1024) {
+    if (wellcond && unit && N <= STRIDE * 1024) {
         // every sample has |v|^2 > 0: no sample is skipped.  Two samples (a whole pair of the
         // pair table) per step, their FP32 arithmetic as packed pairs: each half of a packed
         // operation rounds as the scalar one would, so the terms are those of sample_terms.
@@ -547,20 +572,19 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
             const f2 c0 = f2_mul(v[0], v[0]), c1 = f2_mul(v[1], v[1]), c2 = f2_mul(v[2], v[2]);
             const f2 n2 = f2_add(f2_add(c0, c1), c2);
             const f2 t6 = f2_mul(k36, n2), t2 = f2_mul(k04, n2);
-            float a0, b0, a1, b1, a2, b2, a6, b6, a4, b4, an, bn;
+            float a0, b0, a1, b1, a2, b2, a6, b6, a4, b4;
             f2_unpack(c0, a0, b0);
             f2_unpack(c1, a1, b1);
             f2_unpack(c2, a2, b2);
             f2_unpack(t6, a6, b6);
             f2_unpack(t2, a4, b4);
-            f2_unpack(n2, an, bn);
             h[0] = h[0] - (int32_t)ge_mask(a0, a6) - (int32_t)ge_mask(b0, b6);
             h[1] = h[1] - (int32_t)ge_mask(a1, a6) - (int32_t)ge_mask(b1, b6);
             h[2] = h[2] - (int32_t)ge_mask(a2, a6) - (int32_t)ge_mask(b2, b6);
             h[3] = h[3] - (int32_t)ge_mask(a0, a4) - (int32_t)ge_mask(b0, b4);
             h[4] = h[4] - (int32_t)ge_mask(a1, a4) - (int32_t)ge_mask(b1, b4);
             h[5] = h[5] - (int32_t)ge_mask(a2, a4) - (int32_t)ge_mask(b2, b4);
-            const f2 s20 = f2_mul(f2_pack(__frcp_rn(an), __frcp_rn(bn)), k20);
+            const f2 s20 = f2_mul(f2_rcp(n2), k20);
             // each term is folded into its sum as soon as it is formed (short live ranges)
             f2 x = f2_fma(c0, s20, koff);
             q[0] = q[0] + (uint32_t)x + (uint32_t)(x >> 32);
@@ -586,7 +610,6 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
             }
         }
         const uint32_t ns = 2u * (tid < NP ? (uint32_t)((NP - 1 - tid) / STRIDE + 1) : 0u) + (last ? 1u : 0u);
-        cnt = (int)ns;
 #pragma unroll
         for (int c = 0; c < 6; ++c) Q[c] = (int32_t)(q[c] - ns * 0x4B400000u);
     } else
@@ -624,18 +647,20 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
 #pragma unroll
         for (int c = 0; c < 6; ++c) Q[c] += q[c];
     }
+    // warp sums by the integer reduction; a moment sum in two parts of 16 and at most 17 bits, so
+    // that 32 of them fit 32 bits
+    const bool all = wellcond && unit && N <= STRIDE * 1024;   // every sample counted
+    if (!all) cnt = __reduce_add_sync(0xffffffffu, cnt);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            h[c] += __shfl_xor_sync(0xffffffffu, h[c], o);
-            Q[c] += __shfl_xor_sync(0xffffffffu, Q[c], o);
-        }
+    for (int c = 0; c < 6; ++c) {
+        h[c] = __reduce_add_sync(0xffffffffu, h[c]);
+        const int lo = __reduce_add_sync(0xffffffffu, (int)(Q[c] & 0xffff));
+        const int hi = __reduce_add_sync(0xffffffffu, (int)(Q[c] >> 16));
+        Q[c] = ((long long)hi << 16) + lo;
     }
     if (G > 1) {
         const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        __syncthreads();
+        red += (turn & 1) * (G * 13);
         if (lane == 0) {
             red[w * 13 + 0] = cnt;
 #pragma unroll
@@ -648,6 +673,7 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
         // thread c < 6 keeps component c only (the result below reads nothing else)
         if (tid < 6) {
             long long tc = 0, th = 0, tq = 0;
+#pragma unroll
             for (int ww = 0; ww < G; ++ww) {
                 tc += red[ww * 13];
                 th += red[ww * 13 + 1 + tid];
@@ -657,7 +683,6 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
             h[0] = (int32_t)th;
             Q[0] = tq;
         }
-        __syncthreads();
     }
     // component `tid` (tid < 6) of the histogram and of M^ (one FP64 division per thread)
     LobeOwn own;
@@ -673,7 +698,10 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
         }
     }
     own.mh = 0.0f;
-    if (tid < 6 && cnt > 0) own.mh = (float)((double)q / ((double)cnt * 1048576.0));
+    if (all)
+        own.mh = (float)div_by((double)q, (double)N * 1048576.0, inv_n);
+    else if (tid < 6 && cnt > 0)
+        own.mh = (float)((double)q / ((double)cnt * 1048576.0));
     return own;
 }
 
@@ -716,16 +744,24 @@ __device__ const PairTable kPairTable = make_pair_table();
 
 // float3 direction table -> float4 (one 16-byte load per sample), followed by the table of
 // whole pairs: directions 2j and 2j + 1 as {x0, x1, y0, y1} and {z0, z1, 0, 0}, so that each
-// coordinate of the two loads as one packed FP32 pair
-__global__ void k_pack_dirs(const float* __restrict__ d, int n, float4* __restrict__ out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) out[k] = make_float4(d[3 * k], d[3 * k + 1], d[3 * k + 2], 0.0f);
-    if (k < n / 2) {
-        float4* pr = out + n;
-        const float* a = d + 6 * k;
-        pr[2 * k] = make_float4(a[0], a[3], a[1], a[4]);
-        pr[2 * k + 1] = make_float4(a[2], a[5], 0.0f, 0.0f);
+// coordinate of the two loads as one packed FP32 pair, and by a word that is 1 when every |u|^2
+// lies in [1/4, 4].  One block.
+__global__ void __launch_bounds__(1024) k_pack_dirs(const float* __restrict__ d, int n, float4* __restrict__ out) {
+    float4* const pr = out + n;
+    bool bad = false;
+    for (int k = threadIdx.x; k < n; k += 1024) {
+        const float x = d[3 * k], y = d[3 * k + 1], z = d[3 * k + 2];
+        out[k] = make_float4(x, y, z, 0.0f);
+        const float uu = (x * x + y * y) + z * z;
+        bad = bad || !(uu >= 0.25f && uu <= 4.0f);
+        if (k < n / 2) {
+            const float* a = d + 6 * k;
+            pr[2 * k] = make_float4(a[0], a[3], a[1], a[4]);
+            pr[2 * k + 1] = make_float4(a[2], a[5], 0.0f, 0.0f);
+        }
     }
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) pr[2 * (n / 2)] = make_float4(any ? 0.0f : 1.0f, 0.0f, 0.0f, 0.0f);
 }
 
 // One parent listed in `work` per group of G warps (G = 1: a warp per parent, for levels
@@ -747,6 +783,9 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 
     const ClusterView sm = cluster_view(smem_raw + cluster_bytes(slots) * group, slots);
     long long* red = (long long*)(smem_raw + cluster_bytes(slots) * GROUPS);
     __shared__ unsigned long long bestred[G];
+    const bool unit = dirs[N + 2 * (N / 2)].x == 1.0f;
+    const double inv_n = 1.0 / ((double)N * 1048576.0);
+    int turn = 0;
     const int tid = (G == 1) ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
     constexpr int NT = 32 * G;
     const int lane = threadIdx.x & 31;
@@ -804,7 +843,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 
         int sampled = 0;
         for (int l = 0; l < n; ++l) {
             if (sm.alive[l] != 2) continue;
-            const LobeOwn st = sample_lobe<G>(sm.S + l * 6, dirs, N, red);
+            const LobeOwn st = sample_lobe<G>(sm.S + l * 6, dirs, N, unit, inv_n, red, turn++);
             if (tid < 6) {
                 sm.H[l * 6 + tid] = st.h;
                 sm.Mh[l * 6 + tid] = st.mh;
@@ -851,7 +890,6 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 
                 __syncthreads();
                 best = bestred[0];
                 for (int ww = 1; ww < G; ++ww) best = bestred[ww] < best ? bestred[ww] : best;
-                __syncthreads();
             }
             const int bi = (int)((best >> 8) & 0xffull), bj = (int)(best & 0xffull);
             // merge 0: pooled samples, (M^_i + M^_j) / 2; merge 1: mass-weighted moments
@@ -868,7 +906,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 
                 sm.alive[next] = 1;
             }
             gsync();
-            const LobeOwn st = sample_lobe<G>(sm.S + next * 6, dirs, N, red);
+            const LobeOwn st = sample_lobe<G>(sm.S + next * 6, dirs, N, unit, inv_n, red, turn++);
             if (tid < 6) {
                 sm.H[next * 6 + tid] = st.h;
                 sm.Mh[next * 6 + tid] = st.mh;
@@ -910,7 +948,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 
 
 // Dynamic shared memory of the three clustering tiers for K lobes.
 inline size_t cluster_smem(int G, int K) {
-    return G == 1 ? cluster_bytes(16 * K) * CL_WARPS : cluster_bytes(16 * K) + sizeof(long long) * 13 * G;
+    return G == 1 ? cluster_bytes(16 * K) * CL_WARPS : cluster_bytes(16 * K) + sizeof(long long) * 2 * 13 * G;
 }
 
 cudaError_t cluster_set_smem(int K) {
@@ -1087,7 +1125,7 @@ vx_status build_levels(vx_context* ctx, const vx_level* in, const vx_lod_params*
     if (K > 1) {
         VX_TRY(vx_ws_ensure(ctx, WS_LOD_TMP, vx_dirs_bytes(params->n_samples), s));
         dirs4 = (float4*)ctx->ws[WS_LOD_TMP].p;
-        VX_LAUNCH(ctx, ST_LOD_HEADS, s, k_pack_dirs<<<(params->n_samples + 255) / 256, 256, 0, s>>>(
+        VX_LAUNCH(ctx, ST_LOD_HEADS, s, k_pack_dirs<<<1, 1024, 0, s>>>(
                                             params->dirs, params->n_samples, dirs4));
         VX_CUDA_TRY(cluster_set_smem(K));
     }
@@ -1129,7 +1167,7 @@ vx_status build_levels(vx_context* ctx, const vx_level* in, const vx_lod_params*
 // before any capture): dirs [n][3] -> the direction table (vx_dirs_bytes(n) bytes at dirs4).
 cudaError_t vx_lod_batched_prepare(int K, const float* dirs, int n, float4* dirs4, cudaStream_t s) {
     if (K <= 1) return cudaSuccess;
-    k_pack_dirs<<<(n + 255) / 256, 256, 0, s>>>(dirs, n, dirs4);
+    k_pack_dirs<<<1, 1024, 0, s>>>(dirs, n, dirs4);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? cluster_set_smem(K) : e;
 }

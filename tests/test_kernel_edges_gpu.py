@@ -144,3 +144,20 @@ def test_adjoint_walks_every_voxel(kind, n, R, levels, kw):
             ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **geom)
         assert e.value.status == 3
     ctx.close()
+
+
+@pytest.mark.parametrize("N,scale", [(1, 1.0), (31, 1.0), (333, 0.3), (1000, 5.0), (2049, 1.0)])
+def test_lobe_sampling_paths(N, scale):
+    """Direction counts below and around a warp, odd ones, and directions that are not unit vectors
+    (outside the range of the packed reciprocal): every level against the oracle."""
+    ctrl, off, grid = synth.random_segments(12, 40, 16, seed=5, radius=(0.2, 0.8), step=(0.2, 1.5))
+    dirs = (synth.sample_directions(max(N, 2))[:N] * np.float32(scale)).astype(np.float32)
+    ctx = vx.Context(DEV)
+    L0 = ctx.voxelize(grid, ctrl=torch.from_numpy(ctrl).to(DEV), fiber_offsets=torch.from_numpy(off).to(DEV))
+    got = ctx.build_lod(L0, K=2, dirs=torch.from_numpy(dirs).to(DEV))
+    refs = oracle.build_pyramid(oracle.voxelize_fibers(ctrl, off, grid, K=1), 16, 2, dirs)
+    for lv, r in zip(got, refs):
+        g = lv.host()
+        assert np.array_equal(g["keys"], r["keys"]) and np.array_equal(g["lobe_count"], r["lobe_count"])
+        assert np.max(np.abs(g["lobes"] - r["lobes"])[..., :6]) <= 1e-5
+    ctx.close()
