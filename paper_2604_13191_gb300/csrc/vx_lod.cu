@@ -417,9 +417,14 @@ __device__ bool sqrtm3(const float* S, float* Rm) {
             // tan of the rotation angle, sgn(d) 2 apq / (|d| + sqrt(d^2 + 4 apq^2)) with
             // d = aqq - app (the smaller root of t^2 + 2 t d / (2 apq) - 1 = 0)
             const float d = aqq - app, e = 2.0f * apq;
-            float t = e / (fabsf(d) + sqrtf(d * d + e * e));
+            const float dd = d * d + e * e;
+            float t;
+            if (dd >= 1e-30f && dd <= 1e30f && fabsf(e) >= 1e-24f)
+                t = vx_div(e, fabsf(d) + vx_sqrt(dd));
+            else
+                t = e / (fabsf(d) + sqrtf(dd));
             if (d < 0.0f) t = -t;
-            const float c = __frcp_rn(sqrtf(t * t + 1.0f));
+            const float c = vx_rcp(vx_sqrt(t * t + 1.0f));   // |t| <= 1
             rotated = true;
             const float sn = t * c;
             a[p][p] = app - t * apq;
@@ -442,7 +447,10 @@ __device__ bool sqrtm3(const float* S, float* Rm) {
     }
     float sg[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) sg[i] = sqrtf(a[i][i] > 0.0f ? a[i][i] : 0.0f);
+    for (int i = 0; i < 3; ++i) {
+        const float x = a[i][i];
+        sg[i] = x >= 1e-30f && x <= 1e30f ? vx_sqrt(x) : sqrtf(x > 0.0f ? x : 0.0f);
+    }
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -460,7 +468,8 @@ __device__ __forceinline__ uint32_t ge_mask(float a, float b) {
 }
 
 // One direction sample of a well-conditioned lobe (|v|^2 > 0): the six histogram masks and
-// the six moment terms as raw FP32 bit patterns (x * 2^20 / |v|^2 + 1.5 * 2^23, rounded once).
+// the six moment terms as raw FP32 bit patterns (x / |v|^2 + 12, rounded once: between 8 and 16 an
+// FP32 value is a multiple of 2^-20).
 struct SampleTerms {
     uint32_t m[6];
     uint32_t x[6];
@@ -480,13 +489,13 @@ __device__ __forceinline__ SampleTerms sample_terms(const float* Rm, float4 u4) 
     r.m[3] = ge_mask(c0, t2);
     r.m[4] = ge_mask(c1, t2);
     r.m[5] = ge_mask(c2, t2);
-    const float s20 = __frcp_rn(n2) * 1048576.0f;
-    r.x[0] = __float_as_uint(__fmaf_rn(c0, s20, 12582912.0f));
-    r.x[1] = __float_as_uint(__fmaf_rn(c1, s20, 12582912.0f));
-    r.x[2] = __float_as_uint(__fmaf_rn(c2, s20, 12582912.0f));
-    r.x[3] = __float_as_uint(__fmaf_rn(v[0] * v[1], s20, 12582912.0f));
-    r.x[4] = __float_as_uint(__fmaf_rn(v[0] * v[2], s20, 12582912.0f));
-    r.x[5] = __float_as_uint(__fmaf_rn(v[1] * v[2], s20, 12582912.0f));
+    const float inv = __frcp_rn(n2);
+    r.x[0] = __float_as_uint(__fmaf_rn(c0, inv, 12.0f));
+    r.x[1] = __float_as_uint(__fmaf_rn(c1, inv, 12.0f));
+    r.x[2] = __float_as_uint(__fmaf_rn(c2, inv, 12.0f));
+    r.x[3] = __float_as_uint(__fmaf_rn(v[0] * v[1], inv, 12.0f));
+    r.x[4] = __float_as_uint(__fmaf_rn(v[0] * v[2], inv, 12.0f));
+    r.x[5] = __float_as_uint(__fmaf_rn(v[1] * v[2], inv, 12.0f));
     return r;
 }
 
@@ -498,11 +507,7 @@ __device__ __forceinline__ int rint_prod(float x, float s) {
     return __float_as_int(__fmaf_rn(x, s, 12582912.0f)) - 0x4B400000;
 }
 
-// 1 / n per half, correctly rounded, for n of magnitude 2^-100 .. 2^100: the hardware's approximation
-// (within 1 ulp) and one Newton step with fused multiply-adds, x' = x + x (1 - n x), which
-// Markstein (IBM J. Res. Dev. 34, 1990) shows to round correctly from such a start but for
-// isolated mantissas; compared with __frcp_rn on every mantissa at 137 exponents of that range, it
-// is the same throughout.  No slow path, so the sample loop holds no branch.
+// vx_rcp of both halves
 __device__ __forceinline__ f2 f2_rcp(f2 n) {
     float a, b, x, y;
     f2_unpack(n, a, b);
@@ -550,54 +555,60 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
         // every sample has |v|^2 > 0: no sample is skipped.  Two samples (a whole pair of the
         // pair table) per step, their FP32 arithmetic as packed pairs: each half of a packed
         // operation rounds as the scalar one would, so the terms are those of sample_terms.
-        // Histogram masks are -1 / 0; each moment term carries the constant 1.5 * 2^23, removed
+        // A threshold is compared by the sign of c - t (exact: the difference of two floats is
+        // zero or has the sign of the comparison); the signs are shifted into one word per
+        // counter and counted every 16 steps.  Each moment term carries the constant 12, removed
         // at the end: the sums wrap modulo 2^32, and the true sum of at most 1025 terms of
         // magnitude <= 2^20 is recovered exactly.
+        // What bounds the loop is the dispatch port, which a packed operation holds for two
+        // cycles: about 54 for the packed arithmetic, 24 for the twelve compares and 12 more.
         f2 R2[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) R2[i] = f2_pack(Rm[i], Rm[i]);
-        const f2 k36 = f2_pack(0.36f, 0.36f), k04 = f2_pack(0.04f, 0.04f);
-        const f2 k20 = f2_pack(1048576.0f, 1048576.0f), koff = f2_pack(12582912.0f, 12582912.0f);
+        const f2 k36 = f2_pack(-0.36f, -0.36f), k04 = f2_pack(-0.04f, -0.04f), koff = f2_pack(12.0f, 12.0f);
         const int NP = N >> 1;
         const ulonglong2* __restrict__ pr = reinterpret_cast<const ulonglong2*>(dirs + N);
         uint32_t q[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll 1
-        for (int j = tid; j < NP; j += STRIDE) {
-            const ulonglong2 xy = __ldg(pr + 2 * j);
-            const f2 z = __ldg(reinterpret_cast<const unsigned long long*>(pr + 2 * j + 1));
-            f2 v[3];
+        auto below = [](uint32_t& bits, f2 c, f2 nt) {   // appends the signs of c - t
+            // (scalar additions: the compiler contracts a packed one with the product before it,
+            // and two cost the dispatch port no more)
+            float c0, c1, t0, t1;
+            f2_unpack(c, c0, c1);
+            f2_unpack(nt, t0, t1);
+            bits = __funnelshift_l(__float_as_uint(__fadd_rn(c0, t0)), bits, 1);
+            bits = __funnelshift_l(__float_as_uint(__fadd_rn(c1, t1)), bits, 1);
+        };
+        auto add = [](uint32_t& sum, f2 x) { sum = sum + (uint32_t)x + (uint32_t)(x >> 32); };
+        for (int j = tid; j < NP;) {
+            uint32_t bits[6] = {0, 0, 0, 0, 0, 0};
+            const int steps = min(16, (NP - 1 - j) / STRIDE + 1);
+#pragma unroll 2
+            for (int k = 0; k < steps; ++k, j += STRIDE) {
+                const ulonglong2 xy = __ldg(pr + 2 * j);
+                const f2 z = __ldg(reinterpret_cast<const unsigned long long*>(pr + 2 * j + 1));
+                f2 v[3];
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-                v[i] = f2_fma(R2[3 * i + 2], z, f2_fma(R2[3 * i + 1], xy.y, f2_mul(R2[3 * i], xy.x)));
-            const f2 c0 = f2_mul(v[0], v[0]), c1 = f2_mul(v[1], v[1]), c2 = f2_mul(v[2], v[2]);
-            const f2 n2 = f2_add(f2_add(c0, c1), c2);
-            const f2 t6 = f2_mul(k36, n2), t2 = f2_mul(k04, n2);
-            float a0, b0, a1, b1, a2, b2, a6, b6, a4, b4;
-            f2_unpack(c0, a0, b0);
-            f2_unpack(c1, a1, b1);
-            f2_unpack(c2, a2, b2);
-            f2_unpack(t6, a6, b6);
-            f2_unpack(t2, a4, b4);
-            h[0] = h[0] - (int32_t)ge_mask(a0, a6) - (int32_t)ge_mask(b0, b6);
-            h[1] = h[1] - (int32_t)ge_mask(a1, a6) - (int32_t)ge_mask(b1, b6);
-            h[2] = h[2] - (int32_t)ge_mask(a2, a6) - (int32_t)ge_mask(b2, b6);
-            h[3] = h[3] - (int32_t)ge_mask(a0, a4) - (int32_t)ge_mask(b0, b4);
-            h[4] = h[4] - (int32_t)ge_mask(a1, a4) - (int32_t)ge_mask(b1, b4);
-            h[5] = h[5] - (int32_t)ge_mask(a2, a4) - (int32_t)ge_mask(b2, b4);
-            const f2 s20 = f2_mul(f2_rcp(n2), k20);
-            // each term is folded into its sum as soon as it is formed (short live ranges)
-            f2 x = f2_fma(c0, s20, koff);
-            q[0] = q[0] + (uint32_t)x + (uint32_t)(x >> 32);
-            x = f2_fma(c1, s20, koff);
-            q[1] = q[1] + (uint32_t)x + (uint32_t)(x >> 32);
-            x = f2_fma(c2, s20, koff);
-            q[2] = q[2] + (uint32_t)x + (uint32_t)(x >> 32);
-            x = f2_fma(f2_mul(v[0], v[1]), s20, koff);
-            q[3] = q[3] + (uint32_t)x + (uint32_t)(x >> 32);
-            x = f2_fma(f2_mul(v[0], v[2]), s20, koff);
-            q[4] = q[4] + (uint32_t)x + (uint32_t)(x >> 32);
-            x = f2_fma(f2_mul(v[1], v[2]), s20, koff);
-            q[5] = q[5] + (uint32_t)x + (uint32_t)(x >> 32);
+                for (int i = 0; i < 3; ++i)
+                    v[i] = f2_fma(R2[3 * i + 2], z, f2_fma(R2[3 * i + 1], xy.y, f2_mul(R2[3 * i], xy.x)));
+                const f2 c0 = f2_mul(v[0], v[0]), c1 = f2_mul(v[1], v[1]), c2 = f2_mul(v[2], v[2]);
+                const f2 n2 = f2_add(f2_add(c0, c1), c2);
+                const f2 t6 = f2_mul(k36, n2), t2 = f2_mul(k04, n2);
+                below(bits[0], c0, t6);
+                below(bits[1], c1, t6);
+                below(bits[2], c2, t6);
+                below(bits[3], c0, t2);
+                below(bits[4], c1, t2);
+                below(bits[5], c2, t2);
+                const f2 inv = f2_rcp(n2);
+                add(q[0], f2_fma(c0, inv, koff));
+                add(q[1], f2_fma(c1, inv, koff));
+                add(q[2], f2_fma(c2, inv, koff));
+                add(q[3], f2_fma(f2_mul(v[0], v[1]), inv, koff));
+                add(q[4], f2_fma(f2_mul(v[0], v[2]), inv, koff));
+                add(q[5], f2_fma(f2_mul(v[1], v[2]), inv, koff));
+            }
+#pragma unroll
+            for (int c = 0; c < 6; ++c) h[c] += 2 * steps - __popc(bits[c]);
         }
         // an odd N leaves one sample, taken by the thread next in line
         const bool last = (N & 1) && tid == NP % STRIDE;
@@ -611,7 +622,7 @@ __device__ LobeOwn sample_lobe(const float* S, const float4* __restrict__ dirs, 
         }
         const uint32_t ns = 2u * (tid < NP ? (uint32_t)((NP - 1 - tid) / STRIDE + 1) : 0u) + (last ? 1u : 0u);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) Q[c] = (int32_t)(q[c] - ns * 0x4B400000u);
+        for (int c = 0; c < 6; ++c) Q[c] = (int32_t)(q[c] - ns * 0x41400000u);
     } else
     // per-thread int32 partial sums (|term| <= 2^20), flushed to int64 every 1024 samples
     for (int k0 = tid; k0 < N; k0 += STRIDE * 1024) {
@@ -764,6 +775,10 @@ __global__ void __launch_bounds__(1024) k_pack_dirs(const float* __restrict__ d,
     if (threadIdx.x == 0) pr[2 * (n / 2)] = make_float4(any ? 0.0f : 1.0f, 0.0f, 0.0f, 0.0f);
 }
 
+// The warp tier's residency: 5 blocks per SM (90 registers, no spill, two steps of the sample
+// loop in flight) cluster the 768k-capsule yarn in 7.1 ms; 6 blocks in 7.24, 4 blocks with four
+// steps in 8.0.  Before the compares by sign, the branch-free roots and the constant folded into
+// the terms: 7.79 ms.
 // One parent listed in `work` per group of G warps (G = 1: a warp per parent, for levels
 // with many parents; G = CL_BLOCK_WARPS: a block per parent, for the few coarse parents
 // whose long merge chains would otherwise run on a single warp).
@@ -771,7 +786,7 @@ constexpr int CL_BLOCK_WARPS = 8;
 constexpr int CL_WIDE_WARPS = 16;   // levels with at most one parent per SM
 
 template <int G>
-__global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 7 : 0) k_sggx_cluster(
+__global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 0) k_sggx_cluster(
     LevelIn in, const uint32_t* __restrict__ starts, const uint32_t* __restrict__ work,
     const uint32_t* __restrict__ nwork_p, vx_level out, int K, const float4* __restrict__ dirs, int N,
     const LobeStats* __restrict__ cst, LobeStats* __restrict__ pst, unsigned long long* __restrict__ nsampled,
@@ -974,7 +989,7 @@ void launch_cluster(const LevelIn& li, const uint32_t* starts, const uint32_t* w
                     unsigned long long* nsampled, uint32_t n, int merge, cudaStream_t s, int tier = -1) {
     if (tier < 0) tier = n > (uint32_t)(vx::kSMs * 16) ? 0 : 1;
     if (tier == 0) {
-        const unsigned cb = (unsigned)std::min<size_t>((n + CL_WARPS - 1) / CL_WARPS, (size_t)vx::kSMs * 7);
+        const unsigned cb = (unsigned)std::min<size_t>((n + CL_WARPS - 1) / CL_WARPS, (size_t)vx::kSMs * 5);
         k_sggx_cluster<1><<<cb, CL_WARPS * 32, cluster_smem(1, K), s>>>(li, starts, work, wcnt, out, K, dirs4, N,
                                                                           cst, pst, nsampled, merge);
     } else if (tier == 1) {

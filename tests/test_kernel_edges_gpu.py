@@ -161,3 +161,25 @@ def test_lobe_sampling_paths(N, scale):
         assert np.array_equal(g["keys"], r["keys"]) and np.array_equal(g["lobe_count"], r["lobe_count"])
         assert np.max(np.abs(g["lobes"] - r["lobes"])[..., :6]) <= 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("N", [20001, 65535])
+def test_lobe_counts_at_the_thresholds(N):
+    """Histogram counts are compared at FP32 rounding: with many directions some samples fall within
+    one rounding of a threshold, and a mesh's nearly equal lobes turn a count that is off by one
+    into another merge.  Every lobe equals the oracle's bit for bit."""
+    tris = synth.heightfield(30, seed=N, sigma=0.1)
+    grid = synth.Grid((0.0, 0.0, -0.5), 1.0 / 32, 32)
+    dirs = synth.sample_directions(N)
+    ctx = vx.Context(DEV)
+    L0 = ctx.voxelize(grid, tri_verts=torch.from_numpy(tris).to(DEV))
+    got = ctx.build_lod(L0, K=2, dirs=torch.from_numpy(dirs).to(DEV))
+    w = synth.Workload("hf", "triangles", grid, tri_verts=tris, K=2)
+    refs = oracle.build_pyramid(oracle.voxelize(w, K=1), 32, 2, dirs)
+    for lv, r in zip(got, refs):
+        g = lv.host()
+        assert np.array_equal(g["lobe_count"], r["lobe_count"])
+        for k in range(2):
+            sel = r["lobe_count"] > k
+            assert np.array_equal(g["lobes"][sel, k].view(np.uint32), r["lobes"][sel, k].astype(np.float32).view(np.uint32))
+    ctx.close()
