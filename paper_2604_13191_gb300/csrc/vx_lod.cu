@@ -58,18 +58,6 @@ __global__ void k_level_counts(const uint64_t* __restrict__ keys, uint32_t n, in
         if (blk[l]) atomicAdd(&counts[l], blk[l]);
 }
 
-__global__ void k_parent_flags(const uint64_t* __restrict__ keys, uint32_t n, uint32_t* __restrict__ flags) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flags[i] = (i == 0 || (keys[i] >> 3) != (keys[i - 1] >> 3)) ? 1u : 0u;
-}
-
-__global__ void k_parent_starts(const uint64_t* __restrict__ keys, uint32_t n, const uint32_t* __restrict__ idx,
-                                uint32_t np, uint32_t* __restrict__ starts) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && (i == 0 || (keys[i] >> 3) != (keys[i - 1] >> 3))) starts[idx[i]] = i;
-    if (i == 0) starts[np] = n;
-}
-
 // 2x2x2 OR-downsample of two z-slabs a, b of a child mask (bit x + 8 y) into the parent word of
 // its octant (ox, oy): the 4 x 4 result lands at bit 4 ox + qx + 8 (4 oy + qy).  The folds run on
 // 32-bit halves (rows 0-3 low, 4-7 high): z, then the row pairs (2qy, 2qy + 1), then the x pairs;
@@ -1120,10 +1108,8 @@ vx_status build_levels(vx_context* ctx, const vx_level* in, const vx_lod_params*
     const int K = params->K;
     const uint32_t n0 = (uint32_t)in->num_voxels;
     // ---- per level ------------------------------------------------------------------------
-    VX_TRY(vx_ws_ensure(ctx, WS_LOD_FLAGS, (size_t)std::max<uint32_t>(n0, 1) * 4, s));
     VX_TRY(vx_ws_ensure(ctx, WS_LOD_STARTS, (size_t)std::max<uint32_t>(n0, 1) * 4 + 8, s));
     VX_TRY(vx_ws_ensure(ctx, WS_LOD_WORK, (size_t)std::max<uint32_t>(n0, 1) * 4, s));
-    uint32_t* flags = (uint32_t*)ctx->ws[WS_LOD_FLAGS].p;
     uint32_t* starts = (uint32_t*)ctx->ws[WS_LOD_STARTS].p;
     uint32_t* work = (uint32_t*)ctx->ws[WS_LOD_WORK].p;
     // per-lobe statistics of the previous and the current level (K > 1), ping-pong
@@ -1154,10 +1140,8 @@ vx_status build_levels(vx_context* ctx, const vx_level* in, const vx_lod_params*
         LevelIn li;
         li.keys = prev->keys; li.mask = prev->mask; li.mass = prev->mass; li.moment = prev->moment;
         li.lobe_count = prev->lobe_count; li.lobes = prev->lobes; li.K = prev->K;
-        VX_LAUNCH(ctx, ST_LOD_HEADS, s, k_parent_flags<<<grid_for(nprev, 256), 256, 0, s>>>(prev->keys, nprev, flags));
-        VX_TRY(vx_scan_u32(ctx, flags, flags, nprev, nullptr, s));
-        VX_LAUNCH(ctx, ST_LOD_HEADS, s, k_parent_starts<<<grid_for(nprev, 256), 256, 0, s>>>(prev->keys, nprev, flags, ncur, starts));
-        VX_CUDA_TRY(cudaMemsetAsync(misc + 40, 0, 8, s));   // [40] clustered parents, [41] taken
+        // (and clears [40] clustered parents, [41] taken)
+        VX_TRY(vx_parent_starts(ctx, prev->keys, nprev, starts, misc + 40, s));
         vx_stage_units(ctx, ST_LOD_REDUCE, ncur);
         // statistics kept by the child level (none for the input level) and by this one
         const LobeStats* cst = (K > 1 && l > 1) ? stats[l & 1] : nullptr;

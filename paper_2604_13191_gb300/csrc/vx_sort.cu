@@ -63,11 +63,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const uint32_t* __
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-// Single-block exclusive scan of the block partials (any length).
+// Single-block exclusive scan of the block partials (any length); zero: two words cleared for the
+// caller (or NULL).
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(uint32_t* part, uint32_t nb,
-                                                                uint32_t* total) {
+                                                                uint32_t* total, uint32_t* zero = nullptr) {
     __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
     uint32_t carry = 0;
+    if (zero && threadIdx.x < 2) zero[threadIdx.x] = 0u;
     for (uint32_t b = 0; b < nb; b += SCAN_TILE) {
         uint32_t v[SCAN_ITEMS];
         uint32_t s = 0;
@@ -144,48 +146,63 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_small(const uint32_t* in,
 }
 
 // ---- segment starts ---------------------------------------------------------------
-// Heads of the runs of equal keys in a sorted array: element e is a head when e == 0 or
-// keys[e] != keys[e - 1].  A thread takes SCAN_ITEMS consecutive elements (as k_scan_down).
-__device__ __forceinline__ uint32_t head_bits(const uint32_t* __restrict__ keys, uint32_t n, size_t e0) {
-    static_assert(SCAN_ITEMS == 8, "two 16-byte loads per thread");
-    uint32_t k[SCAN_ITEMS];
-    if (e0 + SCAN_ITEMS <= n) {
-        // e0 is a multiple of 8 and the key arrays are 256-byte aligned
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(keys + e0));
-        const uint4 y = __ldg(reinterpret_cast<const uint4*>(keys + e0) + 1);
-        k[0] = x.x; k[1] = x.y; k[2] = x.z; k[3] = x.w;
-        k[4] = y.x; k[5] = y.y; k[6] = y.z; k[7] = y.w;
+// Heads of the runs of equal keys >> shift in a sorted array: element e is a head when e == 0 or
+// its shifted key differs from the one before.  A thread takes SCAN_ITEMS consecutive elements
+// (as k_scan_down), e0 a multiple of SCAN_ITEMS; with `wide` (16-byte aligned keys) a full
+// thread loads them 16 bytes at a time.
+template <class T>
+__device__ __forceinline__ uint32_t head_bits(const T* __restrict__ keys, uint32_t n, size_t e0, int shift, bool wide) {
+    static_assert(SCAN_ITEMS == 8, "whole 16-byte loads per thread");
+    T k[SCAN_ITEMS];
+    if (wide && e0 + SCAN_ITEMS <= n) {
+        const uint4* p = reinterpret_cast<const uint4*>(keys + e0);
+        constexpr int PER = 16 / sizeof(T);
+#pragma unroll
+        for (int q = 0; q < SCAN_ITEMS / PER; ++q) {
+            const uint4 x = __ldg(p + q);
+            if (sizeof(T) == 4) {
+                k[q * PER] = (T)x.x;
+                k[q * PER + 1] = (T)x.y;
+                k[q * PER + PER - 2] = (T)x.z;
+                k[q * PER + PER - 1] = (T)x.w;
+            } else {
+                k[q * PER] = (T)(((uint64_t)x.y << 32) | x.x);
+                k[q * PER + PER - 1] = (T)(((uint64_t)x.w << 32) | x.z);
+            }
+        }
     } else {
 #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) k[j] = e0 + j < n ? keys[e0 + j] : 0u;
+        for (int j = 0; j < SCAN_ITEMS; ++j) k[j] = e0 + j < n ? keys[e0 + j] : (T)0;
     }
-    uint32_t prev = e0 > 0 && e0 - 1 < n ? keys[e0 - 1] : 0u;
+    T prev = e0 > 0 && e0 - 1 < n ? keys[e0 - 1] : (T)0;
     uint32_t bits = 0;
 #pragma unroll
     for (int j = 0; j < SCAN_ITEMS; ++j) {
         const size_t e = e0 + j;
-        if (e < n && (e == 0 || k[j] != prev)) bits |= 1u << j;
+        if (e < n && (e == 0 || (k[j] >> shift) != (prev >> shift))) bits |= 1u << j;
         prev = k[j];
     }
     return bits;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_count(const uint32_t* __restrict__ keys, uint32_t n,
+template <class T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_seg_count(const T* __restrict__ keys, uint32_t n, int shift, bool wide,
                                                             uint32_t* __restrict__ part) {
     __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
     const size_t e0 = (size_t)blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_ITEMS;
     uint32_t tot;
-    block_excl_scan(__popc(head_bits(keys, n, e0)), sm, tot);
+    block_excl_scan(__popc(head_bits(keys, n, e0, shift, wide)), sm, tot);
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_seg_starts(const uint32_t* __restrict__ keys, uint32_t n,
+template <class T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_seg_starts(const T* __restrict__ keys, uint32_t n, int shift, bool wide,
                                                              const uint32_t* __restrict__ part,
                                                              const uint32_t* __restrict__ nseg,
                                                              uint32_t* __restrict__ starts) {
     __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
     const size_t e0 = (size_t)blockIdx.x * SCAN_TILE + (size_t)threadIdx.x * SCAN_ITEMS;
-    uint32_t bits = head_bits(keys, n, e0);
+    uint32_t bits = head_bits(keys, n, e0, shift, wide);
     uint32_t tot;
     uint32_t idx = block_excl_scan(__popc(bits), sm, tot) + part[blockIdx.x];
     while (bits) {
@@ -194,6 +211,42 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_seg_starts(const uint32_t* __r
         starts[idx++] = (uint32_t)(e0 + j);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) starts[*nseg] = n;
+}
+
+// The same for a short array in one launch: one block takes its tiles in order with a running
+// carry (the counting pass and the scan of its counts are two more launches, 3 us each, where a
+// tile of 8192 elements takes about 1.5 us).  zero: two words cleared for the caller (or NULL).
+constexpr int STARTS_THREADS = 1024;
+constexpr uint32_t STARTS_SMALL = 4u * STARTS_THREADS * SCAN_ITEMS;
+template <class T>
+__global__ void __launch_bounds__(STARTS_THREADS) k_seg_starts_small(const T* __restrict__ keys, uint32_t n, int shift,
+                                                                     bool wide, uint32_t* __restrict__ nseg,
+                                                                     uint32_t* __restrict__ starts,
+                                                                     uint32_t* __restrict__ zero) {
+    __shared__ uint32_t ws[STARTS_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (zero && threadIdx.x < 2) zero[threadIdx.x] = 0u;
+    uint32_t carry = 0;
+    for (uint32_t b = 0; b < n; b += STARTS_THREADS * SCAN_ITEMS) {
+        const size_t e0 = (size_t)b + (size_t)threadIdx.x * SCAN_ITEMS;
+        uint32_t bits = head_bits(keys, n, e0, shift, wide);
+        const uint32_t cnt = __popc(bits), inc = warp_incl_scan(cnt);
+        if (lane == 31) ws[w] = inc;
+        __syncthreads();
+        const uint32_t t = ws[lane], ti = warp_incl_scan(t);
+        uint32_t idx = carry + __shfl_sync(0xffffffffu, ti - t, w) + inc - cnt;
+        carry += __shfl_sync(0xffffffffu, ti, 31);
+        while (bits) {
+            const int j = __ffs(bits) - 1;
+            bits &= bits - 1;
+            starts[idx++] = (uint32_t)(e0 + j);
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        starts[carry] = n;
+        if (nseg) *nseg = carry;
+    }
 }
 
 // ---- radix sort ----------------------------------------------------------------
@@ -590,21 +643,42 @@ vx_status vx_scan_u32(vx_context* ctx, const uint32_t* in, uint32_t* out, uint32
     return VX_OK;
 }
 
-vx_status vx_segment_starts(vx_context* ctx, const uint32_t* keys, uint32_t n, uint32_t* nseg, uint32_t* starts,
-                            cudaStream_t s) {
+namespace {
+template <class T>
+vx_status segment_starts(vx_context* ctx, int stage, const T* keys, uint32_t n, int shift, uint32_t* nseg,
+                         uint32_t* starts, uint32_t* zero, cudaStream_t s) {
     if (n == 0) {
-        VX_CUDA_TRY(cudaMemsetAsync(nseg, 0, 4, s));
+        if (nseg) VX_CUDA_TRY(cudaMemsetAsync(nseg, 0, 4, s));
+        if (zero) VX_CUDA_TRY(cudaMemsetAsync(zero, 0, 8, s));
         VX_CUDA_TRY(cudaMemsetAsync(starts, 0, 4, s));
         return VX_OK;
     }
+    const bool wide = ((uintptr_t)keys & 15) == 0;
     const uint32_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     VX_TRY(vx_ws_ensure(ctx, WS_SCAN_TMP, (size_t)nb * 4 + 256, s));
     uint32_t* part = (uint32_t*)ctx->ws[WS_SCAN_TMP].p;
-    VX_LAUNCH(ctx, ST_HEADS, s, k_seg_count<<<nb, SCAN_THREADS, 0, s>>>(keys, n, part));
-    VX_LAUNCH(ctx, ST_HEADS, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, nseg));
-    VX_LAUNCH(ctx, ST_HEADS, s, k_seg_starts<<<nb, SCAN_THREADS, 0, s>>>(keys, n, part, nseg, starts));
+    if (n <= STARTS_SMALL) {
+        VX_LAUNCH(ctx, stage, s, (k_seg_starts_small<T><<<1, STARTS_THREADS, 0, s>>>(keys, n, shift, wide, nseg, starts, zero)));
+        VX_CUDA_TRY(cudaGetLastError());
+        return VX_OK;
+    }
+    uint32_t* const total = nseg ? nseg : part + nb;
+    VX_LAUNCH(ctx, stage, s, (k_seg_count<T><<<nb, SCAN_THREADS, 0, s>>>(keys, n, shift, wide, part)));
+    VX_LAUNCH(ctx, stage, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, total, zero));
+    VX_LAUNCH(ctx, stage, s, (k_seg_starts<T><<<nb, SCAN_THREADS, 0, s>>>(keys, n, shift, wide, part, total, starts)));
     VX_CUDA_TRY(cudaGetLastError());
     return VX_OK;
+}
+}  // namespace
+
+vx_status vx_segment_starts(vx_context* ctx, const uint32_t* keys, uint32_t n, uint32_t* nseg, uint32_t* starts,
+                            cudaStream_t s) {
+    return segment_starts<uint32_t>(ctx, ST_HEADS, keys, n, 0, nseg, starts, nullptr, s);
+}
+
+vx_status vx_parent_starts(vx_context* ctx, const uint64_t* keys, uint32_t n, uint32_t* starts, uint32_t* zero,
+                           cudaStream_t s) {
+    return segment_starts<uint64_t>(ctx, ST_LOD_HEADS, keys, n, 3, nullptr, starts, zero, s);
 }
 
 // Digit widths of the passes of a `bits`-bit key: as few passes as 9-bit digits allow, digits
