@@ -523,80 +523,8 @@ __device__ __forceinline__ bool family_pass(int fam, const float v[3][3], const 
     return ok;
 }
 
-// What the mask steps of one (triangle, voxel) pair read, computed once by one lane.
-//   line[3 fam + j]  edge j of family fam as (alpha, beta, gamma, lo): the centre of sub-cell
-//                    pair (i0, i1) is off the middle of the edge axis' passing interval by
-//                    t = alpha i0 + beta i1 + gamma, and |t| <= half passes (see tri_record);
-//                    lo = half - eps
-//   plane            face normal and the box radius along it
-//   v0               first vertex (voxel-local), w = 2 eps
-//   box              bits 0-7, 8-15, 16-23: sub-cell columns the x, y, z box axes let pass
-struct TriRecord {
-    float4 line[9];
-    float4 plane;
-    float4 v0;
-};
-
-// The 13-axis test of a sub-cell separates on an edge axis when min_k p_k > rad or
-// max_k p_k < -rad, p_k the three vertices' projections relative to the sub-cell's centre.  The
-// centre enters all three as the same linear function E(i0, i1), so in exact arithmetic the
-// axis passes when -rad - max_k p_k(0) <= E <= rad - min_k p_k(0): |E - mid| <= half.  Both the
-// FP32 evaluation of the definition (family_pass) and that of t, mid and half here are within
-// 12 half ulps (2^-24) of (|q_a| + |q_b|)(V + 1), V the largest local coordinate; eps takes 33 of them
-// for the largest edge component (and 1e-37 for products that underflow).  So |t| <= half - eps is a pass of the definition and |t| > half
-// + eps a separation; what lies between, or is NaN, is decided by family_pass itself.
-__device__ __forceinline__ uint32_t tri_record(const float v[3][3], const float f[3][3], TriRecord& rec) {
-    const float e = 0.0625f;
-    float V = 0.0f, Q = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        V = fmaxf(V, fmax3(fabsf(v[k][0]), fabsf(v[k][1]), fabsf(v[k][2])));
-        Q = fmaxf(Q, fmax3(fabsf(f[k][0]), fabsf(f[k][1]), fabsf(f[k][2])));
-    }
-    const float B = Q * (V + 1.0f);
-    const float eps = B < 1e30f ? 4e-6f * B + 1e-37f : INFINITY;   // overflow, underflow: always open
-#pragma unroll
-    for (int fam = 0; fam < 3; ++fam) {
-        const int a0 = fam == 0 ? 1 : 0, a1 = fam == 2 ? 1 : 2;   // the family's coordinates (i0, i1)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            // p_k = s0 (v_a0 - c0) + s1 (v_a1 - c1), as family_pass
-            const float s0 = fam == 1 ? f[j][2] : -f[j][fam == 0 ? 2 : 1];
-            const float s1 = fam == 1 ? -f[j][0] : f[j][fam == 0 ? 1 : 0];
-            float p[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) p[k] = s1 * (v[k][a1] - e) + s0 * (v[k][a0] - e);
-            const float mn = fminf(fminf(p[0], p[1]), p[2]), mx = fmax3(p[0], p[1], p[2]);
-            const float half = e * (fabsf(s0) + fabsf(s1)) + 0.5f * (mx - mn);
-            // E = -(s0 i0 + s1 i1) / 8, mid = -(mn + mx) / 2
-            rec.line[3 * fam + j] = make_float4(-0.125f * s0, -0.125f * s1, 0.5f * (mn + mx), half - eps);
-        }
-    }
-    const float n0 = f[0][1] * f[1][2] - f[0][2] * f[1][1];
-    const float n1 = f[0][2] * f[1][0] - f[0][0] * f[1][2];
-    const float n2 = f[0][0] * f[1][1] - f[0][1] * f[1][0];
-    rec.plane = make_float4(n0, n1, n2, e * ((fabsf(n0) + fabsf(n1)) + fabsf(n2)));
-    rec.v0 = make_float4(v[0][0], v[0][1], v[0][2], 2.0f * eps);
-    uint32_t box = 0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float c = (float)(2 * k + 1) * 0.0625f;
-            if (!sep3(v[0][i] - c, v[1][i] - c, v[2][i] - c, e)) box |= 1u << (8 * i + k);
-        }
-    return box;
-}
-
-// max of three where a NaN wins
-__device__ __forceinline__ float fmax3_nan(float a, float b, float c) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
-// The definition of one edge family's test of pair (i0, i1), for the rare pairs that the records
-// leave open.
+// The definition of one edge family's test of pair (i0, i1), for the rare rows that the intervals
+// below leave open.
 __device__ __noinline__ bool family_exact(float4 a, float4 b, float4 c, int vi, int vj, int vk, int fam, int i0,
                                           int i1) {
     float v[3][3], f[3][3];
@@ -604,58 +532,198 @@ __device__ __noinline__ bool family_exact(float4 a, float4 b, float4 c, int vi, 
     return family_pass(fam, v, f, i0, i1);
 }
 
-// 16 sub-cell bits of one lane (sx 0..7, sy0+{0,1}, sz).  Warp-collective: every lane
-// of the warp must call it with the same triangle.  Each edge family's 64 pairs are tested two per
-// lane (i0 = lane & 7, i1 = lane >> 3 and that plus 4) and collected by ballots; a row's
-// candidates are then one byte of each family, and the face normal is tested for the rows
-// that have any.  exact(fam, i0, i1): the definition, called for pairs within eps of a boundary.
-template <class Exact>
-__device__ __forceinline__ uint32_t tri_bits16(const TriRecord& rec, uint32_t box, int sy0, int sz, Exact exact) {
-    const int lane = threadIdx.x & 31;
-    const float i0 = (float)(lane & 7), i1 = (float)(lane >> 3);
-    const float4 v0 = rec.v0;
-    uint32_t flo[3], fhi[3];
+// One edge axis as an interval of i0 for each i1.  The 13-axis test of a sub-cell separates on the axis
+// when min_k p_k > rad or max_k p_k < -rad, p_k = s0 w0 + s1 w1 the three vertices' projections
+// relative to the sub-cell's centre.  The centre enters all three as the same linear function, so
+// in exact arithmetic the axis passes when |T| <= half, T = alpha i0 + beta i1 + gamma.
+// With B = |s0| (V0 + 1) + |s1| (V1 + 1), V the largest coordinates of the vertices, every product
+// and sum is at most B; the FP32 evaluation of the definition (family_pass) is within 3.2 u B
+// (u = 2^-24) of it, and the coefficients here within 10 u B.  They are scaled by 1 / B, so |T| <=
+// half - 20 u is a pass of the definition and |T| > half + 20 u a separation.
+//   inv != 0: i0 between -(beta i1 + gamma) inv -+ r, r = half |inv|; with the 20 u and the rounding
+//     of the bounds a bound is uncertain by less than delta = 20 u |inv| + 5 u (9 + 2 r) + 8 u.
+//   inv == 0 (alpha below 1e-4): the row passes or fails as a whole by the sign of half - |beta i1 +
+//     gamma|, times 1e9 in the place of r; uncertain when it is within near = 7 |alpha| + 23 u.
+struct EdgeAxis {
+    float inv, beta, gamma, half, r, scale, near;
+};
+__device__ __forceinline__ EdgeAxis edge_axis(const float v0[3], const float v1[3], float V0, float V1, float s0, float s1,
+                                              float& delta, bool& fit) {
+    const float e = 0.0625f;
+    float p[3];
 #pragma unroll
-    for (int fa = 0; fa < 3; ++fa) {
-        float dlo[3], dhi[3];
+    for (int k = 0; k < 3; ++k) p[k] = s1 * (v1[k] - e) + s0 * (v0[k] - e);
+    const float mn = fminf(fminf(p[0], p[1]), p[2]), mx = fmax3(p[0], p[1], p[2]);
+    const float B = fabsf(s0) * V0 + fabsf(s1) * V1;
+    fit = fit && B > 1e-30f && B < 1e30f;   // nothing overflows, underflows or is NaN
+    const float q = vx_rcp(B);
+    const float alpha = -0.125f * s0 * q;
+    EdgeAxis a;
+    a.beta = -0.125f * s1 * q;
+    a.gamma = 0.5f * (mn + mx) * q;
+    a.half = (e * (fabsf(s0) + fabsf(s1)) + 0.5f * (mx - mn)) * q;
+    const bool row = fabsf(alpha) < 1e-4f;
+    a.inv = row ? 0.0f : vx_rcp(alpha);
+    a.r = a.half * fabsf(a.inv);
+    a.scale = row ? 1e9f : 0.0f;
+    a.near = row ? 8.0f * fabsf(alpha) + 1.5e-6f : -1.0f;
+    delta = fmaxf(delta, 1.3e-6f * fabsf(a.inv) + (7e-7f * a.r + 7e-6f));
+    return a;
+}
+
+// The integers of 0..7 in [a, b] as bits; `un` is raised when a bound is within delta of an integer.
+__device__ __forceinline__ uint32_t interval_bits(float a, float b, float delta, bool& un) {
+    constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer
+    // first = ceil(a), past = floor(b) + 1, both as the rounding of the bound plus a half
+    a = fminf(fmaxf(a, -0.5f), 7.5f) + 0.5f;
+    b = fmaxf(fminf(b + 0.5f, 8.0f), a);
+    const float am = a + MAGIC, bm = b + MAGIC;
+    un = un || fmaxf(fabsf(a - (am - MAGIC)), fabsf(b - (bm - MAGIC))) > 0.5f - delta;
+    // (the shifts take the low five bits of the biased integers; past >= first)
+    return __funnelshift_l(0u, 1u, __float_as_uint(bm)) - __funnelshift_l(0u, 1u, __float_as_uint(am));
+}
+
+// The 64 pairs of one family as two words, from its three edge axes; rows (i1) that are uncertain
+// are marked in `open`.
+__device__ __forceinline__ void family_rows(const EdgeAxis ax[3], float delta, uint32_t& lo, uint32_t& hi, uint32_t& open) {
+    lo = hi = open = 0;
+#pragma unroll 2
+    for (int i1 = 0; i1 < 8; ++i1) {
+        const float y = (float)i1;
+        float l[3], h[3], near[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const float4 l = rec.line[3 * fa + j];
-            const float t0 = __fmaf_rn(l.x, i0, l.z);
-            dlo[j] = fabsf(__fmaf_rn(l.y, i1, t0)) - l.w;
-            dhi[j] = fabsf(__fmaf_rn(l.y, i1 + 4.0f, t0)) - l.w;
+            const float u = __fmaf_rn(ax[j].beta, y, ax[j].gamma);
+            const float w = ax[j].half - fabsf(u);
+            const float r = __fmaf_rn(w, ax[j].scale, ax[j].r);
+            const float c = -u * ax[j].inv;
+            l[j] = c - r;
+            h[j] = c + r;
+            near[j] = ax[j].near - fabsf(w);
         }
-        const float wlo = fmax3_nan(dlo[0], dlo[1], dlo[2]), whi = fmax3_nan(dhi[0], dhi[1], dhi[2]);
-        bool plo = wlo <= 0.0f, phi = whi <= 0.0f;
-        const bool olo = !plo && !(wlo > v0.w), ohi = !phi && !(whi > v0.w);
-        if (olo) plo = exact(fa, lane & 7, lane >> 3);
-        if (ohi) phi = exact(fa, lane & 7, (lane >> 3) + 4);
-        flo[fa] = __ballot_sync(0xffffffffu, plo);
-        fhi[fa] = __ballot_sync(0xffffffffu, phi);
+        bool un = fmax3(near[0], near[1], near[2]) >= 0.0f;
+        const uint32_t bits = interval_bits(fmax3(l[0], l[1], l[2]), -fmax3(-h[0], -h[1], -h[2]), delta, un);
+        const uint32_t at = bits << (8 * (i1 & 3));
+        if (i1 < 4) lo |= at; else hi |= at;
+        open |= un ? 1u << i1 : 0u;
     }
-    // rows sy0, sy0 + 1 of slab sz as two bytes: family 1 (x, z), family 2 (x, y), the x box
-    // axis, and the rows that family 0 (y, z) and the y and z box axes let pass
-    const uint32_t bx = box & 0xffu;
-    uint32_t rows = __byte_perm(flo[0], fhi[0], sz) >> sy0;
-    rows &= box >> (8 + sy0);
-    if (!((box >> (16 + sz)) & 1u)) rows = 0;
-    const uint32_t on = ((rows & 1u) ? 0xffu : 0u) | ((rows & 2u) ? 0xff00u : 0u);
-    uint32_t bits = __byte_perm(flo[1], fhi[1], sz * 0x11) & __byte_perm(flo[2], fhi[2], sy0 * 0x11 + 0x10) &
-                    (bx | (bx << 8)) & on;
-    if (!__any_sync(0xffffffffu, bits != 0u)) return 0;
-    // face normal plane
-    const float4 n = rec.plane;
-    const float cz = (float)(2 * sz + 1) * 0.0625f;
-    const float pz = n.z * (v0.z - cz);
-    const float py0 = n.y * (v0.y - (float)(2 * sy0 + 1) * 0.0625f);
-    const float py1 = n.y * (v0.y - (float)(2 * sy0 + 3) * 0.0625f);
+}
+
+// The sub-cells of one (triangle, voxel) pair as 64 bytes (row sy + 8 sz, bit sx): v and f the
+// local vertices and edges of (A, B, C) in voxel (vi, vj, vk).  One lane per pair: an axis decides a
+// whole row of sub-cells as an interval, about 70 dispatch slots for 28 triangles at once, where
+// the warp testing sub-cells one triangle at a time took about 200 for every triangle.
+constexpr int TRI_MASK = 68;   // bytes from one pair's mask to the next (17 words: no bank conflict)
+__device__ __forceinline__ void tri_mask(const float v[3][3], const float f[3][3], float4 A, float4 B, float4 C, int vi,
+                                         int vj, int vk, uint8_t* __restrict__ out) {
+    const float e = 0.0625f;
+    float x[3][3], V[3];
+    uint32_t box[3];
 #pragma unroll
-    for (int sx = 0; sx < 8; ++sx) {
-        const float px = n.x * (v0.x - (float)(2 * sx + 1) * 0.0625f);
-        if (fabsf((px + py0) + pz) > n.w) bits &= ~(1u << sx);
-        if (fabsf((px + py1) + pz) > n.w) bits &= ~(256u << sx);
+    for (int q = 0; q < 16; ++q) reinterpret_cast<uint32_t*>(out)[q] = 0u;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) x[i][k] = v[k][i];
+        V[i] = fmax3(fabsf(x[i][0]), fabsf(x[i][1]), fabsf(x[i][2])) + 1.0f;
+        box[i] = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float c = (float)(2 * k + 1) * 0.0625f;
+            if (!sep3(x[i][0] - c, x[i][1] - c, x[i][2] - c, e)) box[i] |= 1u << k;
+        }
     }
-    return bits;
+    // the pairs (i0 + 8 i1) that pass the edge axes of families 0 (y, z), 1 (x, z), 2 (x, y)
+    uint32_t fam[6];
+#pragma unroll
+    for (int fa = 0; fa < 3; ++fa) {
+        const int a0 = fa == 0 ? 1 : 0, a1 = fa == 2 ? 1 : 2;   // the family's coordinates (i0, i1)
+        EdgeAxis ax[3];
+        float delta = 0.0f;
+        bool fit = true;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            // p_k = s0 (v_a0 - c0) + s1 (v_a1 - c1), as family_pass
+            const float s0 = fa == 1 ? f[j][2] : -f[j][fa == 0 ? 2 : 1];
+            const float s1 = fa == 1 ? -f[j][0] : f[j][fa == 0 ? 1 : 0];
+            ax[j] = edge_axis(x[a0], x[a1], V[a0], V[a1], s0, s1, delta, fit);
+        }
+        uint32_t lo, hi, open;
+        family_rows(ax, delta, lo, hi, open);
+        if (!fit) open = 0xffu;
+        open &= box[a1];   // (rows outside the box need no decision)
+        while (open) {
+            const int i1 = __ffs(open) - 1;
+            open &= open - 1;
+            uint32_t bits = 0;
+            for (int i0 = 0; i0 < 8; ++i0)
+                if (family_exact(A, B, C, vi, vj, vk, fa, i0, i1)) bits |= 1u << i0;
+            const int sh = 8 * (i1 & 3);
+            if (i1 < 4) lo = (lo & ~(0xffu << sh)) | (bits << sh);
+            else hi = (hi & ~(0xffu << sh)) | (bits << sh);
+        }
+        fam[2 * fa] = lo;
+        fam[2 * fa + 1] = hi;
+    }
+    // the box axes: y columns and z rows of family 0, x columns of family 1
+    const uint32_t ycols = box[1] * 0x01010101u, xcols = box[0] * 0x01010101u;
+    uint32_t zlo = 0, zhi = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        zlo |= (box[2] >> k) & 1u ? 0xffu << (8 * k) : 0u;
+        zhi |= (box[2] >> (4 + k)) & 1u ? 0xffu << (8 * k) : 0u;
+    }
+    fam[0] &= ycols & zlo;
+    fam[1] &= ycols & zhi;
+    fam[2] &= xcols;
+    fam[3] &= xcols;
+    // the face normal, scaled and bounded as the edge axes (sums of three products: within 16 u)
+    const float n0 = f[0][1] * f[1][2] - f[0][2] * f[1][1];
+    const float n1 = f[0][2] * f[1][0] - f[0][0] * f[1][2];
+    const float n2 = f[0][0] * f[1][1] - f[0][1] * f[1][0];
+    const float rad = e * ((fabsf(n0) + fabsf(n1)) + fabsf(n2));
+    const float Bn = fabsf(n0) * V[0] + (fabsf(n1) * V[1] + fabsf(n2) * V[2]);
+    const bool fit = Bn > 1e-30f && Bn < 1e30f;
+    const float q = vx_rcp(Bn);
+    const float alpha = -0.125f * n0 * q, beta = -0.125f * n1 * q, zeta = -0.125f * n2 * q, half = rad * q;
+    const float gamma = ((n0 * (v[0][0] - e) + n1 * (v[0][1] - e)) + n2 * (v[0][2] - e)) * q;
+    const bool row = fabsf(alpha) < 1e-4f;
+    const float inv = row ? 0.0f : vx_rcp(alpha), r0 = half * fabsf(inv), scale = row ? 1e9f : 0.0f;
+    const float near = row ? 8.0f * fabsf(alpha) + 1.5e-6f : -1.0f;
+    const float delta = 1.3e-6f * fabsf(inv) + (7e-7f * r0 + 7e-6f);
+    // rows with candidates, in the order of their bits in family 0
+    uint32_t w = fam[0];
+    int z0 = 0;
+    for (;;) {
+        if (w == 0u) {
+            if (z0) break;
+            z0 = 4;
+            w = fam[1];
+            if (w == 0u) break;
+        }
+        const int bit = __ffs(w) - 1, sy = bit & 7, sz = z0 + (bit >> 3);
+        w &= w - 1u;
+        uint32_t bits = __byte_perm(fam[2], fam[3], sz) & __byte_perm(fam[4], fam[5], sy) & 0xffu;
+        if (bits) {
+            const float u = __fmaf_rn(beta, (float)sy, __fmaf_rn(zeta, (float)sz, gamma));
+            const float wd = half - fabsf(u);
+            const float r = __fmaf_rn(wd, scale, r0), c = -u * inv;
+            bool un = !fit || fabsf(wd) <= near;
+            const uint32_t pass = interval_bits(c - r, c + r, delta, un);
+            if (!un) {
+                bits &= pass;
+            } else {
+                // the definition, sub-cell by sub-cell
+                const float pz = n2 * (v[0][2] - (float)(2 * sz + 1) * 0.0625f);
+                const float py = n1 * (v[0][1] - (float)(2 * sy + 1) * 0.0625f);
+                for (int sx = 0; sx < 8; ++sx) {
+                    const float px = n0 * (v[0][0] - (float)(2 * sx + 1) * 0.0625f);
+                    if (fabsf((px + py) + pz) > rad) bits &= ~(1u << sx);
+                }
+            }
+            out[sy + 8 * sz] = (uint8_t)bits;
+        }
+    }
 }
 
 // Clipped-polygon buffers of the triangle measure: two polygons of up to 12 vertices per
@@ -664,23 +732,25 @@ __device__ __forceinline__ uint32_t tri_bits16(const TriRecord& rec, uint32_t bo
 // banks.
 constexpr int POLY_FLOATS = 2 * 12 * 3 * 32;
 
-// Sutherland-Hodgman clip of polygon `pi` (n vertices) against coord_axis >= c (ge) or
-// <= c into polygon `po`; returns the new vertex count.  An edge emits its crossing of the plane
-// (when its ends lie on different sides), then its end vertex (when inside); the end of one
-// edge is kept in registers as the start of the next.
-__device__ __forceinline__ int clip_plane_s(float* __restrict__ buf, int pi, int po, int n, int axis, float c, bool ge) {
+// Sutherland-Hodgman clip of polygon `pi` (n vertices, the first at index `off`) against
+// coord_axis >= c (ge) or <= c into polygon `po` (first at 0); returns the new vertex count.  An
+// edge emits its crossing of the plane (when its ends lie on different sides), then its end vertex
+// (when inside); the end of one edge is kept in registers as the start of the next.
+__device__ __forceinline__ int clip_plane_s(float* __restrict__ buf, int pi, int po, int n, int off, int axis, float c,
+                                            bool ge) {
     const int t = threadIdx.x & 31;
     auto at = [&](int poly, int v, int j) -> float& { return buf[((poly * 12 + v) * 3 + j) * 32 + t]; };
-    int m = 0;
-    float S[3] = {at(pi, 0, 0), at(pi, 0, 1), at(pi, 0, 2)};
+    int m = 0, v = off;
+    float S[3] = {at(pi, off, 0), at(pi, off, 1), at(pi, off, 2)};
     for (int k = 0; k < n; ++k) {
-        const int kn = (k + 1) == n ? 0 : k + 1;
-        const float E[3] = {at(pi, kn, 0), at(pi, kn, 1), at(pi, kn, 2)};
+        v = v + 1 == n ? 0 : v + 1;
+        const float E[3] = {at(pi, v, 0), at(pi, v, 1), at(pi, v, 2)};
         const float Sa = sel3(axis, S[0], S[1], S[2]), Ea = sel3(axis, E[0], E[1], E[2]);
         const bool sin_ = ge ? (Sa >= c) : (Sa <= c);
         const bool ein = ge ? (Ea >= c) : (Ea <= c);
         if (sin_ != ein) {
-            const float sv = (c - Sa) / (Ea - Sa);
+            const float num = c - Sa, den = Ea - Sa;
+            const float sv = fabsf(num) >= 1e-24f && fabsf(den) <= 1e30f ? vx_div(num, den) : num / den;
 #pragma unroll
             for (int j = 0; j < 3; ++j) at(po, m, j) = (j == axis) ? c : S[j] + sv * (E[j] - S[j]);
             ++m;
@@ -697,29 +767,51 @@ __device__ __forceinline__ int clip_plane_s(float* __restrict__ buf, int pi, int
 }
 
 // area (voxel units^2) of the triangle clipped to the voxel [0,1]^3; buf: the warp's
-// POLY_FLOATS of shared memory
+// POLY_FLOATS of shared memory.  Against a plane that every vertex lies inside of, by more than the
+// rounding of the clipped vertices, a clip would only move the first vertex to the end: those
+// planes are counted instead (`off`), so that a lane clips against the planes its triangle
+// reaches, one after the other whatever their number, and the sum's order stays.
 __device__ float tri_measure(const float v[3][3], float* __restrict__ buf) {
     const int t = threadIdx.x & 31;
     auto at = [&](int poly, int vv, int j) -> float& { return buf[((poly * 12 + vv) * 3 + j) * 32 + t]; };
+    uint32_t need = 0;   // bit 2 axis: the plane 0, bit 2 axis + 1: the plane 1
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int j = 0; j < 3; ++j) {
 #pragma unroll
-        for (int j = 0; j < 3; ++j) at(0, k, j) = v[k][j];
-    int n = 3;
-    for (int axis = 0; axis < 3 && n > 0; ++axis) {
-        n = clip_plane_s(buf, 0, 1, n, axis, 0.0f, true);
-        if (n == 0) break;
-        n = clip_plane_s(buf, 1, 0, n, axis, 1.0f, false);
+        for (int k = 0; k < 3; ++k) at(0, k, j) = v[k][j];
+        const float mn = fminf(fminf(v[0][j], v[1][j]), v[2][j]), mx = fmax3(v[0][j], v[1][j], v[2][j]);
+        const float near = 1e-5f * (fmaxf(fabsf(mn), fabsf(mx)) + 1.0f);
+        if (!(mn > near)) need |= 1u << (2 * j);
+        if (!(mx < 1.0f - near)) need |= 2u << (2 * j);
+    }
+    int n = 3, off = 0, cur = 0, next = 0;
+    while (need) {
+        const int c = __ffs(need) - 1;
+        need &= need - 1u;
+        off += c - next;
+        while (off >= n) off -= n;
+        n = clip_plane_s(buf, cur, cur ^ 1, n, off, c >> 1, (c & 1) ? 1.0f : 0.0f, !(c & 1));
+        if (n < 1) return 0.0f;
+        cur ^= 1;
+        off = 0;
+        next = c + 1;
     }
     if (n < 3) return 0.0f;
+    off += 6 - next;
+    while (off >= n) off -= n;
+    auto vertex = [&](int k) { return off + k >= n ? off + k - n : off + k; };
     float cx = 0.0f, cy = 0.0f, cz = 0.0f;
-    const float a0 = at(0, 0, 0), a1 = at(0, 0, 1), a2 = at(0, 0, 2);
+    const float a0 = at(cur, off, 0), a1 = at(cur, off, 1), a2 = at(cur, off, 2);
+    int w = vertex(1);
+    float e1[3] = {at(cur, w, 0) - a0, at(cur, w, 1) - a1, at(cur, w, 2) - a2};
     for (int k = 1; k + 1 < n; ++k) {
-        const float e1[3] = {at(0, k, 0) - a0, at(0, k, 1) - a1, at(0, k, 2) - a2};
-        const float e2[3] = {at(0, k + 1, 0) - a0, at(0, k + 1, 1) - a1, at(0, k + 1, 2) - a2};
+        w = vertex(k + 1);
+        const float e2[3] = {at(cur, w, 0) - a0, at(cur, w, 1) - a1, at(cur, w, 2) - a2};
         cx = cx + (e1[1] * e2[2] - e1[2] * e2[1]);
         cy = cy + (e1[2] * e2[0] - e1[0] * e2[2]);
         cz = cz + (e1[0] * e2[1] - e1[1] * e2[0]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) e1[j] = e2[j];
     }
     return 0.5f * sqrtf((cx * cx + cy * cy) + cz * cz);
 }
@@ -1258,14 +1350,16 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint3
     }
 }
 
-// Warp per candidate voxel, up to eight voxels per step (fewer when the grid's warps would
+// Warp per candidate voxel, up to 28 voxels per step (fewer when the grid's warps would
 // otherwise run out of voxels).  Consecutive voxels whose triangles fit one batch (at most 32
 // together) form a group: lane l takes the group's l-th pair and computes its clipped area, its
-// moment terms and the record that the mask steps read, so that a mesh's few triangles per
-// voxel fill the lanes.  Then the masks run voxel by voxel, triangle by triangle, over the whole
-// warp.  A voxel of more than 32 triangles is a group of its own and runs in batches of 32.
-// Issue-bound (DRAM idle): 2.09 M triangles at 1024^3, 28.5 M pairs, 3.9 per voxel, 12.0 ms against
-// 45.9 ms for a voxel's triangles alone in the lanes and every projection of family_pass.
+// moment terms and its 512-bit mask, so that a mesh's few triangles per voxel fill the lanes.  Then
+// each voxel's masks are ORed, lane L on bits 16 L .. 16 L + 15.  A voxel of more than 32 triangles
+// is a group of its own and runs in batches of 32.
+// Bound by dispatch (DRAM idle).  2.09 M triangles at 1024^3, 28.5 M pairs, 3.9 per voxel: 8.9 ms, of
+// which the areas take 2.4, the edge axes 2.7 and the face normal 2.4 (45.9 ms with a voxel's
+// triangles alone in the lanes and the warp on one triangle's sub-cells; 12.0 ms with grouped
+// areas and records but the warp still on one triangle).  6 blocks per SM: 9.1 ms.
 __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_t* __restrict__ keys,
                                                                 const uint32_t* __restrict__ prims,
                                                                 const uint32_t* __restrict__ starts,
@@ -1275,14 +1369,13 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
                                                                 const float4* __restrict__ r2, SegOut out,
                                                                 int bx, int by, int bz,
                                                                 uint32_t* __restrict__ next) {
-    constexpr uint32_t STEP = 8;
+    constexpr uint32_t STEP = 28;   // their starts and the end sit in the lanes of one register
     const int lane = threadIdx.x & 31;
     const uint32_t nseg = *nseg_p;
-    const int sz = lane >> 2, sy0 = (lane & 3) * 2;
-    // the polygons of the measure, then the records of the masks, in the same memory
+    // the polygons of the measure, then the pairs' masks, in the same memory
     union Shared {
         float poly[POLY_FLOATS];
-        TriRecord rec[32];
+        uint8_t mask[32 * TRI_MASK];
     };
     __shared__ Shared shared[RED_WARPS];
     __shared__ float qs[RED_WARPS][32 * 7];       // per-pair w mu, w mu T(n) (pair-major)
@@ -1304,17 +1397,19 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
             const uint32_t m = max(1u, (uint32_t)__popc(fit));
             const uint32_t gend = __shfl_sync(0xffffffffu, st, g + m);
             uint32_t chunk = 0;
-            bool full = false;
             float accc = 0.0f;   // one voxel's sums, lane c < 7: component c
             for (uint32_t base = gbeg; base < gend; base += 32) {
                 const uint32_t cnt = min(32u, gend - base);
-                uint32_t box = 0, p = 0, key = 0;
+                uint32_t key = 0;
+                float4 a, b, c;
                 float v[3][3], f[3][3];
                 __syncwarp();   // the previous batch's masks and sums have read the shared state
                 if ((uint32_t)lane < cnt) {
                     key = keys[base + lane];
-                    p = prims[base + lane];
-                    const float4 a = r0[p], b = r1[p], c = r2[p];
+                    const uint32_t p = prims[base + lane];
+                    a = r0[p];
+                    b = r1[p];
+                    c = r2[p];
                     tri_local(a, b, c, (int)vx_compact1by2(key) + bx, (int)vx_compact1by2(key >> 1) + by,
                               (int)vx_compact1by2(key >> 2) + bz, v, f);
                     const float mu = tri_measure(v, sh.poly);
@@ -1334,8 +1429,10 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
                     q[5] = cc * (t[0] * t[2]);
                     q[6] = cc * (t[1] * t[2]);
                 }
-                __syncwarp();   // every lane's polygons are done: the records take their place
-                if ((uint32_t)lane < cnt) box = tri_record(v, f, sh.rec[lane]);
+                __syncwarp();   // every lane's polygons are done: the masks take their place
+                if ((uint32_t)lane < cnt)
+                    tri_mask(v, f, a, b, c, (int)vx_compact1by2(key) + bx, (int)vx_compact1by2(key >> 1) + by,
+                             (int)vx_compact1by2(key >> 2) + bz, sh.mask + lane * TRI_MASK);
                 __syncwarp();
                 // sums in primitive order, one component of one voxel per lane (one FP32 running
                 // sum each)
@@ -1358,16 +1455,8 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
                 for (uint32_t u = 0; u < m; ++u) {
                     const uint32_t ub = m > 1 ? __shfl_sync(0xffffffffu, st, g + u) - base : 0u;
                     const uint32_t ue = m > 1 ? __shfl_sync(0xffffffffu, st, g + u + 1) - base : cnt;
-                    for (uint32_t j = ub; j < ue && !full; ++j) {
-                        const uint32_t bj = __shfl_sync(0xffffffffu, box, j);
-                        const uint32_t pj = __shfl_sync(0xffffffffu, p, j), kj = __shfl_sync(0xffffffffu, key, j);
-                        chunk |= tri_bits16(sh.rec[j], bj, sy0, sz, [&](int fam, int i0, int i1) {
-                            return family_exact(r0[pj], r1[pj], r2[pj], (int)vx_compact1by2(kj) + bx,
-                                                (int)vx_compact1by2(kj >> 1) + by, (int)vx_compact1by2(kj >> 2) + bz,
-                                                fam, i0, i1);
-                        });
-                        full = __all_sync(0xffffffffu, chunk == 0xffffu);
-                    }
+                    for (uint32_t j = ub; j < ue; ++j)
+                        chunk |= *reinterpret_cast<const uint16_t*>(sh.mask + j * TRI_MASK + 2 * lane);
                     if (m > 1 || base + cnt >= gend) {
                         write_mask(out, s0 + g + u, __shfl_sync(0xffffffffu, key, ub), chunk);
                         if (m == 1 && lane < 7) {
@@ -1375,7 +1464,6 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
                             else out.moment[(size_t)(s0 + g) * 6 + lane - 1] = accc;
                         }
                         chunk = 0;
-                        full = false;
                     }
                 }
             }
