@@ -227,13 +227,16 @@ __device__ __forceinline__ void capsule_row(const CapsuleSlot& cs, const AxisTer
     const float xg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
     const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-    set = 0;
-    open = 0;
+    // a comparison x <= T by the sign of T - x (the exact sign of the difference), shifted into a
+    // word: additions run on the FMA pipe, where compares and selects load the ALU pipe, the busier
+    uint32_t out = 0, shut = 0;
 #pragma unroll
-    for (int sx = 0; sx < 8; ++sx) {
-        set |= ((xa[sx] <= TA) || (xb[sx] <= TB) ? 1u : 0u) << sx;
-        open |= (xg[sx] <= TG ? 1u : 0u) << sx;
+    for (int sx = 7; sx >= 0; --sx) {
+        out = __funnelshift_l(__float_as_uint(TA - xa[sx]) & __float_as_uint(TB - xb[sx]), out, 1);
+        shut = __funnelshift_l(__float_as_uint(TG - xg[sx]), shut, 1);
     }
+    set = ~out & 0xffu;
+    open = ~shut & 0xffu;
 }
 
 // The unset sub-cells of one lane's two rows, as packed pairs (row sy0, row sy0 + 1): the centres
