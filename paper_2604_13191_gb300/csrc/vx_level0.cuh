@@ -1006,10 +1006,155 @@ __device__ __forceinline__ bool tri_voxel_candidate(float4 a, float4 b, float4 c
 // count / emit: warp per primitive over its voxel range
 // ------------------------------------------------------------------------------------
 // With `ballots`, the count pass stores each primitive's hit ballots (one word per 32 voxels
-// of its range, ranges of at most 32 * CAND_BALLOTS voxels) and the emit pass of the same
+// of its range, ranges of at most 32 * stride voxels) and the emit pass of the same
 // window reads them instead of testing again; larger ranges are tested in both passes.
 // The ballots are the same bits either way, so the emitted order does not change.
-constexpr int CAND_BALLOTS = 8;
+constexpr int CAND_BALLOTS = 8;   // words per primitive in the batched path
+
+// One primitive of the pass, by a whole warp (see k_candidates); `stride` words of `ballots` per
+// primitive.  Returns its number of candidates.
+template <bool FIBER, bool EMIT>
+__device__ __forceinline__ uint32_t candidates_of(uint32_t p, float4 a, float4 b, float4 c, const Range& rg,
+                                                  const Window& R, uint32_t base, uint32_t* __restrict__ keys,
+                                                  uint32_t* __restrict__ vals, uint32_t* __restrict__ ballots,
+                                                  uint32_t stride) {
+    const int lane = threadIdx.x & 31;
+    uint32_t n = 0;
+    const long long tot = rg.total;
+    const bool stored = ballots != nullptr && tot <= 32ll * stride;
+    uint32_t* const pb = stored ? ballots + (size_t)p * stride : nullptr;
+    for (long long idx0 = 0; idx0 < tot; idx0 += 32) {
+        const long long idx = idx0 + lane;
+        bool hit = false;
+        int vi = 0, vj = 0, vk = 0;
+        if (idx < tot) {
+            int ix, iy, iz;
+            voxel_of(idx, tot, rg, ix, iy, iz);
+            vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
+            if (EMIT && stored) hit = (pb[idx0 >> 5] >> lane) & 1u;
+            else hit = FIBER ? capsule_voxel_candidate(a, b, vi, vj, vk) : tri_voxel_candidate(a, b, c, vi, vj, vk);
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+        if (!EMIT && stored && lane == 0) pb[idx0 >> 5] = bal;
+        if (EMIT && hit) {
+            const uint32_t pos = base + n + __popc(bal & ((1u << lane) - 1u));
+            keys[pos] = vx_morton3((uint32_t)(vi - R.lo[0]), (uint32_t)(vj - R.lo[1]), (uint32_t)(vk - R.lo[2]));
+            vals[pos] = p;
+        }
+        n += __popc(bal);
+    }
+    return n;
+}
+
+template <bool FIBER>
+__device__ __forceinline__ Range prim_range(const float4* __restrict__ r0, const float4* __restrict__ r1,
+                                            const float4* __restrict__ r2, uint32_t p, const Window& R, float4& a,
+                                            float4& b, float4& c) {
+    a = r0[p];
+    b = r1[p];
+    if (FIBER) return capsule_range(a, b, R);
+    c = r2[p];
+    return tri_range(a, b, c, R);
+}
+
+// Emit from the stored ballots.  A warp takes 32 consecutive primitives; their pairs are consecutive
+// in the output, so it walks their words 32 at a time, a lane per word: the lane writes the pairs
+// of its word's bits to the warp's staging buffer, which then goes out in order with whole lines.
+// (A warp per primitive left most of its lanes to the addresses of one word: 0.52 ms against
+// EMIT_NEW for the 75 M pairs of the 768k-capsule yarn.)  Morton codes come from a table of one
+// coordinate's spread bits in shared memory.  A group with a primitive whose range was too large
+// to be stored is taken primitive by primitive, as k_candidates does.
+constexpr int STAGE_WARPS = 4;
+template <bool FIBER>
+__global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* __restrict__ r0,
+                                                                  const float4* __restrict__ r1,
+                                                                  const float4* __restrict__ r2, uint32_t np, Window R,
+                                                                  const uint32_t* __restrict__ offs,
+                                                                  uint32_t* __restrict__ keys,
+                                                                  uint32_t* __restrict__ vals,
+                                                                  uint32_t* __restrict__ ballots, uint32_t stride) {
+    __shared__ uint32_t spread[1024];
+    __shared__ uint32_t stage_k[STAGE_WARPS][1024], stage_v[STAGE_WARPS][1024];
+    const int lane = threadIdx.x & 31;
+    uint32_t* const sk = stage_k[threadIdx.x >> 5];
+    uint32_t* const sv = stage_v[threadIdx.x >> 5];
+    for (uint32_t i = threadIdx.x; i < 1024; i += STAGE_WARPS * 32) spread[i] = vx_part1by2(i);
+    __syncthreads();
+    const uint32_t groups = (uint32_t)(((uint64_t)np + 31) / 32), warps = gridDim.x * STAGE_WARPS;
+    for (uint32_t g = blockIdx.x * STAGE_WARPS + (threadIdx.x >> 5); g < groups; g += warps) {
+        const uint32_t p0 = g * 32u, p = p0 + (uint32_t)lane;
+        Range rg;
+        rg.total = 0;
+        rg.lo[0] = rg.lo[1] = rg.lo[2] = 0;
+        rg.n[0] = rg.n[1] = rg.n[2] = 0;
+        if (p < np) {
+            float4 a, b, c;
+            rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
+        }
+        if (__any_sync(0xffffffffu, rg.total > 32ll * stride)) {
+            for (uint32_t q = p0; q < min(p0 + 32u, np); ++q) {
+                float4 a, b, c;
+                const Range rq = prim_range<FIBER>(r0, r1, r2, q, R, a, b, c);
+                candidates_of<FIBER, true>(q, a, b, c, rq, R, offs[q], keys, vals, ballots, stride);
+            }
+            continue;
+        }
+        // ranges of at most 2048 voxels: i / n as the high word of i (2^32 / n + 1), exact for i n < 2^32
+        const uint32_t tot = (uint32_t)rg.total, nw = (tot + 31u) / 32u;
+        const uint32_t n0 = (uint32_t)max(rg.n[0], 1), n1 = (uint32_t)max(rg.n[1], 1);
+        const uint32_t m0 = 0xffffffffu / n0 + 1u, m1 = 0xffffffffu / n1 + 1u;   // (0 for n = 1: see below)
+        uint32_t end = nw;   // inclusive scan: the words up to this lane's primitive
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += t;
+        }
+        const uint32_t words = __shfl_sync(0xffffffffu, end, 31);
+        uint32_t pos = offs[p0];
+        for (uint32_t w0 = 0; w0 < words; w0 += 32) {
+            const uint32_t s = w0 + (uint32_t)lane;
+            // the primitive of word s: the number of lanes whose words end at or before it
+            int own = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, end, own + o - 1) <= s) own += o;
+            own = min(own, 31);
+            const uint32_t first = __shfl_sync(0xffffffffu, end - nw, own);
+            const uint32_t on0 = __shfl_sync(0xffffffffu, n0, own), on1 = __shfl_sync(0xffffffffu, n1, own);
+            const uint32_t om0 = __shfl_sync(0xffffffffu, m0, own), om1 = __shfl_sync(0xffffffffu, m1, own);
+            const uint32_t lx = (uint32_t)(__shfl_sync(0xffffffffu, rg.lo[0], own) - R.lo[0]);
+            const uint32_t ly = (uint32_t)(__shfl_sync(0xffffffffu, rg.lo[1], own) - R.lo[1]);
+            const uint32_t lz = (uint32_t)(__shfl_sync(0xffffffffu, rg.lo[2], own) - R.lo[2]);
+            uint32_t bits = s < words ? ballots[(size_t)(p0 + (uint32_t)own) * stride + (s - first)] : 0u;
+            uint32_t at = __popc(bits);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += t;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
+            at -= __popc(bits);
+            const uint32_t i0 = (s - first) * 32u;
+            while (bits) {
+                const uint32_t i = i0 + (uint32_t)__ffs(bits) - 1u;
+                bits &= bits - 1u;
+                const uint32_t t = on0 == 1u ? i : __umulhi(i, om0);
+                const uint32_t z = on1 == 1u ? t : __umulhi(t, om1);
+                const uint32_t x = lx + (i - t * on0), y = ly + (t - z * on1);
+                sk[at] = spread[x] | (spread[y] << 1) | (spread[lz + z] << 2);
+                sv[at] = p0 + (uint32_t)own;
+                ++at;
+            }
+            __syncwarp();
+            for (uint32_t k = (uint32_t)lane; k < total; k += 32) {
+                keys[pos + k] = sk[k];
+                vals[pos + k] = sv[k];
+            }
+            __syncwarp();
+            pos += total;
+        }
+    }
+}
 
 template <bool FIBER, bool EMIT>
 __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __restrict__ r0,
@@ -1019,56 +1164,13 @@ __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __
                                                                 const uint32_t* __restrict__ offs,
                                                                 uint32_t* __restrict__ keys,
                                                                 uint32_t* __restrict__ vals,
-                                                                uint32_t* __restrict__ ballots = nullptr) {
+                                                                uint32_t* __restrict__ ballots, uint32_t stride) {
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * EMIT_WARPS;
     for (uint32_t p = blockIdx.x * EMIT_WARPS + (threadIdx.x >> 5); p < np; p += warps) {
-        float4 a = r0[p], b = r1[p], c;
-        Range rg;
-        if (FIBER) {
-            rg = capsule_range(a, b, R);
-        } else {
-            c = r2[p];
-            rg = tri_range(a, b, c, R);
-        }
-        uint32_t n = 0;
-        uint32_t base = EMIT ? offs[p] : 0u;
-        const long long tot = rg.total;
-        const bool stored = ballots != nullptr && tot <= 32ll * CAND_BALLOTS;
-        uint32_t* const pb = stored ? ballots + (size_t)p * CAND_BALLOTS : nullptr;
-        // emit: the primitive's stored words, one per lane, broadcast per step below
-        uint32_t words = 0;
-        if (EMIT && stored && (long long)lane * 32 < tot) words = pb[lane];
-        for (long long idx0 = 0; idx0 < tot; idx0 += 32) {
-            long long idx = idx0 + lane;
-            bool hit = false;
-            int vi = 0, vj = 0, vk = 0;
-            uint32_t bal;
-            if (EMIT && stored) {
-                bal = __shfl_sync(0xffffffffu, words, (int)(idx0 >> 5));
-                hit = (bal >> lane) & 1u;
-                if (hit) {
-                    int ix, iy, iz;
-                    voxel_of(idx, tot, rg, ix, iy, iz);
-                    vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
-                }
-            } else {
-                if (idx < tot) {
-                    int ix, iy, iz;
-                    voxel_of(idx, tot, rg, ix, iy, iz);
-                    vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
-                    hit = FIBER ? capsule_voxel_candidate(a, b, vi, vj, vk) : tri_voxel_candidate(a, b, c, vi, vj, vk);
-                }
-                bal = __ballot_sync(0xffffffffu, hit);
-                if (!EMIT && stored && lane == 0) pb[idx0 >> 5] = bal;
-            }
-            if (EMIT && hit) {
-                uint32_t pos = base + n + __popc(bal & ((1u << lane) - 1u));
-                keys[pos] = vx_morton3((uint32_t)(vi - R.lo[0]), (uint32_t)(vj - R.lo[1]), (uint32_t)(vk - R.lo[2]));
-                vals[pos] = p;
-            }
-            n += __popc(bal);
-        }
+        float4 a, b, c;
+        const Range rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
+        const uint32_t n = candidates_of<FIBER, EMIT>(p, a, b, c, rg, R, EMIT ? offs[p] : 0u, keys, vals, ballots, stride);
         if (!EMIT && lane == 0) counts[p] = n;
     }
 }

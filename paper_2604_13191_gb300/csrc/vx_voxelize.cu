@@ -38,15 +38,21 @@ __global__ void k_sum_u64(const uint32_t* __restrict__ cnt, uint32_t n, unsigned
     if ((threadIdx.x & 31) == 0 && acc) atomicAdd(total, acc);
 }
 
-// The count pass's ballot store (WS_BALLOTS, CAND_BALLOTS words per primitive) in *out, or
-// NULL when it would take more than 256 MB (the emit pass then tests every voxel again).
-// Errors: VX_ERR_OUT_OF_MEMORY, as for any workspace.
-vx_status window_ballots(vx_context* ctx, uint32_t np, cudaStream_t s, uint32_t** out) {
+// The count pass's ballot store (WS_BALLOTS) in *out and its words per primitive in *stride: 64 (ranges
+// of up to 2048 voxels, a capsule of 5 voxels' radius), 32 or 8, the most that takes at most 256 MB;
+// NULL when 8 take more (the emit pass then tests every voxel again).  A range's unused words
+// are never touched.  Errors: VX_ERR_OUT_OF_MEMORY, as for any workspace.
+vx_status window_ballots(vx_context* ctx, uint32_t np, cudaStream_t s, uint32_t** out, uint32_t* stride) {
     *out = nullptr;
-    const size_t bytes = (size_t)np * CAND_BALLOTS * 4;
-    if (bytes > ((size_t)256 << 20)) return VX_OK;
-    VX_TRY(vx_ws_ensure(ctx, WS_BALLOTS, bytes, s));
-    *out = (uint32_t*)ctx->ws[WS_BALLOTS].p;
+    *stride = 0;
+    for (uint32_t words : {64u, 32u, 8u}) {
+        const size_t bytes = (size_t)np * words * 4;
+        if (bytes > ((size_t)256 << 20)) continue;
+        VX_TRY(vx_ws_ensure(ctx, WS_BALLOTS, bytes, s));
+        *out = (uint32_t*)ctx->ws[WS_BALLOTS].p;
+        *stride = words;
+        break;
+    }
     return VX_OK;
 }
 
@@ -61,8 +67,10 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
     uint32_t* offs = (uint32_t*)ctx->ws[WS_OFFS].p;
     ctx->ballots = nullptr;
     uint32_t* ballots = nullptr;
-    VX_TRY(window_ballots(ctx, np, s, &ballots));
+    uint32_t stride = 0;
+    VX_TRY(window_ballots(ctx, np, s, &ballots, &stride));
     ctx->ballots = ballots;
+    ctx->ballots_stride = stride;
     ctx->ballots_np = np;
     for (int i = 0; i < 3; ++i) {
         ctx->ballots_win[i] = win.lo[i];
@@ -71,10 +79,10 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
     const unsigned cblocks = (unsigned)std::min<size_t>((np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
     if (fiber)
         VX_LAUNCH(ctx, ST_COUNT, s, k_candidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots));
+                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots, stride));
     else
         VX_LAUNCH(ctx, ST_COUNT, s, k_candidates<false, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots));
+                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots, stride));
     VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s));
     unsigned long long* t64 = (unsigned long long*)(misc + 8);
     VX_CUDA_TRY(cudaMemsetAsync(t64, 0, 8, s));
@@ -130,13 +138,22 @@ vx_status window_segments(vx_context* ctx, bool fiber, uint32_t np, const Window
     bool same = ctx->ballots != nullptr && ctx->ballots_np == np;
     for (int i = 0; i < 3; ++i)
         same = same && ctx->ballots_win[i] == win.lo[i] && ctx->ballots_win[3 + i] == win.hi[i];
-    uint32_t* ballots = same ? ctx->ballots : nullptr;
-    if (fiber)
+    if (same) {
+        const unsigned eblocks = (unsigned)std::min<size_t>(((size_t)np + 32 * STAGE_WARPS - 1) / (32 * STAGE_WARPS),
+                                                            (size_t)vx::kSMs * 6);
+        if (fiber)
+            VX_LAUNCH(ctx, ST_EMIT, s, k_emit_stored<true><<<eblocks, STAGE_WARPS * 32, 0, s>>>(
+                                           r0, r1, r2, np, win, offs, *k0, *v0, ctx->ballots, ctx->ballots_stride));
+        else
+            VX_LAUNCH(ctx, ST_EMIT, s, k_emit_stored<false><<<eblocks, STAGE_WARPS * 32, 0, s>>>(
+                                           r0, r1, r2, np, win, offs, *k0, *v0, ctx->ballots, ctx->ballots_stride));
+    } else if (fiber) {
         VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<true, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, ballots));
-    else
+                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, nullptr, 0u));
+    } else {
         VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<false, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, ballots));
+                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, nullptr, 0u));
+    }
     VX_CUDA_TRY(cudaGetLastError());
     VX_TRY(vx_radix_sort_u32(ctx, k0, v0, k1, v1, npairs, 3 * bits, s, misc));
     VX_TRY(vx_ws_ensure(ctx, WS_FLAGS, (size_t)npairs * 4, s));
@@ -1427,7 +1444,7 @@ extern "C" vx_status vx_backward_noalloc(const vx_primitives* prims, const vx_gr
                                                      prims->weights, np, g, r0, r1, misc);
     const unsigned cblocks = (unsigned)std::min<size_t>((np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
     k_candidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(r0, r1, nullptr, np, full_window((int)R), cnt,
-                                                                  nullptr, nullptr, nullptr);
+                                                                  nullptr, nullptr, nullptr, nullptr, 0u);
     // the exact 64-bit total
     k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
         cnt, np, (unsigned long long*)(misc + 8));
