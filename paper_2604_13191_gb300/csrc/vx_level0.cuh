@@ -1061,7 +1061,7 @@ __device__ __forceinline__ Range prim_range(const float4* __restrict__ r0, const
 // in the output, so it walks their words 32 at a time, a lane per word: the lane writes the pairs
 // of its word's bits to the warp's staging buffer, which then goes out in order with whole lines.
 // (A warp per primitive left most of its lanes to the addresses of one word: 0.52 ms against
-// EMIT_NEW for the 75 M pairs of the 768k-capsule yarn.)  Morton codes come from a table of one
+// 0.22 ms for the 75 M pairs of the 768k-capsule yarn.)  Morton codes come from a table of one
 // coordinate's spread bits in shared memory.  A group with a primitive whose range was too large
 // to be stored is taken primitive by primitive, as k_candidates does.
 constexpr int STAGE_WARPS = 4;
