@@ -115,35 +115,84 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const uint32_t* in, 
     }
 }
 
-// Single-block exclusive scan of a short array (a few tiles): the tiles in order with a
-// running carry, each thread on SCAN_ITEMS consecutive elements (in place allowed: a thread
-// reads its elements before it writes them); *total (optional) receives the sum.
-constexpr uint32_t SCAN_SMALL_TILES = 16;
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_small(const uint32_t* in, uint32_t* out, uint32_t n,
-                                                             uint32_t* total) {
-    __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
-    uint32_t carry = 0;
-    for (uint32_t b = 0; b < n; b += SCAN_TILE) {
-        uint32_t v[SCAN_ITEMS];
+// Single-block exclusive scan of a short array (in place allowed: a thread reads its elements
+// before it writes them); *total receives the sum modulo 2^32 and *total64 the exact sum (each
+// optional).  1024 threads on 8 consecutive elements each: 24k elements in 8 us, where 256 threads
+// took three times the tiles and 26 us, each tile a chain of loads, shuffles and barriers.  The next
+// tile's elements load while the current one is scanned.  pin: words copied to the host's buffer
+// once the totals are written.
+constexpr uint32_t SCAN_SMALL = 32768;
+constexpr int SMALL_THREADS = 1024;
+__global__ void __launch_bounds__(SMALL_THREADS) k_scan_small(const uint32_t* in, uint32_t* out, uint32_t n, bool wide,
+                                                              uint32_t* total, unsigned long long* total64,
+                                                              vx_pin_copy pin) {
+    __shared__ uint32_t ws[2][SMALL_THREADS / 32];
+    __shared__ unsigned long long ws64[SMALL_THREADS / 32];
+    constexpr uint32_t TILE = SMALL_THREADS * SCAN_ITEMS;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto load = [&](uint32_t e, uint32_t* v) {
+        if (wide && e + SCAN_ITEMS <= n) {
+            const uint4 a = *reinterpret_cast<const uint4*>(in + e), b = *reinterpret_cast<const uint4*>(in + e + 4);
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < SCAN_ITEMS; ++j) v[j] = e + j < n ? in[e + j] : 0u;
+        }
+    };
+    uint32_t cur[SCAN_ITEMS], carry = 0;
+    unsigned long long sum64 = 0;
+    load(threadIdx.x * SCAN_ITEMS, cur);
+    int turn = 0;
+    for (uint32_t b = 0; b < n; b += TILE, turn ^= 1) {
+        const uint32_t e = b + threadIdx.x * SCAN_ITEMS;
+        uint32_t nxt[SCAN_ITEMS] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (b + TILE < n) load(e + TILE, nxt);
         uint32_t s = 0;
 #pragma unroll
         for (int j = 0; j < SCAN_ITEMS; ++j) {
-            const uint32_t e = b + threadIdx.x * SCAN_ITEMS + j;
-            v[j] = (e < n) ? in[e] : 0u;
-            s += v[j];
+            s += cur[j];
+            sum64 += cur[j];
         }
-        uint32_t tot;
-        uint32_t run = carry + block_excl_scan(s, sm, tot);
+        const uint32_t inc = warp_incl_scan(s);
+        if (lane == 31) ws[turn][w] = inc;
+        __syncthreads();   // (the other half of ws is written before the next barrier)
+        const uint32_t t = ws[turn][lane], ti = warp_incl_scan(t);
+        uint32_t run = carry + __shfl_sync(0xffffffffu, ti - t, w) + inc - s;
+        carry += __shfl_sync(0xffffffffu, ti, 31);
+        uint32_t r[SCAN_ITEMS];
 #pragma unroll
         for (int j = 0; j < SCAN_ITEMS; ++j) {
-            const uint32_t e = b + threadIdx.x * SCAN_ITEMS + j;
-            if (e < n) out[e] = run;
-            run += v[j];
+            r[j] = run;
+            run += cur[j];
+            cur[j] = nxt[j];
         }
-        carry += tot;
+        if (wide && e + SCAN_ITEMS <= n) {
+            *reinterpret_cast<uint4*>(out + e) = make_uint4(r[0], r[1], r[2], r[3]);
+            *reinterpret_cast<uint4*>(out + e + 4) = make_uint4(r[4], r[5], r[6], r[7]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < SCAN_ITEMS; ++j)
+                if (e + j < n) out[e + j] = r[j];
+        }
     }
-    if (threadIdx.x == 0 && total) *total = carry;
+    if (total64) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum64 += __shfl_xor_sync(0xffffffffu, sum64, o);
+        if (lane == 0) ws64[w] = sum64;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        if (total) *total = carry;
+        if (total64) {
+            unsigned long long t = 0;
+            for (int k = 0; k < SMALL_THREADS / 32; ++k) t += ws64[k];
+            *total64 = t;
+        }
+        vx_pin_words(pin);
+    }
 }
+inline bool scan_wide(const uint32_t* in, const uint32_t* out) { return (((uintptr_t)in | (uintptr_t)out) & 15) == 0; }
 
 // ---- segment starts ---------------------------------------------------------------
 // Heads of the runs of equal keys >> shift in a sorted array: element e is a head when e == 0 or
@@ -220,9 +269,9 @@ constexpr int STARTS_THREADS = 1024;
 constexpr uint32_t STARTS_SMALL = 4u * STARTS_THREADS * SCAN_ITEMS;
 template <class T>
 __global__ void __launch_bounds__(STARTS_THREADS) k_seg_starts_small(const T* __restrict__ keys, uint32_t n, int shift,
-                                                                     bool wide, uint32_t* __restrict__ nseg,
+                                                                     bool wide, uint32_t* nseg,
                                                                      uint32_t* __restrict__ starts,
-                                                                     uint32_t* __restrict__ zero) {
+                                                                     uint32_t* __restrict__ zero, vx_pin_copy pin) {
     __shared__ uint32_t ws[STARTS_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (zero && threadIdx.x < 2) zero[threadIdx.x] = 0u;
@@ -246,6 +295,7 @@ __global__ void __launch_bounds__(STARTS_THREADS) k_seg_starts_small(const T* __
     if (threadIdx.x == 0) {
         starts[carry] = n;
         if (nseg) *nseg = carry;
+        vx_pin_words(pin);
     }
 }
 
@@ -622,18 +672,20 @@ __global__ void k_selftest_wait(uint32_t limit, uint32_t* flag) {
 }  // namespace
 
 vx_status vx_scan_u32(vx_context* ctx, const uint32_t* in, uint32_t* out, uint32_t n,
-                      uint32_t* total, cudaStream_t s) {
+                      uint32_t* total, cudaStream_t s, unsigned long long* total64, vx_pin_copy pin, bool* done) {
     uint32_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (nb == 0) nb = 1;
+    if (done) *done = false;
     VX_TRY(vx_ws_ensure(ctx, WS_SCAN_TMP, (size_t)nb * 4 + 256, s));
     uint32_t* part = (uint32_t*)ctx->ws[WS_SCAN_TMP].p;
     if (n == 0) {
         if (total) VX_CUDA_TRY(cudaMemsetAsync(total, 0, 4, s));
         return VX_OK;
     }
-    if (nb <= SCAN_SMALL_TILES) {   // one launch for a short array
-        VX_LAUNCH(ctx, ST_SCAN, s, k_scan_small<<<1, SCAN_THREADS, 0, s>>>(in, out, n, total));
+    if (n <= SCAN_SMALL) {   // one launch for a short array
+        VX_LAUNCH(ctx, ST_SCAN, s, k_scan_small<<<1, SMALL_THREADS, 0, s>>>(in, out, n, scan_wide(in, out), total, total64, pin));
         VX_CUDA_TRY(cudaGetLastError());
+        if (done) *done = true;
         return VX_OK;
     }
     VX_LAUNCH(ctx, ST_SCAN, s, k_scan_reduce<<<nb, SCAN_THREADS, 0, s>>>(in, n, part));
@@ -646,7 +698,8 @@ vx_status vx_scan_u32(vx_context* ctx, const uint32_t* in, uint32_t* out, uint32
 namespace {
 template <class T>
 vx_status segment_starts(vx_context* ctx, int stage, const T* keys, uint32_t n, int shift, uint32_t* nseg,
-                         uint32_t* starts, uint32_t* zero, cudaStream_t s) {
+                         uint32_t* starts, uint32_t* zero, cudaStream_t s, vx_pin_copy pin, bool* done) {
+    if (done) *done = false;
     if (n == 0) {
         if (nseg) VX_CUDA_TRY(cudaMemsetAsync(nseg, 0, 4, s));
         if (zero) VX_CUDA_TRY(cudaMemsetAsync(zero, 0, 8, s));
@@ -658,8 +711,9 @@ vx_status segment_starts(vx_context* ctx, int stage, const T* keys, uint32_t n, 
     VX_TRY(vx_ws_ensure(ctx, WS_SCAN_TMP, (size_t)nb * 4 + 256, s));
     uint32_t* part = (uint32_t*)ctx->ws[WS_SCAN_TMP].p;
     if (n <= STARTS_SMALL) {
-        VX_LAUNCH(ctx, stage, s, (k_seg_starts_small<T><<<1, STARTS_THREADS, 0, s>>>(keys, n, shift, wide, nseg, starts, zero)));
+        VX_LAUNCH(ctx, stage, s, (k_seg_starts_small<T><<<1, STARTS_THREADS, 0, s>>>(keys, n, shift, wide, nseg, starts, zero, pin)));
         VX_CUDA_TRY(cudaGetLastError());
+        if (done) *done = true;
         return VX_OK;
     }
     uint32_t* const total = nseg ? nseg : part + nb;
@@ -672,13 +726,13 @@ vx_status segment_starts(vx_context* ctx, int stage, const T* keys, uint32_t n, 
 }  // namespace
 
 vx_status vx_segment_starts(vx_context* ctx, const uint32_t* keys, uint32_t n, uint32_t* nseg, uint32_t* starts,
-                            cudaStream_t s) {
-    return segment_starts<uint32_t>(ctx, ST_HEADS, keys, n, 0, nseg, starts, nullptr, s);
+                            cudaStream_t s, vx_pin_copy pin, bool* done) {
+    return segment_starts<uint32_t>(ctx, ST_HEADS, keys, n, 0, nseg, starts, nullptr, s, pin, done);
 }
 
 vx_status vx_parent_starts(vx_context* ctx, const uint64_t* keys, uint32_t n, uint32_t* starts, uint32_t* zero,
                            cudaStream_t s) {
-    return segment_starts<uint64_t>(ctx, ST_LOD_HEADS, keys, n, 3, nullptr, starts, zero, s);
+    return segment_starts<uint64_t>(ctx, ST_LOD_HEADS, keys, n, 3, nullptr, starts, zero, s, vx_pin_copy{}, nullptr);
 }
 
 // Digit widths of the passes of a `bits`-bit key: as few passes as 9-bit digits allow, digits
@@ -750,8 +804,8 @@ cudaError_t vx_scan_u32_scratch(const uint32_t* in, uint32_t* out, uint32_t n, u
                                 uint32_t* partials, cudaStream_t s) {
     if (n == 0) return total ? cudaMemsetAsync(total, 0, 4, s) : cudaSuccess;
     const uint32_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (nb <= SCAN_SMALL_TILES) {   // one launch for a short array
-        k_scan_small<<<1, SCAN_THREADS, 0, s>>>(in, out, n, total);
+    if (n <= SCAN_SMALL) {   // one launch for a short array
+        k_scan_small<<<1, SMALL_THREADS, 0, s>>>(in, out, n, scan_wide(in, out), total, nullptr, vx_pin_copy{});
         return cudaGetLastError();
     }
     k_scan_reduce<<<nb, SCAN_THREADS, 0, s>>>(in, n, partials);
