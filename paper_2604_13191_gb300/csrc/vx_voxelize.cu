@@ -549,10 +549,10 @@ namespace {
 // before i: key i starts a parent of level l when its bits above 3 l differ from the previous
 // key's, so it starts one at every level up to head_level(i).  A warp takes 256 consecutive keys;
 // k_adj_counts stores each warp's parents per level, k_adj_scan turns them into offsets, and
-// k_adj_bcast ranks its keys by ballots and adds the levels' gradients in registers, so the
-// FP64 adjoints are written once instead of being read and written for each level.
-// 1.01 M voxels and 4 coarser levels: 0.17 ms (7 FP64 conversions and sums per level and voxel) against
-// 0.27 ms for a flag pass, a scan and an update per level.
+// k_adj_bcast ranks its keys by ballots.  The sums are FP64, whose rate bounds the pass, so they are
+// taken once per level-1 parent (levels 1 and up, a quarter of the keys) and then once per voxel.
+// 1.01 M voxels and 4 coarser levels: 0.116 ms against 0.17 ms when every voxel added every level
+// and 0.27 ms for a flag pass, a scan and an update of the sums per level.
 constexpr int ADJ_MAX_LEVELS = 11;
 constexpr uint32_t ADJ_TILE = 256;   // keys per warp
 struct AdjGrads {
@@ -617,41 +617,86 @@ __global__ void __launch_bounds__(1024) k_adj_scan(uint32_t* __restrict__ part, 
     }
 }
 
-__global__ void __launch_bounds__(256) k_adj_bcast(const uint64_t* __restrict__ keys, uint32_t n, int L, uint32_t nw,
-                                                   const uint32_t* __restrict__ part, AdjGrads G,
-                                                   double* __restrict__ gm, double* __restrict__ gM) {
+constexpr int ADJ_BC_WARPS = 4;
+__global__ void __launch_bounds__(ADJ_BC_WARPS * 32) k_adj_bcast(const uint64_t* __restrict__ keys, uint32_t n, int L,
+                                                                 uint32_t nw, const uint32_t* __restrict__ part,
+                                                                 AdjGrads G, double* __restrict__ gm,
+                                                                 double* __restrict__ gM) {
+    struct Shared {
+        double sum[7 * 64];                      // the parents' sums, component-major
+        uint32_t row[ADJ_MAX_LEVELS * 64];       // the parents' rows in levels 1 .. L
+    };
+    __shared__ Shared shared[ADJ_BC_WARPS];
+    Shared& sh = shared[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const uint32_t w = (blockIdx.x * 256u + threadIdx.x) >> 5;
+    const uint32_t w = blockIdx.x * ADJ_BC_WARPS + (threadIdx.x >> 5);
     if (w >= nw) return;
-    uint32_t base[ADJ_MAX_LEVELS];   // parents of level l + 1 before this warp's keys
+    uint32_t base[ADJ_MAX_LEVELS];   // parents of level l + 1 before this chunk's keys
 #pragma unroll
     for (int l = 0; l < ADJ_MAX_LEVELS; ++l) base[l] = l < L ? part[(size_t)l * nw + w] : 0u;
-    for (uint32_t r = 0; r < ADJ_TILE; r += 32) {
-        const uint32_t i = w * ADJ_TILE + r + lane;
-        const int h = head_level(keys, i, n, L);
-        double m = 0.0, M[6] = {0, 0, 0, 0, 0, 0};
-        if (i < n) {
-            m = (double)G.mass[0][i];
+    for (uint32_t r = 0; r < ADJ_TILE; r += 64) {
+        const uint32_t i0 = w * ADJ_TILE + r;
+        if (i0 >= n) break;
+        uint32_t loc[2] = {0, 0}, first = 0;
+        if (L > 0) {
 #pragma unroll
-            for (int c = 0; c < 6; ++c) M[c] = (double)G.moment[0][(size_t)i * 6 + c];
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t i = i0 + 32u * half + lane;
+                const int h = head_level(keys, i, n, L);
+                uint32_t p[ADJ_MAX_LEVELS];
+#pragma unroll
+                for (int l = 0; l < ADJ_MAX_LEVELS; ++l) {
+                    if (l >= L) break;
+                    const uint32_t b = __ballot_sync(0xffffffffu, h > l);
+                    p[l] = base[l] + __popc(b & (0xffffffffu >> (31 - lane))) - 1u;   // key i's own start counts
+                    base[l] += __popc(b);
+                }
+                if (half == 0) first = __shfl_sync(0xffffffffu, p[0], 0);
+                loc[half] = p[0] - first;
+                // a parent's rows from its first key in the chunk
+                if (i < n && (h > 0 || (half == 0 && lane == 0))) {
+#pragma unroll
+                    for (int l = 0; l < ADJ_MAX_LEVELS; ++l) {
+                        if (l >= L) break;
+                        sh.row[l * 64 + loc[half]] = p[l];
+                    }
+                }
+            }
+            __syncwarp();
+            const uint32_t parents = base[0] - first;
+            for (uint32_t q = lane; q < parents; q += 32) {
+                double m = 0.0, M[6] = {0, 0, 0, 0, 0, 0};
+                for (int l = 0; l < L; ++l) {
+                    const uint32_t p = sh.row[l * 64 + q];
+                    const float* g = G.moment[l + 1] + (size_t)p * 6;
+                    m += (double)G.mass[l + 1][p];
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) M[c] += (double)g[c];
+                }
+                sh.sum[q] = m;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) sh.sum[(c + 1) * 64 + q] = M[c];
+            }
+            __syncwarp();
         }
 #pragma unroll
-        for (int l = 0; l < ADJ_MAX_LEVELS; ++l) {
-            if (l >= L) break;
-            const uint32_t b = __ballot_sync(0xffffffffu, h > l);
-            const uint32_t p = base[l] + __popc(b & (0xffffffffu >> (31 - lane))) - 1u;   // key i's own start counts
-            base[l] += __popc(b);
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t i = i0 + 32u * half + lane;
             if (i < n) {
-                m = m + (double)G.mass[l + 1][p];
+                double g[7];
+                g[0] = (double)G.mass[0][i];
 #pragma unroll
-                for (int c = 0; c < 6; ++c) M[c] = M[c] + (double)G.moment[l + 1][(size_t)p * 6 + c];
+                for (int c = 0; c < 6; ++c) g[c + 1] = (double)G.moment[0][(size_t)i * 6 + c];
+                if (L > 0) {
+#pragma unroll
+                    for (int c = 0; c < 7; ++c) g[c] += sh.sum[c * 64 + loc[half]];
+                }
+                gm[i] = g[0];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) gM[(size_t)i * 6 + c] = g[c + 1];
             }
         }
-        if (i < n) {
-            gm[i] = m;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) gM[(size_t)i * 6 + c] = M[c];
-        }
+        __syncwarp();   // the sums have been read
     }
 }
 
@@ -669,29 +714,53 @@ cudaError_t adj_broadcast(const uint64_t* keys, uint32_t n, int L, const float* 
         k_adj_counts<<<blocks, 256, 0, s>>>(keys, n, L, nw, part);
         k_adj_scan<<<L, 1024, 0, s>>>(part, nw);
     }
-    k_adj_bcast<<<blocks, 256, 0, s>>>(keys, n, L, nw, part, G, gm, gM);
+    k_adj_bcast<<<(nw + ADJ_BC_WARPS - 1) / ADJ_BC_WARPS, ADJ_BC_WARPS * 32, 0, s>>>(keys, n, L, nw, part, G, gm, gM);
     return cudaGetLastError();
 }
 inline size_t adj_part_bytes(uint32_t n, int L) { return ((size_t)n / ADJ_TILE + 1) * std::max(L, 1) * 4; }
 
+// FP64 operations of the adjoint are few per clock (two lanes per SM), so what can run elsewhere
+// does: reciprocals and inverse roots start from the special-function unit's approximation and take
+// two Newton steps (relative error below 2^-51; no bit-exact contract here), and comparisons of
+// doubles whose order is that of their bits as integers run as integers.
+__device__ __forceinline__ double d_rcp(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double d_rsqrt(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double h = 0.5 * x;
+    y = fma(y, fma(-h * y, y, 0.5), y);
+    return fma(y, fma(-h * y, y, 0.5), y);
+}
+
 // Per-segment constants of the fiber adjoint (grid units, FP64), in a warp's shared memory with
-// the segment's slot fastest: A, d = B - A, 1 / d per component (0 for 0), unit tangent, |d|, r, w.
-constexpr int SEGC = 15;
+// the segment's slot fastest: A, d = B - A, 1 / d per component (0 for 0), unit tangent, |d|, r, w,
+// 1 / |d|, 1 / r.
+constexpr int SEGC = 17;
 __device__ __forceinline__ void seg_constants(float4 Af, float4 Bf, double* __restrict__ c, int slot) {
     const double A[3] = {Af.x, Af.y, Af.z};
     const double d[3] = {(double)Bf.x - Af.x, (double)Bf.y - Af.y, (double)Bf.z - Af.z};
-    const double dn = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    const double idn = dn > 0.0 ? 1.0 / dn : 0.0;
+    const double d2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+    const bool some = d2 > 0.0;
+    const double idn = some ? d_rsqrt(d2) : 0.0;
+    const double dn = d2 * idn;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         c[i * 32 + slot] = A[i];
         c[(3 + i) * 32 + slot] = d[i];
-        c[(6 + i) * 32 + slot] = d[i] != 0.0 ? 1.0 / d[i] : 0.0;
+        c[(6 + i) * 32 + slot] = d[i] != 0.0 ? d_rcp(d[i]) : 0.0;
         c[(9 + i) * 32 + slot] = d[i] * idn;
     }
     c[12 * 32 + slot] = dn;
     c[13 * 32 + slot] = Af.w;
     c[14 * 32 + slot] = Bf.w;
+    // (a segment without length or radius has gradients that are not numbers, as 0 / 0)
+    c[15 * 32 + slot] = some ? idn : INFINITY;
+    c[16 * 32 + slot] = Af.w != 0.0f ? d_rcp((double)Af.w) : INFINITY;
 }
 
 // The part [t0, t1] of segment `slot` inside voxel (vi, vj, vk), and the axes whose planes cut it
@@ -705,16 +774,19 @@ __device__ __forceinline__ bool seg_clip(const double* __restrict__ c, int slot,
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const double a = c[i * 32 + slot] - v[i], d = c[(3 + i) * 32 + slot], inv = c[(6 + i) * 32 + slot];
-        if (d == 0.0) {
+        const long long sign = __double_as_longlong(d);
+        if ((sign & 0x7fffffffffffffffll) == 0) {
             if (a < 0.0 || a > 1.0) return false;
         } else {
-            const double ta = -a * inv, tb = (1.0 - a) * inv;
-            const double tn = d > 0.0 ? ta : tb, tf = d > 0.0 ? tb : ta;
-            if (tn > t0) { t0 = tn; ax0 = i; }
-            if (tf < t1) { t1 = tf; ax1 = i; }
+            const double ta = -a * inv, tb = fma(-a, inv, inv);
+            const double tn = sign >= 0 ? ta : tb, tf = sign >= 0 ? tb : ta;
+            // (t0 >= 0, so a larger tn has the larger bits; once t1 is negative the part is empty,
+            // whichever negative value it takes next)
+            if (__double_as_longlong(tn) > __double_as_longlong(t0)) { t0 = tn; ax0 = i; }
+            if (__double_as_longlong(tf) < __double_as_longlong(t1)) { t1 = tf; ax1 = i; }
         }
     }
-    return t1 > t0;
+    return __double_as_longlong(t1) > __double_as_longlong(t0);
 }
 
 // d/d(A, B, r, w) of  w * pi r^2 len * (gm + gM . T(t))  for the part [t0, t1] of segment `slot`
@@ -738,7 +810,7 @@ __device__ __forceinline__ void pair_grad(const double* __restrict__ c, int slot
     const double tg = fma(t[0], gt[0], fma(t[1], gt[1], t[2] * gt[2]));
     const double G = fma(0.5, tg, gm);
     out[7] = mu * G;                     // d/dw
-    out[6] = w * (2.0 * mu / r) * G;     // d/dr
+    out[6] = w * (2.0 * mu * c[16 * 32 + slot]) * G;     // d/dr
     // d len / d A, d B: the clipped ends (1 - t_e) A + t_e B move with both endpoints, and an
     // end on a voxel plane also slides along the segment (its t_e depends on the endpoints)
     const double dte = t1 - t0;
@@ -746,7 +818,7 @@ __device__ __forceinline__ void pair_grad(const double* __restrict__ c, int slot
     const double f1 = ax1 >= 0 ? dn * c[(6 + ax1) * 32 + slot] : 0.0;
     const double sA0 = (1.0 - t0) * f0, sB0 = t0 * f0, sA1 = (1.0 - t1) * f1, sB1 = t1 * f1;
     const double kmu = w * pr2 * G;
-    const double wmd = w * mu / dn;
+    const double wmd = w * mu * c[15 * 32 + slot];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         double cA = -dte * t[k], cB = dte * t[k];
@@ -854,8 +926,8 @@ struct SegWalk {
 // twenty, so the voxels come from the axis alone.  They go into a queue of the warp and are taken
 // 32 at a time, so that the FP64 work (the bound: 2 operations per clock and SM) runs with full
 // lanes whatever the segments' lengths; each segment's terms are added in the order of its walk.
-// 768k segments at 256^3: 0.44 ms, against 9.8 ms for a warp per segment over its candidate pairs
-// (and 0.5 ms to count and emit those).
+// 768k segments at 256^3: 0.34 ms (0.44 with IEEE quotients and roots), against 9.8 ms for a warp per
+// segment over its candidate pairs (and 0.5 ms to count and emit those).
 constexpr int ADJ_WARPS = 4;
 __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4* __restrict__ ra,
                                                                    const float4* __restrict__ rb, uint32_t np, int R,
@@ -1015,14 +1087,18 @@ __global__ void k_adjoint_ctrl(const int64_t* __restrict__ off, int64_t F, const
 // border row) stays inside, and its derivative is that of the piece it belongs to.
 // Only the planes that some vertex of the triangle lies beyond are clipped against.
 // buf: the warp's two polygons, ADJ_POLY doubles (element (poly, vertex, coord) of lane t at
-// [((poly * 12 + vertex) * 5 + coord) * 32 + t]); a vertex carries x, y, z (exact for the
+// [((poly * ADJ_VERTS + vertex) * 5 + coord) * 32 + t]); a vertex carries x, y, z (exact for the
 // triangle's own vertices) and s, t.
-constexpr int ADJ_POLY = 2 * 12 * 5 * 32;
-__device__ __forceinline__ bool tri_pair_grad(const float4 P0, const float4 P1, const float4 P2, int vi, int vj, int vk,
-                                              const double* __restrict__ gmp, const double* __restrict__ gMp,
+// (six planes cut a triangle into a polygon of at most nine vertices)
+constexpr int ADJ_VERTS = 9;
+constexpr int ADJ_POLY = 2 * ADJ_VERTS * 5 * 32;
+// Called by the whole warp, `on` telling which lanes have a pair: every clip is made by all lanes that
+// need one together.
+__device__ __forceinline__ bool tri_pair_grad(bool on, const float4 P0, const float4 P1, const float4 P2, int vi, int vj,
+                                              int vk, const double* __restrict__ gmp, const double* __restrict__ gMp,
                                               double* __restrict__ buf, double* out) {
     const int lane = threadIdx.x & 31;
-    auto at = [&](int poly, int v, int c) -> double& { return buf[((poly * 12 + v) * 5 + c) * 32 + lane]; };
+    auto at = [&](int poly, int v, int c) -> double& { return buf[((poly * ADJ_VERTS + v) * 5 + c) * 32 + lane]; };
     const int vox[3] = {vi, vj, vk};
     const float U[3][3] = {{P0.x, P0.y, P0.z}, {P1.x, P1.y, P1.z}, {P2.x, P2.y, P2.z}};
     uint32_t need = 0;   // bit 2 k + side: plane k = vox (side 0) or vox + 1 has a vertex beyond it
@@ -1039,49 +1115,93 @@ __device__ __forceinline__ bool tri_pair_grad(const float4 P0, const float4 P1, 
     // label of the edge i -> i + 1, four bits each: 0 a triangle edge, 1 + plane a voxel plane
     uint64_t lab = 0;
     int n = 3, cur = 0;
-    while (need && n > 0) {
-        const int c = __ffs(need) - 1, k = c >> 1;
-        need &= need - 1;
+    if (!on) need = 0;
+    while (__any_sync(0xffffffffu, need != 0u)) {
+        const bool work = need != 0u;
+        const int c = work ? __ffs(need) - 1 : 0, k = c >> 1;
+        need &= need - 1u;
         const bool hi = c & 1;
-        const double bound = hi ? 1.0 : 0.0;
-        uint64_t qlab = 0;
-        int m = 0;
-        double xi = at(cur, 0, k);
-        const double x0 = xi;
-        bool in = hi ? xi <= 1.0 : xi >= 0.0;
-        const bool in0 = in;
-        for (int i = 0; i < n; ++i) {
-            const bool last = i + 1 == n;
-            const int j = last ? 0 : i + 1;
-            const double xj = last ? x0 : at(cur, j, k);
-            const bool jn = last ? in0 : (hi ? xj <= 1.0 : xj >= 0.0);
-            const uint64_t li = (lab >> (4 * i)) & 15u;
-            if (in && m < 12) {
-#pragma unroll
-                for (int q = 0; q < 5; ++q) at(cur ^ 1, m, q) = at(cur, i, q);
-                qlab |= li << (4 * m);
-                ++m;
+        // inside x >= 0 (x <= 1), on the bits as integers: the polygon holds no negative zero
+        uint32_t in = 0;
+        if (work)
+            for (int i = 0; i < n; ++i) {
+                const long long x = __double_as_longlong(at(cur, i, k));
+                in |= (hi ? x <= 0x3ff0000000000000ll : x >= 0ll) ? 1u << i : 0u;
             }
-            if (in != jn && m < 12) {
-                const double l = (bound - xi) / (xj - xi);
+        __syncwarp();
+        const uint32_t whole = (1u << n) - 1u;
+        if (work && in == 0u) {
+            n = 0;
+            need = 0;
+        }
+        if (work && in != 0u && in != whole) {
+            const double bound = hi ? 1.0 : 0.0;
+            const int nx = cur ^ 1;
+            uint64_t qlab = 0;
+            int m = 0;
+            // the vertices inside whose predecessor is outside: one, unless rounding has bent the
+            // polygon.  Then the part inside is one run, s .. e, and its two crossings are computed
+            // together, instead of in every turn of a loop over the edges.
+            const uint32_t before = ((in << 1) | (in >> (n - 1))) & whole;   // bit i: vertex i - 1 is inside
+            const uint32_t entries = in & ~before;
+            const int run = __popc(in);
+            if ((entries & (entries - 1u)) == 0u && run + 2 <= ADJ_VERTS) {
+                const int s = __ffs(entries) - 1, p = s == 0 ? n - 1 : s - 1;
+                const int e = s + run - 1 >= n ? s + run - 1 - n : s + run - 1, f = e + 1 == n ? 0 : e + 1;
+                const double x0 = at(cur, p, k), x1 = at(cur, e, k);
+                const double l0 = (bound - x0) * d_rcp(at(cur, s, k) - x0), l1 = (bound - x1) * d_rcp(at(cur, f, k) - x1);
 #pragma unroll
                 for (int q = 0; q < 5; ++q) {
-                    const double a = at(cur, i, q);
-                    at(cur ^ 1, m, q) = q == k ? bound : fma(l, at(cur, j, q) - a, a);
+                    const double a0 = at(cur, p, q), a1 = at(cur, e, q);
+                    const double y0 = fma(l0, at(cur, s, q) - a0, a0), y1 = fma(l1, at(cur, f, q) - a1, a1);
+                    at(nx, 0, q) = q == k ? bound : y0;
+                    at(nx, run + 1, q) = q == k ? bound : y1;
                 }
-                qlab |= (in ? (uint64_t)(c + 1) : li) << (4 * m);
-                ++m;
+                qlab = ((lab >> (4 * p)) & 15u) | ((uint64_t)(c + 1) << (4 * (run + 1)));
+                int i = s;
+                for (m = 1; m <= run; ++m) {
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) at(nx, m, q) = at(cur, i, q);
+                    qlab |= ((lab >> (4 * i)) & 15u) << (4 * m);
+                    i = i + 1 == n ? 0 : i + 1;
+                }
+                m = run + 2;
+            } else {
+                for (int i = 0; i < n; ++i) {
+                    const int j = i + 1 == n ? 0 : i + 1;
+                    const bool a = (in >> i) & 1u, b = (in >> j) & 1u;
+                    const uint64_t li = (lab >> (4 * i)) & 15u;
+                    if (a && m < ADJ_VERTS) {
+                        for (int q = 0; q < 5; ++q) at(nx, m, q) = at(cur, i, q);
+                        qlab |= li << (4 * m);
+                        ++m;
+                    }
+                    if (a != b && m < ADJ_VERTS) {
+                        const double xi = at(cur, i, k), l = (bound - xi) * d_rcp(at(cur, j, k) - xi);
+                        for (int q = 0; q < 5; ++q) {
+                            const double y = at(cur, i, q);
+                            at(nx, m, q) = q == k ? bound : fma(l, at(cur, j, q) - y, y);
+                        }
+                        qlab |= (a ? (uint64_t)(c + 1) : li) << (4 * m);
+                        ++m;
+                    }
+                }
             }
-            xi = xj;
-            in = jn;
+            n = m;
+            lab = qlab;
+            cur = nx;
         }
-        n = m;
-        lab = qlab;
-        cur ^= 1;
+        __syncwarp();
     }
-    if (n < 3) return false;
+    if (!on || n < 3) return false;
     const double e1[3] = {(double)P1.x - P0.x, (double)P1.y - P0.y, (double)P1.z - P0.z};
     const double e2[3] = {(double)P2.x - P0.x, (double)P2.y - P0.y, (double)P2.z - P0.z};
+    double ig2[3];   // 1 / |grad g|^2 per axis (0: the plane's constraint does not vary)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double g2 = fma(e1[k], e1[k], e2[k] * e2[k]);
+        ig2[k] = g2 > 0.0 ? d_rcp(g2) : 0.0;
+    }
     double A = 0.0;
     double dA[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     double si = at(cur, 0, 3), ti = at(cur, 0, 4);
@@ -1094,19 +1214,18 @@ __device__ __forceinline__ bool tri_pair_grad(const float4 P0, const float4 P1, 
         if (c >= 0) {
             const int k = c >> 1;
             const double a = k == 0 ? e1[0] : (k == 1 ? e1[1] : e1[2]), b = k == 0 ? e2[0] : (k == 1 ? e2[1] : e2[2]);
-            const double g2 = fma(a, a, b * b);
-            if (g2 > 0.0) {
-                const double f = -fabs(fma(tj - ti, a, -(sj - si) * b)) / g2 * ((c & 1) ? 1.0 : -1.0);
-                const double sm = 0.5 * (si + sj), tm = 0.5 * (ti + tj);
-                const double d0 = f * (1.0 - sm - tm), d1 = f * sm, d2 = f * tm;
+            const double g = k == 0 ? ig2[0] : (k == 1 ? ig2[1] : ig2[2]);
+            const double len = fabs(fma(tj - ti, a, (si - sj) * b)) * g;
+            const double f = (c & 1) ? -len : len;
+            const double sm = 0.5 * (si + sj), tm = 0.5 * (ti + tj);
+            const double d1 = f * sm, d2 = f * tm, d0 = (f - d1) - d2;
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (k == q) {
-                        dA[0][q] += d0;
-                        dA[1][q] += d1;
-                        dA[2][q] += d2;
-                    }
-            }
+            for (int q = 0; q < 3; ++q)
+                if (k == q) {
+                    dA[0][q] += d0;
+                    dA[1][q] += d1;
+                    dA[2][q] += d2;
+                }
         }
         si = sj;
         ti = tj;
@@ -1114,9 +1233,9 @@ __device__ __forceinline__ bool tri_pair_grad(const float4 P0, const float4 P1, 
     A *= 0.5;
     const double nr[3] = {fma(e1[1], e2[2], -e1[2] * e2[1]), fma(e1[2], e2[0], -e1[0] * e2[2]),
                           fma(e1[0], e2[1], -e1[1] * e2[0])};
-    const double J = sqrt(fma(nr[0], nr[0], fma(nr[1], nr[1], nr[2] * nr[2])));
-    if (!(J > 0.0) || !(A > 0.0)) return false;
-    const double iJ = 1.0 / J;
+    const double J2 = fma(nr[0], nr[0], fma(nr[1], nr[1], nr[2] * nr[2]));
+    if (!(J2 > 0.0) || !(A > 0.0)) return false;
+    const double iJ = d_rsqrt(J2), J = J2 * iJ;
     const double nh[3] = {nr[0] * iJ, nr[1] * iJ, nr[2] * iJ};
     const double mu = J * A;
     double gM[6];
@@ -1152,9 +1271,10 @@ __device__ __forceinline__ bool tri_pair_grad(const float4 P0, const float4 P1, 
 // triangles per block of one warp: lanes test the voxels of their triangle's box and queue its
 // candidates, which are taken 32 at a time so that the FP64 work runs with full lanes; each
 // triangle's terms are added in the order in which its lanes found them.  One warp per block: its
-// polygons take 31 KB of shared memory, which leaves six resident per SM, enough for the FP64
-// pipe that bounds the kernel.  178,802 triangles at 256^3: 1.6 ms, against 10.1 ms for a warp per
-// triangle (eight pairs in its lanes), six planes and polygons in local memory.
+// polygons take 23 KB of shared memory, which leaves eight resident per SM, enough for the FP64
+// pipe that bounds the kernel (76 % busy).  178,802 triangles at 256^3: 1.1 ms; 1.6 ms with the
+// crossings inside a loop over the edges, 1.8 ms with each lane clipping at its own pace, 10.1 ms for
+// a warp per triangle (eight pairs in its lanes), six planes and polygons in local memory.
 __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ r0, const float4* __restrict__ r1,
                                                      const float4* __restrict__ r2, uint32_t np, Window R, int lg,
                                                      const uint64_t* __restrict__ keys0, uint32_t V0,
@@ -1201,16 +1321,21 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
             const bool on = (uint32_t)lane < min(qn, 32u);
             const uint64_t e = queue[lane];
             const int own = on ? (int)(e >> 36) : 32;
-            bool hit = false;
             double g[10];
+            int ex = 0, ey = 0, ez = 0;
+            uint32_t v = 0;
+            float4 A = make_float4(0, 0, 0, 0), B = A, C = A;
+            bool found = false;
             if (on) {
-                const int ex = (int)(e >> 24) & 0xfff, ey = (int)(e >> 12) & 0xfff, ez = (int)e & 0xfff;
+                ex = (int)(e >> 24) & 0xfff, ey = (int)(e >> 12) & 0xfff, ez = (int)e & 0xfff;
                 const uint64_t k = voxel_key((uint32_t)ex, (uint32_t)ey, (uint32_t)ez);
-                const uint32_t v = lower_key(keys0, 0, V0, k);
-                if (v < V0 && keys0[v] == k)
-                    hit = tri_pair_grad(r0[p0 + own], r1[p0 + own], r2[p0 + own], ex, ey, ez, gm + v, gM + (size_t)v * 6,
-                                        poly, g);
+                v = lower_key(keys0, 0, V0, k);
+                found = v < V0 && keys0[v] == k;
+                A = r0[p0 + own];
+                B = r1[p0 + own];
+                C = r2[p0 + own];
             }
+            const bool hit = tri_pair_grad(found, A, B, C, ex, ey, ez, gm + v, gM + (size_t)v * 6, poly, g);
             // entries of one triangle are added one after the other, in queue order
             const uint32_t peers = __match_any_sync(0xffffffffu, hit ? own : 32 + lane);
             const int rank = __popc(peers & lt);
