@@ -4,6 +4,7 @@
 // primitive-id order inside each key (stability), which is what makes the per-voxel
 // reductions order-deterministic (the paper sorts samples by block id, Sec. 3.3).
 #include <algorithm>
+#include <type_traits>
 
 #include "vx_internal.cuh"
 
@@ -343,6 +344,19 @@ __global__ void __launch_bounds__(SORT_THREADS) k_radix_hist(const uint32_t* __r
     for (int d = threadIdx.x; d < RB; d += SORT_THREADS) hist[(size_t)d * nt + blockIdx.x] = h[d];
 }
 
+// The lanes whose BITS-bit digit equals this lane's, among those with `valid`: one ballot per bit,
+// five instructions each.  __match_any_sync is one instruction, but its time grows with the number
+// of distinct digits in the warp and it left the scatter waiting for it: the first pass over 27 M
+// pairs, whose lanes hold mostly different digits, took 0.43 ms and takes 0.27 ms.
+template <int BITS>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid) {
+    uint32_t other = ~__ballot_sync(0xffffffffu, valid);
+    int x = (int)(d << (32 - BITS));
+#pragma unroll
+    for (int b = 0; b < BITS; ++b, x <<= 1) other |= __ballot_sync(0xffffffffu, x < 0) ^ (uint32_t)(x >> 31);
+    return ~other;
+}
+
 // Stable scatter of one tile.  Each element's rank inside the tile (digit-major, original
 // order within a digit) is found with per-warp running counters; the tile is then
 // rearranged into that order in shared memory and written out with consecutive threads on
@@ -355,7 +369,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 3) k_radix_scatter(const uint32_
                                                                 const uint32_t* __restrict__ hist,
                                                                 uint32_t* __restrict__ okeys,
                                                                 uint32_t* __restrict__ ovals) {
-    static_assert(RB % SORT_THREADS == 0, "digits per thread");
+    static_assert(RB == 256, "digits per thread and bits of a digit");
     union Stage {
         uint32_t wcnt[SORT_WARPS][RB];           // ranking: per-warp counts, then warp offsets
         struct {
@@ -380,8 +394,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 3) k_radix_scatter(const uint32_
         bool valid = e < n;
         k[j] = valid ? keys[e] : 0u;
         v[j] = valid ? vals[e] : 0u;
-        uint32_t d = valid ? radix_digit<LUT>(k[j], v[j], shift, dmask, lut) : (uint32_t)RB;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
+        uint32_t d = valid ? radix_digit<LUT>(k[j], v[j], shift, dmask, lut) : 0u;
+        uint32_t peers = digit_peers<8>(d, valid);
         uint32_t r = 0;
         if (valid) r = st.wcnt[w][d] + __popc(peers & lt);
         __syncwarp();
@@ -451,6 +465,13 @@ __global__ void __launch_bounds__(SORT_THREADS, 3) k_radix_scatter(const uint32_
 // async copies (cp.async.bulk, completion on an mbarrier).  Each wait is bounded: a wait that
 // gives up sets bit 4 of *err, waits (bounded) for the block's own copies still in flight,
 // and ends the block (the host then reports VX_ERR_TIMEOUT).
+//
+// Bound by instruction issue and the shared-memory pipe together (50 % each at 16 warps per SM);
+// HBM is at 3.3 TB/s.  Tiles of 4,096 by 256 threads, two blocks per SM: three blocks (80
+// registers), 512 threads and tiles of 8,192 were 10 to 30 % slower.  25 M pairs, three passes of
+// nine bits: 1.13 ms, against 1.45 ms with __match_any_sync for the ranking and one more shared
+// word per item for the digit's place in the tile; 27 M pairs, four passes of eight bits: 1.87
+// against 2.35 ms.
 constexpr uint32_t PIPE_SPIN_LIMIT = 1u << 22;   // try_wait polls before a wait gives up
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -486,8 +507,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 
 constexpr size_t pipe_smem(int rb) {
     return (size_t)2 * 2 * SORT_TILE * 4                 // two stages of keys + values
-           + (size_t)SORT_WARPS * rb * 4                 // per-warp digit counters
-           + (size_t)2 * rb * 4                          // gofs, tofs
+           + (size_t)SORT_WARPS * rb * 2                 // per-warp digit counters
+           + (size_t)rb * 4                              // gofs
            + 64;                                         // scan scratch, barriers
 }
 
@@ -499,14 +520,14 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
                                                                       uint32_t* __restrict__ okeys,
                                                                       uint32_t* __restrict__ ovals,
                                                                       uint32_t* __restrict__ err) {
-    static_assert(RB % SORT_THREADS == 0, "digits per thread");
+    static_assert((RB == 256 || RB == 512) && RB % SORT_THREADS == 0, "digit widths");
+    constexpr int BITS = RB == 512 ? 9 : 8;
     extern __shared__ __align__(128) unsigned char sm_raw[];
     // stage s: keys at sm + 2 s TILE, values right after them
     uint32_t* const stage0 = (uint32_t*)sm_raw;
-    uint32_t (*wcnt)[RB] = reinterpret_cast<uint32_t (*)[RB]>((uint32_t*)sm_raw + 4 * SORT_TILE);
-    uint32_t* gofs = (uint32_t*)sm_raw + 4 * SORT_TILE + SORT_WARPS * RB;
-    uint32_t* tofs = gofs + RB;
-    uint32_t* scan_tmp = tofs + RB;                       // SORT_WARPS + 1 words
+    uint16_t (*wcnt)[RB] = reinterpret_cast<uint16_t (*)[RB]>((uint32_t*)sm_raw + 4 * SORT_TILE);
+    uint32_t* gofs = (uint32_t*)sm_raw + 4 * SORT_TILE + SORT_WARPS * RB / 2;
+    uint32_t* scan_tmp = gofs + RB;                               // SORT_WARPS + 1 words
     uint64_t* bar = reinterpret_cast<uint64_t*>(scan_tmp + 12);   // 8-byte aligned: two barriers
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
@@ -533,11 +554,11 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
     int st = 0;
     // this thread's digits' global offsets for the tile in hand, loaded one tile ahead (the
     // digit-major histogram puts a tile's offsets a stride nt apart)
-    constexpr int DPG = RB / SORT_THREADS;
-    uint32_t gcur[DPG];
+    constexpr int DPT = RB / SORT_THREADS;   // digits per thread
+    uint32_t gcur[DPT];
 #pragma unroll
-    for (int i = 0; i < DPG; ++i)
-        gcur[i] = blockIdx.x < nt ? hist[(size_t)(threadIdx.x + i * SORT_THREADS) * nt + blockIdx.x] : 0u;
+    for (int i = 0; i < DPT; ++i)
+        gcur[i] = blockIdx.x < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + blockIdx.x] : 0u;
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x, st ^= 1) {
         // the next tile streams into the other stage (its last reader finished: the loop ends
         // with a barrier); generic writes to that stage are ordered before the async copy
@@ -549,14 +570,81 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
             }
             pending |= 1u << (st ^ 1);
         }
-        uint32_t gnxt[DPG];
+        uint32_t gnxt[DPT];
 #pragma unroll
-        for (int i = 0; i < DPG; ++i)
-            gnxt[i] = tn < nt ? hist[(size_t)(threadIdx.x + i * SORT_THREADS) * nt + tn] : 0u;
+        for (int i = 0; i < DPT; ++i)
+            gnxt[i] = tn < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + tn] : 0u;
         const size_t tile0 = (size_t)t * SORT_TILE;
         const uint32_t tn_items = (uint32_t)min((size_t)SORT_TILE, (size_t)n - tile0);
         uint32_t* const sk = stage0 + (size_t)st * 2 * SORT_TILE;
         uint32_t* const sv = sk + SORT_TILE;
+        // ranks the tile's items and writes them out; WHOLE: no item is out of range
+        auto place = [&](auto whole) {
+            constexpr bool WHOLE = decltype(whole)::value;
+            const uint32_t lb = (uint32_t)w * (32 * SORT_ITEMS) + lane;
+            // rank within the warp: the peers of every item first (independent of each other),
+            // then the running counters, item by item (stable within the tile)
+            uint32_t k[SORT_ITEMS], v[SORT_ITEMS], rk[SORT_ITEMS];
+#pragma unroll
+            for (int j = 0; j < SORT_ITEMS; ++j) {
+                k[j] = sk[lb + j * 32];
+                rk[j] = digit_peers<BITS>((k[j] >> shift) & dmask, WHOLE || lb + j * 32 < tn_items);
+            }
+#pragma unroll
+            for (int j = 0; j < SORT_ITEMS; ++j) {
+                const bool valid = WHOLE || lb + j * 32 < tn_items;
+                const uint32_t d = (k[j] >> shift) & dmask, below = __popc(rk[j] & lt);
+                uint32_t r = 0;
+                if (valid) r = wcnt[w][d];
+                __syncwarp();
+                if (valid && below == 0) wcnt[w][d] = (uint16_t)(r + __popc(rk[j]));
+                __syncwarp();
+                rk[j] = r + below;
+            }
+            __syncthreads();
+            // exclusive prefix over the tile, digit-major, then warp by warp: a counter becomes
+            // the place of its warp's first item of that digit
+            uint32_t c[DPT][SORT_WARPS], sum = 0;
+#pragma unroll
+            for (int i = 0; i < DPT; ++i)
+#pragma unroll
+                for (int ww = 0; ww < SORT_WARPS; ++ww) {
+                    c[i][ww] = wcnt[ww][threadIdx.x * DPT + i];
+                    sum += c[i][ww];
+                }
+            const uint32_t inc = warp_incl_scan(sum);
+            if (lane == 31) scan_tmp[w] = inc;
+            __syncthreads();
+            uint32_t ex = __reduce_add_sync(0xffffffffu, lane < w ? scan_tmp[lane] : 0u) + inc - sum;
+#pragma unroll
+            for (int i = 0; i < DPT; ++i) {
+                gofs[threadIdx.x * DPT + i] = gcur[i] - ex;
+#pragma unroll
+                for (int ww = 0; ww < SORT_WARPS; ++ww) {
+                    wcnt[ww][threadIdx.x * DPT + i] = (uint16_t)ex;
+                    ex += c[i][ww];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < SORT_ITEMS; ++j) v[j] = sv[lb + j * 32];
+            __syncthreads();
+            // the tile in digit order, over the stage it was read from (every item is in registers)
+#pragma unroll
+            for (int j = 0; j < SORT_ITEMS; ++j) {
+                if (WHOLE || lb + j * 32 < tn_items) {
+                    const uint32_t pos = rk[j] + wcnt[w][(k[j] >> shift) & dmask];
+                    sk[pos] = k[j];
+                    sv[pos] = v[j];
+                }
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < (WHOLE ? (uint32_t)SORT_TILE : tn_items); i += SORT_THREADS) {
+                const uint32_t kk = sk[i], vv = sv[i];
+                const uint32_t pos = gofs[(kk >> shift) & dmask] + i;
+                okeys[pos] = kk;
+                ovals[pos] = vv;
+            }
+        };
         bool gave_up = false;
         if ((pending >> st) & 1u) {
             if (mbar_wait(&bar[st], (phase >> st) & 1u)) {
@@ -571,79 +659,16 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
                 sv[i] = vals[tile0 + i];
             }
         }
-        for (int i = threadIdx.x; i < SORT_WARPS * RB; i += SORT_THREADS) (&wcnt[0][0])[i] = 0;
-#pragma unroll
-        for (int i = 0; i < DPG; ++i) gofs[threadIdx.x + i * SORT_THREADS] = gcur[i];
+        for (int i = threadIdx.x; i < SORT_WARPS * RB / 2; i += SORT_THREADS) reinterpret_cast<uint32_t*>(&wcnt[0][0])[i] = 0;
         // the whole block leaves together when any thread's wait gave up
         if (__syncthreads_or(gave_up)) {
             lost = true;
             break;
         }
-        // rank: per-warp running counters (stable within the tile)
-        uint32_t k[SORT_ITEMS], v[SORT_ITEMS], rk[SORT_ITEMS];
-        const uint32_t lb = (uint32_t)w * (32 * SORT_ITEMS);
+        if (tn_items == SORT_TILE) place(std::true_type{});
+        else place(std::false_type{});
 #pragma unroll
-        for (int j = 0; j < SORT_ITEMS; ++j) {
-            const uint32_t e = lb + (uint32_t)j * 32 + lane;
-            const bool valid = e < tn_items;
-            k[j] = valid ? sk[e] : 0u;
-            v[j] = valid ? sv[e] : 0u;
-            const uint32_t d = valid ? ((k[j] >> shift) & dmask) : (uint32_t)RB;
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
-            uint32_t r = 0;
-            if (valid) r = wcnt[w][d] + __popc(peers & lt);
-            __syncwarp();
-            if (valid && lane == __ffs(peers) - 1) wcnt[w][d] += __popc(peers);
-            __syncwarp();
-            rk[j] = r;
-        }
-        __syncthreads();
-        constexpr int DPT = RB / SORT_THREADS;
-        uint32_t cnt[DPT];
-#pragma unroll
-        for (int i = 0; i < DPT; ++i) {
-            const int d = threadIdx.x * DPT + i;
-            uint32_t run = 0;
-#pragma unroll
-            for (int ww = 0; ww < SORT_WARPS; ++ww) {
-                const uint32_t c = wcnt[ww][d];
-                wcnt[ww][d] = run;
-                run += c;
-            }
-            cnt[i] = run;
-        }
-        uint32_t sum = 0;
-#pragma unroll
-        for (int i = 0; i < DPT; ++i) sum += cnt[i];
-        uint32_t total;
-        uint32_t ex = block_excl_scan(sum, scan_tmp, total);
-#pragma unroll
-        for (int i = 0; i < DPT; ++i) {
-            tofs[threadIdx.x * DPT + i] = ex;
-            ex += cnt[i];
-        }
-        __syncthreads();
-        // the tile in digit order, over the stage it was read from (every item is in registers)
-#pragma unroll
-        for (int j = 0; j < SORT_ITEMS; ++j) {
-            const uint32_t e = lb + (uint32_t)j * 32 + lane;
-            if (e < tn_items) {
-                const uint32_t d = (k[j] >> shift) & dmask;
-                const uint32_t pos = rk[j] + tofs[d] + wcnt[w][d];
-                sk[pos] = k[j];
-                sv[pos] = v[j];
-            }
-        }
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < tn_items; i += SORT_THREADS) {
-            const uint32_t kk = sk[i], vv = sv[i];
-            const uint32_t d = (kk >> shift) & dmask;
-            const uint32_t pos = gofs[d] + (i - tofs[d]);
-            okeys[pos] = kk;
-            ovals[pos] = vv;
-        }
-#pragma unroll
-        for (int i = 0; i < DPG; ++i) gcur[i] = gnxt[i];
+        for (int i = 0; i < DPT; ++i) gcur[i] = gnxt[i];
         __syncthreads();
     }
     if (lost) {
@@ -777,7 +802,7 @@ vx_status vx_radix_sort_u32(vx_context* ctx, uint32_t** keys, uint32_t** vals, u
     const int passes = digit_plan(bits, widths);
     int wmax = 0;
     for (int p = 0; p < passes; ++p) wmax = std::max(wmax, widths[p]);
-    if (wmax > 10) return VX_ERR_CAPACITY;
+    if (wmax > 9) return VX_ERR_CAPACITY;
     const uint32_t nt = (n + SORT_TILE - 1) / SORT_TILE;
     const size_t hn = ((size_t)1 << std::max(wmax, 8)) * nt;
     if (hn > 0xffffffffull) return VX_ERR_CAPACITY;
@@ -787,9 +812,7 @@ vx_status vx_radix_sort_u32(vx_context* ctx, uint32_t** keys, uint32_t** vals, u
     for (int p = 0; p < passes; ++p) {
         const int w = widths[p];
         const uint32_t dmask = (1u << w) - 1u;
-        if (w > 9)
-            VX_TRY(sort_pass<1024>(ctx, keys, vals, keys_alt, vals_alt, n, shift, dmask, nt, hist, s, err));
-        else if (w > 8)
+        if (w > 8)
             VX_TRY(sort_pass<512>(ctx, keys, vals, keys_alt, vals_alt, n, shift, dmask, nt, hist, s, err));
         else
             VX_TRY(sort_pass<256>(ctx, keys, vals, keys_alt, vals_alt, n, shift, dmask, nt, hist, s, err));

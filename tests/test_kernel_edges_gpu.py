@@ -183,3 +183,22 @@ def test_lobe_counts_at_the_thresholds(N):
             sel = r["lobe_count"] > k
             assert np.array_equal(g["lobes"][sel, k].view(np.uint32), r["lobes"][sel, k].astype(np.float32).view(np.uint32))
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [2, 33, 4095, 4096, 4097, 8192, 12290])
+@pytest.mark.parametrize("R", [4, 8, 64, 256])
+def test_pair_sort_at_the_tile_edges(n, R):
+    """One pair per triangle (each lies inside a voxel), so that n is the sort's length: below, at and
+    above a tile, with key digits of 6, 9, 9 + 9 and 8 + 8 + 8 bits.  Half of the pairs share one
+    voxel, whose FP32 sums depend on the order that a stable sort keeps."""
+    rng = np.random.default_rng(n + R)
+    cell = rng.integers(0, R, (n, 3))
+    cell[rng.random(n) < 0.5] = cell[0]
+    v = (cell[:, None, :] + rng.uniform(0.3, 0.7, (n, 3, 3))) / R
+    tris = np.zeros((n, 3, 4), np.float32)
+    tris[..., :3] = v
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    w = synth.Workload("cells", "triangles", grid, tri_verts=tris, K=1)
+    ctx = vx.Context(DEV)
+    _same_level0(ctx.voxelize(grid, tri_verts=torch.from_numpy(tris).to(DEV)), oracle.voxelize(w))
+    ctx.close()
