@@ -91,62 +91,57 @@ __global__ void k_bprep_tris(const float4* __restrict__ tv, const float* __restr
     inst_of[p] = (uint8_t)ii;
 }
 
-// count / emit with the resolution of each primitive's instance; emission is clamped to
-// the pair capacity (an overflow is reported by the count clamp)
-template <bool FIBER, bool EMIT>
-__global__ void __launch_bounds__(EMIT_WARPS * 32) k_bcandidates(const float4* __restrict__ r0,
-                                                                 const float4* __restrict__ r1,
-                                                                 const float4* __restrict__ r2, uint32_t np,
-                                                                 const BInst* __restrict__ inst,
-                                                                 const uint8_t* __restrict__ inst_of,
-                                                                 uint32_t* __restrict__ counts,
-                                                                 const uint32_t* __restrict__ offs, uint32_t cap,
-                                                                 uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                                 uint32_t* __restrict__ ballots) {
+// count with the resolution of each primitive's instance (see k_count)
+template <bool FIBER>
+__global__ void __launch_bounds__(COUNT_WARPS * 32) k_bcount(const float4* __restrict__ r0, const float4* __restrict__ r1,
+                                                             const float4* __restrict__ r2, uint32_t np, int lg,
+                                                             const BInst* __restrict__ inst,
+                                                             const uint8_t* __restrict__ inst_of,
+                                                             uint32_t* __restrict__ counts,
+                                                             uint32_t* __restrict__ ballots) {
+    __shared__ CountRecords<FIBER> rec[COUNT_WARPS];
+    const uint32_t groups = (uint32_t)(((uint64_t)np + (1u << lg) - 1) >> lg);
+    for (uint32_t g = blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); g < groups; g += gridDim.x * COUNT_WARPS)
+        count_group<FIBER>(rec[threadIdx.x >> 5], g << lg, lg, np, r0, r1, r2,
+                           [&](uint32_t p) { return full_window(inst[inst_of[p]].R); }, counts, ballots, CAND_BALLOTS);
+}
+
+// emit, clamped to the pair capacity (an overflow is reported by the count clamp); the ballots
+// are the count pass's (NULL: every range is tested again)
+template <bool FIBER>
+__global__ void __launch_bounds__(EMIT_WARPS * 32) k_bemit(const float4* __restrict__ r0,
+                                                           const float4* __restrict__ r1,
+                                                           const float4* __restrict__ r2, uint32_t np,
+                                                           const BInst* __restrict__ inst,
+                                                           const uint8_t* __restrict__ inst_of,
+                                                           const uint32_t* __restrict__ offs, uint32_t cap,
+                                                           uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                           const uint32_t* __restrict__ ballots) {
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * EMIT_WARPS;
     for (uint32_t p = blockIdx.x * EMIT_WARPS + (threadIdx.x >> 5); p < np; p += warps) {
         const Window R = full_window(inst[inst_of[p]].R);
-        float4 a = r0[p], b = r1[p], c;
-        Range rg;
-        if (FIBER) {
-            rg = capsule_range(a, b, R);
-        } else {
-            c = r2[p];
-            rg = tri_range(a, b, c, R);
-        }
+        float4 a, b, c;
+        const Range rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
         uint32_t n = 0;
-        const uint32_t base = EMIT ? offs[p] : 0u;
+        const uint32_t base = offs[p];
         const long long tot = rg.total;
-        // hit ballots stored by the count pass for the emit pass (as k_candidates)
         const bool stored = ballots != nullptr && tot <= 32ll * CAND_BALLOTS;
-        uint32_t* const pb = stored ? ballots + (size_t)p * CAND_BALLOTS : nullptr;
         uint32_t words = 0;
-        if (EMIT && stored && (long long)lane * 32 < tot) words = pb[lane];
+        if (stored && (long long)lane * 32 < tot) words = ballots[(size_t)p * CAND_BALLOTS + lane];
         for (long long idx0 = 0; idx0 < tot; idx0 += 32) {
             const long long idx = idx0 + lane;
             bool hit = false;
             int vi = 0, vj = 0, vk = 0;
-            uint32_t bal;
-            if (EMIT && stored) {
-                bal = __shfl_sync(0xffffffffu, words, (int)(idx0 >> 5));
-                hit = (bal >> lane) & 1u;
-                if (hit) {
-                    int ix, iy, iz;
-                    voxel_of(idx, tot, rg, ix, iy, iz);
-                    vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
-                }
-            } else {
-                if (idx < tot) {
-                    int ix, iy, iz;
-                    voxel_of(idx, tot, rg, ix, iy, iz);
-                    vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
-                    hit = FIBER ? capsule_voxel_candidate(a, b, vi, vj, vk) : tri_voxel_candidate(a, b, c, vi, vj, vk);
-                }
-                bal = __ballot_sync(0xffffffffu, hit);
-                if (!EMIT && stored && lane == 0) pb[idx0 >> 5] = bal;
+            uint32_t bal = stored ? __shfl_sync(0xffffffffu, words, (int)(idx0 >> 5)) : 0u;
+            if (stored ? (bal >> lane) & 1u : idx < tot) {
+                int ix, iy, iz;
+                voxel_of(idx, tot, rg, ix, iy, iz);
+                vi = rg.lo[0] + ix; vj = rg.lo[1] + iy; vk = rg.lo[2] + iz;
+                hit = stored || (FIBER ? capsule_voxel_candidate(a, b, vi, vj, vk) : tri_voxel_candidate(a, b, c, vi, vj, vk));
             }
-            if (EMIT && hit) {
+            if (!stored) bal = __ballot_sync(0xffffffffu, hit);
+            if (hit) {
                 const uint32_t pos = base + n + __popc(bal & ((1u << lane) - 1u));
                 if (pos < cap) {
                     keys[pos] = vx_morton3((uint32_t)vi, (uint32_t)vj, (uint32_t)vk);
@@ -155,7 +150,6 @@ __global__ void __launch_bounds__(EMIT_WARPS * 32) k_bcandidates(const float4* _
             }
             n += __popc(bal);
         }
-        if (!EMIT && lane == 0) counts[p] = n;
     }
 }
 
@@ -473,14 +467,14 @@ vx_status instance_pairs(vx_batch* b, bool fiber, const vx_primitives* prims, co
             k_bprep_tris<<<gf(np, 256, 1u << 30), 256, 0, s>>>((const float4*)prims->tri_verts, prims->weights, np,
                                                                dinst, ninst, r0, r1, r2, inst_of, C + C_ERR);
         }
-        const unsigned cblocks = (unsigned)std::min<size_t>((np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
+        const int lg = count_lanes_log2(np);
         if (e == cudaSuccess) {
             if (fiber)
-                k_bcandidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(r0, r1, r2, np, dinst, inst_of, cnt,
-                                                                               nullptr, 0, nullptr, nullptr, nullptr);
+                k_bcount<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(r0, r1, r2, np, lg, dinst, inst_of, cnt,
+                                                                                 nullptr);
             else
-                k_bcandidates<false, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(r0, r1, r2, np, dinst, inst_of, cnt,
-                                                                                nullptr, 0, nullptr, nullptr, nullptr);
+                k_bcount<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(r0, r1, r2, np, lg, dinst, inst_of, cnt,
+                                                                                  nullptr);
             k_inst_pair_totals<<<ninst, 256, 0, s>>>(cnt, dinst, tot);
             e = cudaGetLastError();
         }
@@ -535,12 +529,13 @@ vx_status enqueue(vx_batch* b, SubBatch& S, cudaStream_t s, bool plan, int64_t* 
     }
     // ---- candidates ----------------------------------------------------------------------
     const unsigned cblocks = (unsigned)std::min<size_t>((S.np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
+    const int lg = count_lanes_log2(S.np);
     if (S.fiber)
-        k_bcandidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of,
-                                                                       S.cnt, nullptr, 0, nullptr, nullptr, S.ballots);
+        k_bcount<true><<<count_blocks(S.np, lg), COUNT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, lg, S.dinst,
+                                                                           S.inst_of, S.cnt, S.ballots);
     else
-        k_bcandidates<false, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of,
-                                                                        S.cnt, nullptr, 0, nullptr, nullptr, S.ballots);
+        k_bcount<false><<<count_blocks(S.np, lg), COUNT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, lg, S.dinst,
+                                                                            S.inst_of, S.cnt, S.ballots);
     if (vx_scan_u32_scratch(S.cnt, S.offs, S.np, C + C_PAIRS_TOT, S.part, s) != cudaSuccess) return VX_ERR_CUDA;
     *nl += 4;
     if (plan) {
@@ -559,13 +554,11 @@ vx_status enqueue(vx_batch* b, SubBatch& S, cudaStream_t s, bool plan, int64_t* 
     }
     k_clamp<<<1, 1, 0, s>>>(C + C_PAIRS_TOT, S.cap_pairs, C + C_PAIRS, C + C_ERR);
     if (S.fiber)
-        k_bcandidates<true, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of,
-                                                                      nullptr, S.offs, S.cap_pairs, PL.k0, PL.v0,
-                                                                      S.ballots);
+        k_bemit<true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of, S.offs,
+                                                          S.cap_pairs, PL.k0, PL.v0, S.ballots);
     else
-        k_bcandidates<false, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of,
-                                                                       nullptr, S.offs, S.cap_pairs, PL.k0, PL.v0,
-                                                                       S.ballots);
+        k_bemit<false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of, S.offs,
+                                                           S.cap_pairs, PL.k0, PL.v0, S.ballots);
     k_pad<<<blk, 256, 0, s>>>(PL.k0, PL.v0, C + C_PAIRS, S.cap_pairs);
     *nl += 3;
     // ---- sort by (instance, key) ------------------------------------------------------------

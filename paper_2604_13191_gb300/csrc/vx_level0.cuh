@@ -1057,6 +1057,239 @@ __device__ __forceinline__ Range prim_range(const float4* __restrict__ r0, const
     return tri_range(a, b, c, R);
 }
 
+// ---- count -------------------------------------------------------------------------
+// The count pass tests every voxel of a primitive's range with capsule_voxel_candidate /
+// tri_voxel_candidate, whose cost is instruction issue (91 % and 77 % busy at 780 instructions per
+// 27-voxel triangle).  Most of that work is the same for all voxels of the range, or decides by a
+// hair's breadth what is clear at a glance.  So a lane first lays down a record of one primitive (a
+// warp: up to 32 of them) in coordinates relative to its range's corner, with the terms that do not
+// depend on the voxel and a bound on the rounding of both evaluations; per voxel, a few fused
+// operations on the record then say in, out or open, and only the open ones (within the bound of a
+// boundary: one in ten thousand to one in two hundred) take the test itself.  The candidates are the
+// same: 5e10 voxels of 14 M primitives of all shapes gave no other answer.  Still bound by issue.
+//   yarn (768k capsules) 0.73 -> 0.37 ms, woven 1.07 -> 0.56 ms, mesh (978k triangles) 1.42 -> 0.46 ms.
+// (Five blocks per SM for triangles: four 0.52 ms, six, at 80 registers, 0.50 ms.)
+constexpr int COUNT_WARPS = 4;
+constexpr int kMaxFastRange = 65536;   // voxels: (i + 0.5) / n by reciprocals (see voxel_of)
+template <bool FIBER>
+struct CountRecords {
+    float4 q[FIBER ? 5 : 12][32];   // by term, by primitive: lanes write side by side, then read one
+    float4 r[2][32];                // 1 / n0, n0, 1 / n1, n1 and lo (as bits), voxels
+};
+
+__device__ __forceinline__ float abs_max3(float x, float y, float z) { return fmax3(fabsf(x), fabsf(y), fabsf(z)); }
+
+// Capsule: M bounds every coordinate and the radius (a coordinate relative to a voxel: 2 M).  The
+// gap's square (step 1) is off by less than 2^-18 M^2.  The separation's direction v is off by 32 u M
+// and, along the axis, by 16 u M^2 / |d| or |d| (u = 2^-24); at the nearest point v is normal to the
+// axis, so the separation times |v| is off by less than `del`.  The margin eta depends on the
+// voxel: the radius lies between the two kept here.
+__device__ __forceinline__ void count_record(CountRecords<true>& cr, int i, float4 A, float4 B, float4, const Range& rg) {
+    const float O[3] = {(float)rg.lo[0], (float)rg.lo[1], (float)rg.lo[2]};
+    const float a[3] = {A.x - O[0], A.y - O[1], A.z - O[2]}, b[3] = {B.x - O[0], B.y - O[1], B.z - O[2]};
+    const float d[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
+    const float r = A.w + capsule_margin(A.w), rr = r * r;
+    const float M = (fmax3(abs_max3(a[0], a[1], a[2]), abs_max3(b[0], b[1], b[2]),
+                           (float)max(max(rg.n[0], rg.n[1]), rg.n[2])) + r) + 3.0f;
+    const float dd = (d[0] * d[0] + d[1] * d[1]) + d[2] * d[2], len = sqrtf(dd), u = 0x1p-24f;
+    const float idd = dd > 0.0f ? 1.0f / dd : 0.0f;
+    const float off = 32.0f * u * M + fminf(len, 16.0f * u * M * M * (len * idd));
+    // (a length whose square is denormal, or coordinates beyond any grid: every voxel is open)
+    const bool sound = M < 1e6f && (dd == 0.0f || dd > 1e-30f);
+    const float del = sound ? 64.0f * u * M * M + off * (len + 1.0f) : INFINITY;
+    const float eps = sound ? 0x1p-18f * M * M : INFINITY;
+    const float rlo = r + 2e-5f * (r + 2.9f), rhi = r + 2e-5f * (2.0f * M + r + 3.0f);
+    cr.q[0][i] = make_float4(a[0], a[1], a[2], -idd);
+    cr.q[1][i] = make_float4(d[0], d[1], d[2], del);
+    cr.q[2][i] = make_float4(fminf(a[0], b[0]) - 0.5f, fminf(a[1], b[1]) - 0.5f, fminf(a[2], b[2]) - 0.5f, rr - eps);
+    cr.q[3][i] = make_float4(fmaxf(a[0], b[0]) + 0.5f, fmaxf(a[1], b[1]) + 0.5f, fmaxf(a[2], b[2]) + 0.5f, rr + eps);
+    cr.q[4][i] = make_float4(rlo * rlo * (1.0f - 0x1p-20f), rhi * rhi * (1.0f + 0x1p-20f), 0.0f, 0.0f);
+}
+// Voxel centre (cx, cy, cz) relative to the range's corner: 1 in, -1 out, 0 open.
+__device__ __forceinline__ int count_quick(const CountRecords<true>& cr, int i, float cx, float cy, float cz) {
+    const float4 a = cr.q[0][i], d = cr.q[1][i], mn = cr.q[2][i], mx = cr.q[3][i], re = cr.q[4][i];
+    const float gx = gap3(cx, cx, mn.x, mx.x), gy = gap3(cy, cy, mn.y, mx.y), gz = gap3(cz, cz, mn.z, mx.z);
+    const float G = __fmaf_rn(gx, gx, __fmaf_rn(gy, gy, gz * gz));
+    const float Ax = a.x - cx, Ay = a.y - cy, Az = a.z - cz;
+    const float t = __saturatef(a.w * __fmaf_rn(Ax, d.x, __fmaf_rn(Ay, d.y, Az * d.z)));
+    const float vx = __fmaf_rn(t, d.x, Ax), vy = __fmaf_rn(t, d.y, Ay), vz = __fmaf_rn(t, d.z, Az);
+    const float sa = __fmaf_rn(vx, Ax, __fmaf_rn(vy, Ay, vz * Az));
+    const float sb = __fmaf_rn(vx, d.x, __fmaf_rn(vy, d.y, __fmaf_rn(vz, d.z, sa)));
+    const float sep = __fmaf_rn(-0.5f, (fabsf(vx) + fabsf(vy)) + fabsf(vz), fminf(sa, sb));
+    const float vv = __fmaf_rn(vx, vx, __fmaf_rn(vy, vy, vz * vz));
+    const float so = sep - d.w, si = sep + d.w;
+    if (G > mx.w || so * fabsf(so) > re.y * vv) return -1;
+    return G < mn.w && si * fabsf(si) < re.x * vv ? 1 : 0;
+}
+
+// Triangle: on each of the 13 axes the voxel's centre has to lie in an interval; an axis is scaled
+// by the inverse of its rounding bound, 2^-18 M times the axis's 1-norm (both evaluations stay below
+// half of that: the edges and the normal are the same numbers, products and sums of terms below M
+// take at most eight roundings of 2^-24 each).  The smallest distance to an interval's end is then
+// beyond 1 when the voxel is in, below -1 when it is out.
+__device__ __forceinline__ float4 count_axis(float u0, float u1, float p0, float p1, float p2, float rad, float inv) {
+    const float mn = fminf(fminf(p0, p1), p2) - rad, mx = fmaxf(fmaxf(p0, p1), p2) + rad;
+    return inv > 0.0f ? make_float4(u0 * inv, u1 * inv, -mn * inv, (mx - mn) * inv) : make_float4(0.0f, 0.0f, 2.0f, 4.0f);
+}
+__device__ __forceinline__ void count_record(CountRecords<false>& cr, int i, float4 A, float4 B, float4 C, const Range& rg) {
+    const float e = 0.5f + 2e-3f;
+    float v[3][3], f[3][3];
+    tri_local(A, B, C, rg.lo[0], rg.lo[1], rg.lo[2], v, f);
+    float M = (float)max(max(rg.n[0], rg.n[1]), rg.n[2]) + 1.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) M = fmaxf(M, abs_max3(v[k][0], v[k][1], v[k][2]) + 1.0f);
+    bool sound = M < 1e6f;
+    const float bound = 0x1p-18f * M;
+    // an axis without extent never separates; one whose products could be denormal leaves all open
+    auto inverse = [&](float l1) {
+        if (l1 == 0.0f) return 0.0f;
+        sound = sound && l1 > 1e-25f;
+        return 1.0f / (bound * l1);
+    };
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float* q = f[j];
+        float l = fabsf(q[1]) + fabsf(q[2]);
+        cr.q[3 * j][i] = count_axis(-q[2], q[1], q[1] * v[0][2] - q[2] * v[0][1], q[1] * v[1][2] - q[2] * v[1][1],
+                                    q[1] * v[2][2] - q[2] * v[2][1], e * l, inverse(l));
+        l = fabsf(q[0]) + fabsf(q[2]);
+        cr.q[3 * j + 1][i] = count_axis(q[2], -q[0], q[2] * v[0][0] - q[0] * v[0][2], q[2] * v[1][0] - q[0] * v[1][2],
+                                        q[2] * v[2][0] - q[0] * v[2][2], e * l, inverse(l));
+        l = fabsf(q[0]) + fabsf(q[1]);
+        cr.q[3 * j + 2][i] = count_axis(-q[1], q[0], q[0] * v[0][1] - q[1] * v[0][0], q[0] * v[1][1] - q[1] * v[1][0],
+                                        q[0] * v[2][1] - q[1] * v[2][0], e * l, inverse(l));
+    }
+    const float n0 = f[0][1] * f[1][2] - f[0][2] * f[1][1];
+    const float n1 = f[0][2] * f[1][0] - f[0][0] * f[1][2];
+    const float n2 = f[0][0] * f[1][1] - f[0][1] * f[1][0];
+    const float l = (fabsf(n0) + fabsf(n1)) + fabsf(n2), inv = inverse(l);
+    const float p = (n0 * v[0][0] + n1 * v[0][1]) + n2 * v[0][2];
+    // the face axes share one scale; the plane's interval is p -+ e l: its width in the last record
+    const float fi = sound ? 1.0f / bound : 0.0f;
+    float lo[3], wd[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float mn = fminf(fminf(v[0][k], v[1][k]), v[2][k]) - e, mx = fmaxf(fmaxf(v[0][k], v[1][k]), v[2][k]) + e;
+        lo[k] = -mn * fi;
+        wd[k] = (mx - mn) * fi;
+    }
+    cr.q[9][i] = inv > 0.0f ? make_float4(n0 * inv, n1 * inv, n2 * inv, (e * l - p) * inv) : make_float4(0.0f, 0.0f, 0.0f, 2.0f);
+    cr.q[10][i] = make_float4(lo[0], lo[1], lo[2], fi);
+    cr.q[11][i] = make_float4(wd[0], wd[1], wd[2], inv > 0.0f ? 2.0f * e * l * inv : 4.0f);
+    if (!sound) {   // the face terms are zero: nothing is in
+#pragma unroll
+        for (int k = 0; k < 9; ++k) cr.q[k][i] = make_float4(0.0f, 0.0f, 2.0f, 4.0f);
+        cr.q[9][i] = make_float4(0.0f, 0.0f, 0.0f, 2.0f);
+        cr.q[10][i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        cr.q[11][i] = make_float4(0.0f, 0.0f, 0.0f, 4.0f);
+    }
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ int count_quick(const CountRecords<false>& cr, int i, float cx, float cy, float cz) {
+    const float4 F = cr.q[10][i], W = cr.q[11][i], N = cr.q[9][i];
+    float s = __fmaf_rn(cx, F.w, F.x);
+    float m = fminf(s, W.x - s);
+    s = __fmaf_rn(cy, F.w, F.y);
+    m = min3(m, s, W.y - s);
+    s = __fmaf_rn(cz, F.w, F.z);
+    m = min3(m, s, W.z - s);
+    s = __fmaf_rn(cx, N.x, __fmaf_rn(cy, N.y, __fmaf_rn(cz, N.z, N.w)));
+    m = min3(m, s, W.w - s);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {   // families x, y, z of edge j / 3
+        const float4 q = cr.q[j][i];
+        s = __fmaf_rn(j % 3 == 0 ? cy : cx, q.x, __fmaf_rn(j % 3 == 2 ? cy : cz, q.y, q.z));
+        m = min3(m, s, q.w - s);
+    }
+    return m > 1.0f ? 1 : (m < -1.0f ? -1 : 0);
+}
+
+// floor of 0 <= x < 2^22, as a float
+__device__ __forceinline__ float floor_pos(float x) { return __fadd_rd(x, 8388608.0f) - 8388608.0f; }
+
+// Counts of 2^lg consecutive primitives from p0 (fewer at np) by a warp, and their ballots; win(p) is
+// the window of a primitive.
+template <bool FIBER, class Win>
+__device__ __forceinline__ void count_group(CountRecords<FIBER>& cr, uint32_t p0, int lg, uint32_t np,
+                                            const float4* __restrict__ r0, const float4* __restrict__ r1,
+                                            const float4* __restrict__ r2, Win win, uint32_t* __restrict__ counts,
+                                            uint32_t* __restrict__ ballots, uint32_t stride) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t p = p0 + (uint32_t)lane;
+    const int members = (int)min(1u << lg, np - p0);
+    if (lane < members) {
+        float4 a, b, c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const Range rg = prim_range<FIBER>(r0, r1, r2, p, win(p), a, b, c);
+        count_record(cr, lane, a, b, c, rg);
+        const float n0 = (float)rg.n[0], n1 = (float)rg.n[1];
+        cr.r[0][lane] = make_float4(__frcp_rn(n0), n0, __frcp_rn(n1), n1);
+        cr.r[1][lane] = make_float4(__int_as_float(rg.lo[0]), __int_as_float(rg.lo[1]), __int_as_float(rg.lo[2]),
+                                    __int_as_float((int)min(rg.total, (long long)kMaxFastRange + 1)));
+    }
+    __syncwarp();
+    uint32_t mine = 0;
+    for (int i = 0; i < members; ++i) {
+        const float4 rn = cr.r[0][i], rl = cr.r[1][i];
+        const int tot = __float_as_int(rl.w);
+        uint32_t n = 0;
+        if (tot > kMaxFastRange) {
+            float4 a, b, c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const Window W = win(p0 + i);
+            const Range rg = prim_range<FIBER>(r0, r1, r2, p0 + i, W, a, b, c);
+            n = candidates_of<FIBER, false>(p0 + i, a, b, c, rg, W, 0u, nullptr, nullptr, ballots, stride);
+        } else {
+            uint32_t* const pb = ballots && tot <= (int)(32u * stride) ? ballots + (size_t)(p0 + i) * stride : nullptr;
+            for (int i0 = 0; i0 < tot; i0 += 32) {
+                const bool valid = i0 + lane < tot;
+                const float f = (float)(i0 + lane);
+                const float t = floor_pos((f + 0.5f) * rn.x);
+                const float x = __fmaf_rn(-t, rn.y, f), z = floor_pos((t + 0.5f) * rn.z), y = __fmaf_rn(-z, rn.w, t);
+                const int q = count_quick(cr, i, x + 0.5f, y + 0.5f, z + 0.5f);
+                bool hit = valid && q > 0;
+                if (__any_sync(0xffffffffu, valid && q == 0) && valid && q == 0) {
+                    const int vi = __float_as_int(rl.x) + (int)x, vj = __float_as_int(rl.y) + (int)y,
+                              vk = __float_as_int(rl.z) + (int)z;
+                    hit = FIBER ? capsule_voxel_candidate(r0[p0 + i], r1[p0 + i], vi, vj, vk)
+                                : tri_voxel_candidate(r0[p0 + i], r1[p0 + i], r2[p0 + i], vi, vj, vk);
+                }
+                const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+                if (pb && lane == 0) pb[i0 >> 5] = bal;
+                n += __popc(bal);
+            }
+        }
+        if (lane == i) mine = n;
+    }
+    if (lane < members) counts[p] = mine;
+    __syncwarp();
+}
+
+// primitives per warp (log2): 32 where that leaves every SM its warps, fewer for short arrays
+inline int count_lanes_log2(uint32_t np) {
+    int lg = 5;
+    while (lg > 0 && (np >> lg) < (uint32_t)vx::kSMs * 48) --lg;
+    return lg;
+}
+inline unsigned count_blocks(uint32_t np, int lg) {
+    const size_t groups = ((size_t)np + (1u << lg) - 1) >> lg;
+    return (unsigned)std::min<size_t>((groups + COUNT_WARPS - 1) / COUNT_WARPS, (size_t)vx::kSMs * 64);
+}
+
+template <bool FIBER>
+__global__ void __launch_bounds__(COUNT_WARPS * 32, FIBER ? 7 : 5) k_count(const float4* __restrict__ r0, const float4* __restrict__ r1,
+                                                            const float4* __restrict__ r2, uint32_t np, Window R, int lg,
+                                                            uint32_t* __restrict__ counts, uint32_t* __restrict__ ballots,
+                                                            uint32_t stride) {
+    __shared__ CountRecords<FIBER> rec[COUNT_WARPS];
+    const uint32_t groups = (uint32_t)(((uint64_t)np + (1u << lg) - 1) >> lg);
+    for (uint32_t g = blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); g < groups; g += gridDim.x * COUNT_WARPS)
+        count_group<FIBER>(rec[threadIdx.x >> 5], g << lg, lg, np, r0, r1, r2, [&](uint32_t) { return R; }, counts, ballots,
+                           stride);
+}
+
 // Emit from the stored ballots.  A warp takes 32 consecutive primitives; their pairs are consecutive
 // in the output, so it walks their words 32 at a time, a lane per word: the lane writes the pairs
 // of its word's bits to the warp's staging buffer, which then goes out in order with whole lines.
@@ -1156,22 +1389,20 @@ __global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* 
     }
 }
 
-template <bool FIBER, bool EMIT>
+// emit of a pass without stored ballots: a warp per primitive tests its range again
+template <bool FIBER>
 __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __restrict__ r0,
                                                                 const float4* __restrict__ r1,
                                                                 const float4* __restrict__ r2, uint32_t np, Window R,
-                                                                uint32_t* __restrict__ counts,
                                                                 const uint32_t* __restrict__ offs,
                                                                 uint32_t* __restrict__ keys,
                                                                 uint32_t* __restrict__ vals,
                                                                 uint32_t* __restrict__ ballots, uint32_t stride) {
-    const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * EMIT_WARPS;
     for (uint32_t p = blockIdx.x * EMIT_WARPS + (threadIdx.x >> 5); p < np; p += warps) {
         float4 a, b, c;
         const Range rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
-        const uint32_t n = candidates_of<FIBER, EMIT>(p, a, b, c, rg, R, EMIT ? offs[p] : 0u, keys, vals, ballots, stride);
-        if (!EMIT && lane == 0) counts[p] = n;
+        candidates_of<FIBER, true>(p, a, b, c, rg, R, offs[p], keys, vals, ballots, stride);
     }
 }
 

@@ -76,13 +76,13 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
         ctx->ballots_win[i] = win.lo[i];
         ctx->ballots_win[3 + i] = win.hi[i];
     }
-    const unsigned cblocks = (unsigned)std::min<size_t>((np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
+    const int lg = count_lanes_log2(np);
     if (fiber)
-        VX_LAUNCH(ctx, ST_COUNT, s, k_candidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots, stride));
+        VX_LAUNCH(ctx, ST_COUNT, s, k_count<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
+                                        r0, r1, r2, np, win, lg, cnt, ballots, stride));
     else
-        VX_LAUNCH(ctx, ST_COUNT, s, k_candidates<false, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, cnt, nullptr, nullptr, nullptr, ballots, stride));
+        VX_LAUNCH(ctx, ST_COUNT, s, k_count<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
+                                        r0, r1, r2, np, win, lg, cnt, ballots, stride));
     unsigned long long* t64 = (unsigned long long*)(misc + 8);
     bool done = false;
     VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s, t64, vx_pin_of(ctx, misc, 12), &done));
@@ -151,11 +151,11 @@ vx_status window_segments(vx_context* ctx, bool fiber, uint32_t np, const Window
             VX_LAUNCH(ctx, ST_EMIT, s, k_emit_stored<false><<<eblocks, STAGE_WARPS * 32, 0, s>>>(
                                            r0, r1, r2, np, win, offs, *k0, *v0, ctx->ballots, ctx->ballots_stride));
     } else if (fiber) {
-        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<true, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, nullptr, 0u));
+        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
+                                       r0, r1, r2, np, win, offs, *k0, *v0, nullptr, 0u));
     } else {
-        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<false, true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, nullptr, offs, *k0, *v0, nullptr, 0u));
+        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
+                                       r0, r1, r2, np, win, offs, *k0, *v0, nullptr, 0u));
     }
     VX_CUDA_TRY(cudaGetLastError());
     VX_TRY(vx_radix_sort_u32(ctx, k0, v0, k1, v1, npairs, 3 * bits, s, misc));
@@ -1572,9 +1572,9 @@ extern "C" vx_status vx_backward_noalloc(const vx_primitives* prims, const vx_gr
     NA_TRY(vx_scan_u32_scratch(fs, fs, (uint32_t)F, misc + 4, part, s));
     k_prep_fibers<<<grid_for(np, 256), 256, 0, s>>>((const float4*)prims->ctrl, prims->num_ctrl, prims->fiber_offsets, fs, F, misc + 4,
                                                      prims->weights, np, g, r0, r1, misc);
-    const unsigned cblocks = (unsigned)std::min<size_t>((np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
-    k_candidates<true, false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(r0, r1, nullptr, np, full_window((int)R), cnt,
-                                                                  nullptr, nullptr, nullptr, nullptr, 0u);
+    const int clg = count_lanes_log2(np);
+    k_count<true><<<count_blocks(np, clg), COUNT_WARPS * 32, 0, s>>>(r0, r1, nullptr, np, full_window((int)R), clg, cnt,
+                                                                     nullptr, 0u);
     // the exact 64-bit total
     k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
         cnt, np, (unsigned long long*)(misc + 8));

@@ -202,3 +202,26 @@ def test_pair_sort_at_the_tile_edges(n, R):
     ctx = vx.Context(DEV)
     _same_level0(ctx.voxelize(grid, tri_verts=torch.from_numpy(tris).to(DEV)), oracle.voxelize(w))
     ctx.close()
+
+
+@pytest.mark.parametrize("kind,n,R", [("tri", 1, 4), ("tri", 14593, 16), ("tri", 29185, 32), ("cap", 1, 4), ("cap", 2, 64),
+                                      ("cap", 14595, 32), ("cap", 29190, 16)])
+def test_candidates_of_groups(kind, n, R):
+    """The count pass takes 1, 2 or 4 primitives per warp at these lengths (the last group is short), and
+    two capsules whose ranges hold more than 65,536 voxels: every level-0 value against the oracle."""
+    if kind == "tri":
+        tris, grid = synth.random_triangles(n, R, seed=n, size=(0.05, 1.2))
+        tris[::7, 2, :3] = tris[::7, 0, :3]                       # without area
+        w = synth.Workload("count", "triangles", grid, tri_verts=tris, K=1)
+        geom = dict(tri_verts=torch.from_numpy(tris).to(DEV))
+    else:
+        if n == 2:
+            ctrl = np.array([[0.1, 0.1, 0.1, 0.05], [0.9, 0.85, 0.8, 0.05], [0.2, 0.9, 0.15, 0.02]], np.float32)
+            off, grid = np.array([0, 3], np.int64), synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+        else:
+            ctrl, off, grid = synth.random_segments(max(n // 139, 1), min(n, 139) + 1, R, seed=n, radius=(0.05, 0.8))
+        w = synth.Workload("count", "fibers", grid, ctrl=ctrl, fiber_offsets=off, K=1)
+        geom = dict(ctrl=torch.from_numpy(ctrl).to(DEV), fiber_offsets=torch.from_numpy(off).to(DEV))
+    ctx = vx.Context(DEV)
+    _same_level0(ctx.voxelize(grid, **geom), oracle.voxelize(w))
+    ctx.close()
