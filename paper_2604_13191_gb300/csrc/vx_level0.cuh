@@ -1861,45 +1861,112 @@ __device__ __forceinline__ void write_lobe(float m, const float* M, float* lobe,
     }
 }
 
-__global__ void k_finalize(SegOut in, const uint32_t* __restrict__ nseg_p, const uint32_t* __restrict__ dst,
-                           vx_level L, uint64_t key_hi) {
-    const uint32_t nseg = *nseg_p;
-    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < nseg; s += gridDim.x * blockDim.x) {
-        if (!in.nonzero[s]) continue;
-        const uint32_t o = dst[s];
-        L.keys[o] = key_hi | (uint64_t)in.key[s];
-        // 16-byte mask and 8-byte moment accesses (mask rows are 64-byte aligned, moment
-        // rows 8-byte aligned in both the temporaries and the level block)
-        uint64_t m[8];
-        const uint4* mi = reinterpret_cast<const uint4*>(in.mask + (size_t)s * 8);
-        uint4* mo = reinterpret_cast<uint4*>(L.mask + (size_t)o * 8);
+// Bound by memory: 130 bytes read and 152 written per voxel.  A warp takes 32 consecutive segments; the rows it
+// keeps are consecutive in the level, so the masks, moments and lobes go through shared memory,
+// compacted, and are read and written with whole lines.  (A lane copying its own 64-, 24- and
+// 28-byte rows waited for the many partly used lines: mesh 0.52 ms, woven 0.53 and yarn 0.34 ms
+// against 0.31, 0.35 and 0.23 ms, 6 TB/s; eight or six blocks per SM 2 and 7 % more.)
+constexpr int FIN_WARPS = 4;
+__global__ void __launch_bounds__(FIN_WARPS * 32, 7) k_finalize(SegOut in, const uint32_t* __restrict__ nseg_p,
+                                                             const uint32_t* __restrict__ dst, vx_level L,
+                                                             uint64_t key_hi) {
+    struct Rows {
+        uint4 mask[32 * 5];        // four 16-byte pieces per row and one of padding
+        float2 moment[32 * 3];
+        float lobes[32 * 7], compact[32 * 6];
+    };
+    __shared__ Rows rows[FIN_WARPS];
+    Rows& W = rows[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const uint32_t nseg = *nseg_p, warps = gridDim.x * FIN_WARPS;
+    for (uint32_t s0 = (blockIdx.x * FIN_WARPS + (threadIdx.x >> 5)) * 32u; s0 < nseg; s0 += warps * 32u) {
+        const uint32_t s = s0 + (uint32_t)lane, n = min(32u, nseg - s0);
+        const bool keep = s < nseg && in.nonzero[s];
+        const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+        if (!kept) continue;
+        const uint32_t count = (uint32_t)__popc(kept), below = (1u << lane) - 1u;
+        const size_t o0 = dst[s0 + (uint32_t)__ffs(kept) - 1u];   // (the same word for the whole warp)
+        const uint32_t rank = (uint32_t)__popc(kept & below);
+        const uint4* const mi = reinterpret_cast<const uint4*>(in.mask + (size_t)s0 * 8);
+        const float2* const Mi = reinterpret_cast<const float2*>(in.moment + (size_t)s0 * 6);
+        uint4 mp[4];
+        float2 Mp[3];
+        bool mk[4], Mk[3];
+        uint32_t mr[4], Mr[3];
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const uint4 q = mi[w];
-            mo[w] = q;
-            m[2 * w] = ((uint64_t)q.y << 32) | q.x;
-            m[2 * w + 1] = ((uint64_t)q.w << 32) | q.z;
+        for (int q = 0; q < 4; ++q) {   // (a row that is not kept is not read)
+            const uint32_t i = q * 32 + lane, r = i >> 2;
+            mk[q] = r < n && ((kept >> r) & 1u);
+            mr[q] = (uint32_t)__popc(kept & ((1u << r) - 1u)) * 5 + (i & 3);
+            if (mk[q]) mp[q] = mi[i];
         }
-        float mass = in.mass[s];
-        float M[6];
-        const float2* Mi = reinterpret_cast<const float2*>(in.moment + (size_t)s * 6);
-        float2* Mo = reinterpret_cast<float2*>(L.moment + (size_t)o * 6);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float2 q = Mi[c];
-            Mo[c] = q;
-            M[2 * c] = q.x;
-            M[2 * c + 1] = q.y;
+        for (int q = 0; q < 3; ++q) {
+            const uint32_t i = q * 32 + lane, r = i / 3;
+            Mk[q] = r < n && ((kept >> r) & 1u);
+            Mr[q] = (uint32_t)__popc(kept & ((1u << r) - 1u)) * 3 + (i - 3 * r);
+            if (Mk[q]) Mp[q] = Mi[i];
         }
-        L.mass[o] = mass;
-        uint16_t occ;
-        uint8_t pj[3];
-        mask_counts(m, occ, pj);
-        L.occ[o] = occ;
-        L.occ_proj[(size_t)o * 3 + 0] = pj[0];
-        L.occ_proj[(size_t)o * 3 + 1] = pj[1];
-        L.occ_proj[(size_t)o * 3 + 2] = pj[2];
-        write_lobe(mass, M, L.lobes + (size_t)o * 7, L.compact + (size_t)o * 6, L.lobe_count + o);
+        const float mass = keep ? in.mass[s] : 0.0f;
+        const uint32_t key = keep ? in.key[s] : 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (mk[q]) W.mask[mr[q]] = mp[q];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (Mk[q]) W.moment[Mr[q]] = Mp[q];
+        __syncwarp();
+        if (keep) {
+            const size_t o = o0 + rank;
+            uint64_t m[8];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const uint4 q = W.mask[rank * 5 + w];
+                m[2 * w] = ((uint64_t)q.y << 32) | q.x;
+                m[2 * w + 1] = ((uint64_t)q.w << 32) | q.z;
+            }
+            float M[6];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float2 q = W.moment[rank * 3 + c];
+                M[2 * c] = q.x;
+                M[2 * c + 1] = q.y;
+            }
+            uint16_t occ;
+            uint8_t pj[3];
+            mask_counts(m, occ, pj);
+            L.keys[o] = key_hi | (uint64_t)key;
+            L.mass[o] = mass;
+            L.occ[o] = occ;
+            L.occ_proj[o * 3 + 0] = pj[0];
+            L.occ_proj[o * 3 + 1] = pj[1];
+            L.occ_proj[o * 3 + 2] = pj[2];
+            write_lobe(mass, M, W.lobes + rank * 7, W.compact + rank * 6, L.lobe_count + o);
+        }
+        __syncwarp();
+        uint4* const mo = reinterpret_cast<uint4*>(L.mask + o0 * 8);
+        float2* const Mo = reinterpret_cast<float2*>(L.moment + o0 * 6);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t i = q * 32 + lane;
+            if (i < count * 4) mo[i] = W.mask[(i >> 2) * 5 + (i & 3)];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const uint32_t i = q * 32 + lane;
+            if (i < count * 3) Mo[i] = W.moment[i];
+        }
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            const uint32_t i = q * 32 + lane;
+            if (i < count * 7) L.lobes[o0 * 7 + i] = W.lobes[i];
+        }
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const uint32_t i = q * 32 + lane;
+            if (i < count * 6) L.compact[o0 * 6 + i] = W.compact[i];
+        }
+        __syncwarp();
     }
 }
 

@@ -222,7 +222,7 @@ vx_status window_reduce(vx_context* ctx, bool fiber, uint32_t np, uint32_t nseg,
         view = *alloc_out;
     }
     if (nvox > 0) {
-        VX_LAUNCH(ctx, ST_FINALIZE, s, k_finalize<<<grid_for(nseg, 256), 256, 0, s>>>(seg, misc + 2, flags, view, key_hi));
+        VX_LAUNCH(ctx, ST_FINALIZE, s, k_finalize<<<grid_for(nseg, FIN_WARPS * 32), FIN_WARPS * 32, 0, s>>>(seg, misc + 2, flags, view, key_hi));
         VX_CUDA_TRY(cudaGetLastError());
     }
     return VX_OK;
