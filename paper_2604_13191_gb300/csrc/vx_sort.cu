@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(SORT_THREADS) k_radix_hist(const uint32_t* __r
                                                              const uint32_t* __restrict__ vals, uint32_t n,
                                                              int shift, uint32_t dmask, uint32_t nt,
                                                              const uint8_t* __restrict__ lut,
-                                                             uint32_t* __restrict__ hist) {
+                                                             uint32_t* __restrict__ hist, bool by_tile = false) {
     __shared__ uint32_t h[RB];
     for (int d = threadIdx.x; d < RB; d += SORT_THREADS) h[d] = 0;
     __syncthreads();
@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(SORT_THREADS) k_radix_hist(const uint32_t* __r
         }
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < RB; d += SORT_THREADS) hist[(size_t)d * nt + blockIdx.x] = h[d];
+    for (int d = threadIdx.x; d < RB; d += SORT_THREADS)
+        hist[by_tile ? (size_t)blockIdx.x * RB + d : (size_t)d * nt + blockIdx.x] = h[d];
 }
 
 // The lanes whose BITS-bit digit equals this lane's, among those with `valid`: one ballot per bit,
@@ -505,6 +506,7 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  : "memory");
 }
 
+constexpr uint32_t FOLD_TILES = 32;   // see sort_pass
 constexpr size_t pipe_smem(int rb) {
     return (size_t)2 * 2 * SORT_TILE * 4                 // two stages of keys + values
            + (size_t)SORT_WARPS * rb * 2                 // per-warp digit counters
@@ -519,7 +521,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
                                                                       const uint32_t* __restrict__ hist,
                                                                       uint32_t* __restrict__ okeys,
                                                                       uint32_t* __restrict__ ovals,
-                                                                      uint32_t* __restrict__ err) {
+                                                                      uint32_t* __restrict__ err, bool fold) {
     static_assert((RB == 256 || RB == 512) && RB % SORT_THREADS == 0, "digit widths");
     constexpr int BITS = RB == 512 ? 9 : 8;
     extern __shared__ __align__(128) unsigned char sm_raw[];
@@ -556,9 +558,34 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
     // digit-major histogram puts a tile's offsets a stride nt apart)
     constexpr int DPT = RB / SORT_THREADS;   // digits per thread
     uint32_t gcur[DPT];
+    if (fold) {
+        // the tile counts themselves, tile by tile: a digit's offset is all smaller digits' items and
+        // those of its own in earlier tiles
+        uint32_t tot[DPT] = {}, pre[DPT] = {}, sum = 0;
+#pragma unroll 8
+        for (uint32_t q = 0; q < nt; ++q)
 #pragma unroll
-    for (int i = 0; i < DPT; ++i)
-        gcur[i] = blockIdx.x < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + blockIdx.x] : 0u;
+            for (int i = 0; i < DPT; ++i) {
+                const uint32_t c = hist[(size_t)q * RB + threadIdx.x * DPT + i];
+                tot[i] += c;
+                if (q < blockIdx.x) pre[i] += c;
+            }
+#pragma unroll
+        for (int i = 0; i < DPT; ++i) sum += tot[i];
+        const uint32_t inc = warp_incl_scan(sum);
+        if (lane == 31) scan_tmp[w] = inc;
+        __syncthreads();
+        uint32_t ex = __reduce_add_sync(0xffffffffu, lane < w ? scan_tmp[lane] : 0u) + inc - sum;
+#pragma unroll
+        for (int i = 0; i < DPT; ++i) {
+            gcur[i] = ex + pre[i];
+            ex += tot[i];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < DPT; ++i)
+            gcur[i] = blockIdx.x < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + blockIdx.x] : 0u;
+    }
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x, st ^= 1) {
         // the next tile streams into the other stage (its last reader finished: the loop ends
         // with a barrier); generic writes to that stage are ordered before the async copy
@@ -573,7 +600,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_radix_scatter_pipe(const ui
         uint32_t gnxt[DPT];
 #pragma unroll
         for (int i = 0; i < DPT; ++i)
-            gnxt[i] = tn < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + tn] : 0u;
+            gnxt[i] = !fold && tn < nt ? hist[(size_t)(threadIdx.x * DPT + i) * nt + tn] : 0u;
         const size_t tile0 = (size_t)t * SORT_TILE;
         const uint32_t tn_items = (uint32_t)min((size_t)SORT_TILE, (size_t)n - tile0);
         uint32_t* const sk = stage0 + (size_t)st * 2 * SORT_TILE;
@@ -784,11 +811,16 @@ vx_status sort_pass(vx_context* ctx, uint32_t** keys, uint32_t** vals, uint32_t*
         attr_set = true;
     }
     const unsigned sblocks = (unsigned)std::min<uint32_t>(nt, (uint32_t)vx::kSMs * 2);
+    // few tiles: a block each, which sums the tiles' counts itself (1.5 us), where the scan is one more
+    // launch of 5 us on the chain.  Every block reads all nt counts of every digit, so the rule stops
+    // at 32 tiles.
+    const bool fold = nt <= FOLD_TILES;
+    static_assert(FOLD_TILES <= vx::kSMs * 2, "a block per tile");
     VX_LAUNCH(ctx, ST_SORT_HIST, s, (k_radix_hist<false, RB><<<nt, SORT_THREADS, 0, s>>>(
-                                        *keys, *vals, n, shift, dmask, nt, nullptr, hist)));
-    VX_TRY(vx_scan_u32(ctx, hist, hist, (uint32_t)((size_t)RB * nt), nullptr, s));
+                                        *keys, *vals, n, shift, dmask, nt, nullptr, hist, fold)));
+    if (!fold) VX_TRY(vx_scan_u32(ctx, hist, hist, (uint32_t)((size_t)RB * nt), nullptr, s));
     VX_LAUNCH(ctx, ST_SORT_SCATTER, s, (k_radix_scatter_pipe<RB><<<sblocks, SORT_THREADS, pipe_smem(RB), s>>>(
-                                           *keys, *vals, n, shift, dmask, nt, hist, *keys_alt, *vals_alt, err)));
+                                           *keys, *vals, n, shift, dmask, nt, hist, *keys_alt, *vals_alt, err, fold)));
     VX_CUDA_TRY(cudaGetLastError());
     uint32_t* t = *keys; *keys = *keys_alt; *keys_alt = t;
     t = *vals; *vals = *vals_alt; *vals_alt = t;

@@ -225,3 +225,24 @@ def test_candidates_of_groups(kind, n, R):
     ctx = vx.Context(DEV)
     _same_level0(ctx.voxelize(grid, **geom), oracle.voxelize(w))
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [131072, 131073])
+def test_pair_sort_with_and_without_its_own_offsets(n):
+    """32 tiles (each block sums the tile counts itself) and 33 (a scan does): the level equals, bit
+    for bit, the one whose pairs are sorted window by window in shorter pieces."""
+    R = 64
+    rng = np.random.default_rng(n)
+    v = (rng.integers(0, R, (n, 1, 3)) + rng.uniform(0.3, 0.7, (n, 3, 3))) / R
+    tris = np.zeros((n, 3, 4), np.float32)
+    tris[..., :3] = v
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    geom = torch.from_numpy(tris).to(DEV)
+    ctx = vx.Context(DEV)
+    whole = ctx.voxelize(grid, tri_verts=geom).host()
+    ctx.set_max_pairs_per_pass(n // 3)
+    parts = ctx.voxelize(grid, tri_verts=geom).host()
+    assert whole["occ"].shape[0] > 90000 and np.all(np.diff(whole["keys"].astype(np.int64)) > 0)
+    for f in ("keys", "mask", "mass", "moment", "occ", "proj", "lobes"):
+        assert np.array_equal(np.asarray(whole[f]).view(np.uint8), np.asarray(parts[f]).view(np.uint8)), f
+    ctx.close()
