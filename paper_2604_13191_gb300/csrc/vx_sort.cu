@@ -50,26 +50,56 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* smem, 
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const uint32_t* __restrict__ in,
-                                                              uint32_t n, uint32_t* __restrict__ part) {
+                                                              uint32_t n, uint32_t* __restrict__ part,
+                                                              unsigned long long* __restrict__ part64 = nullptr) {
     __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
+    __shared__ unsigned long long sm64[SCAN_THREADS / 32];
     const size_t base = (size_t)blockIdx.x * SCAN_TILE;
     uint32_t s = 0;
+    unsigned long long s64 = 0;
 #pragma unroll
     for (int j = 0; j < SCAN_ITEMS; ++j) {
         size_t e = base + (size_t)j * SCAN_THREADS + threadIdx.x;
-        if (e < n) s += in[e];
+        const uint32_t v = e < n ? in[e] : 0u;
+        s += v;
+        s64 += v;
+    }
+    if (part64) {   // the block's exact sum
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s64 += __shfl_xor_sync(0xffffffffu, s64, o);
+        if ((threadIdx.x & 31) == 0) sm64[threadIdx.x >> 5] = s64;
     }
     uint32_t tot;
     block_excl_scan(s, sm, tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = tot;
+        if (part64) {
+            unsigned long long t = 0;
+            for (int k = 0; k < SCAN_THREADS / 32; ++k) t += sm64[k];
+            part64[blockIdx.x] = t;
+        }
+    }
 }
 
 // Single-block exclusive scan of the block partials (any length); zero: two words cleared for the
-// caller (or NULL).
+// caller (or NULL); part64, total64: the blocks' exact sums and theirs (or NULL); pin: words copied
+// to the host's buffer once the totals are written (a launch of their own, 3 us, else).
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(uint32_t* part, uint32_t nb,
-                                                                uint32_t* total, uint32_t* zero = nullptr) {
+                                                                uint32_t* total, uint32_t* zero = nullptr,
+                                                                const unsigned long long* part64 = nullptr,
+                                                                unsigned long long* total64 = nullptr,
+                                                                vx_pin_copy pin = vx_pin_copy{}) {
     __shared__ uint32_t sm[SCAN_THREADS / 32 + 1];
+    __shared__ unsigned long long sm64[SCAN_THREADS / 32];
     uint32_t carry = 0;
+    unsigned long long s64 = 0;
+    if (total64) {
+        for (uint32_t b = threadIdx.x; b < nb; b += SCAN_THREADS) s64 += part64[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s64 += __shfl_xor_sync(0xffffffffu, s64, o);
+        if ((threadIdx.x & 31) == 0) sm64[threadIdx.x >> 5] = s64;
+        __syncthreads();
+    }
     if (zero && threadIdx.x < 2) zero[threadIdx.x] = 0u;
     for (uint32_t b = 0; b < nb; b += SCAN_TILE) {
         uint32_t v[SCAN_ITEMS];
@@ -91,7 +121,15 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(uint32_t* part, 
         }
         carry += tot;
     }
-    if (threadIdx.x == 0 && total) *total = carry;
+    if (threadIdx.x == 0) {
+        if (total) *total = carry;
+        if (total64) {
+            unsigned long long t = 0;
+            for (int k = 0; k < SCAN_THREADS / 32; ++k) t += sm64[k];
+            *total64 = t;
+        }
+        vx_pin_words(pin);
+    }
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const uint32_t* in, uint32_t* out, uint32_t n,
@@ -728,8 +766,10 @@ vx_status vx_scan_u32(vx_context* ctx, const uint32_t* in, uint32_t* out, uint32
     uint32_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (nb == 0) nb = 1;
     if (done) *done = false;
-    VX_TRY(vx_ws_ensure(ctx, WS_SCAN_TMP, (size_t)nb * 4 + 256, s));
+    const size_t at64 = ((size_t)nb * 4 + 255) & ~(size_t)255;   // the exact sums behind the partials
+    VX_TRY(vx_ws_ensure(ctx, WS_SCAN_TMP, at64 + (total64 ? (size_t)nb * 8 : 0) + 256, s));
     uint32_t* part = (uint32_t*)ctx->ws[WS_SCAN_TMP].p;
+    unsigned long long* part64 = total64 ? (unsigned long long*)((char*)part + at64) : nullptr;
     if (n == 0) {
         if (total) VX_CUDA_TRY(cudaMemsetAsync(total, 0, 4, s));
         return VX_OK;
@@ -740,10 +780,11 @@ vx_status vx_scan_u32(vx_context* ctx, const uint32_t* in, uint32_t* out, uint32
         if (done) *done = true;
         return VX_OK;
     }
-    VX_LAUNCH(ctx, ST_SCAN, s, k_scan_reduce<<<nb, SCAN_THREADS, 0, s>>>(in, n, part));
-    VX_LAUNCH(ctx, ST_SCAN, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, total));
+    VX_LAUNCH(ctx, ST_SCAN, s, k_scan_reduce<<<nb, SCAN_THREADS, 0, s>>>(in, n, part, part64));
+    VX_LAUNCH(ctx, ST_SCAN, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, total, nullptr, part64, total64, pin));
     VX_LAUNCH(ctx, ST_SCAN, s, k_scan_down<<<nb, SCAN_THREADS, 0, s>>>(in, out, n, part));
     VX_CUDA_TRY(cudaGetLastError());
+    if (done) *done = true;
     return VX_OK;
 }
 
@@ -770,9 +811,10 @@ vx_status segment_starts(vx_context* ctx, int stage, const T* keys, uint32_t n, 
     }
     uint32_t* const total = nseg ? nseg : part + nb;
     VX_LAUNCH(ctx, stage, s, (k_seg_count<T><<<nb, SCAN_THREADS, 0, s>>>(keys, n, shift, wide, part)));
-    VX_LAUNCH(ctx, stage, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, total, zero));
+    VX_LAUNCH(ctx, stage, s, k_scan_partials<<<1, SCAN_THREADS, 0, s>>>(part, nb, total, zero, nullptr, nullptr, pin));
     VX_LAUNCH(ctx, stage, s, (k_seg_starts<T><<<nb, SCAN_THREADS, 0, s>>>(keys, n, shift, wide, part, total, starts)));
     VX_CUDA_TRY(cudaGetLastError());
+    if (done) *done = true;
     return VX_OK;
 }
 }  // namespace

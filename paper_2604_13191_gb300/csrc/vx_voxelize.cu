@@ -86,10 +86,8 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
     unsigned long long* t64 = (unsigned long long*)(misc + 8);
     bool done = false;
     VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s, t64, vx_pin_of(ctx, misc, 12), &done));
-    if (!done) {
+    if (!done) {   // no primitives
         VX_CUDA_TRY(cudaMemsetAsync(t64, 0, 8, s));
-        VX_LAUNCH(ctx, ST_COUNT, s, k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
-                                        cnt, np, t64));
         VX_TRY(vx_readback_async(ctx, 0, misc, 48, s));
     }
     VX_CUDA_TRY(cudaStreamSynchronize(s));
