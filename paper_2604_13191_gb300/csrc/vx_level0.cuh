@@ -590,7 +590,7 @@ __device__ __forceinline__ uint32_t interval_bits(float a, float b, float delta,
 // are marked in `open`.
 __device__ __forceinline__ void family_rows(const EdgeAxis ax[3], float delta, uint32_t& lo, uint32_t& hi, uint32_t& open) {
     lo = hi = open = 0;
-#pragma unroll 2
+#pragma unroll 1
     for (int i1 = 0; i1 < 8; ++i1) {
         const float y = (float)i1;
         float l[3], h[3], near[3];
@@ -616,6 +616,9 @@ __device__ __forceinline__ void family_rows(const EdgeAxis ax[3], float delta, u
 // local vertices and edges of (A, B, C) in voxel (vi, vj, vk).  One lane per pair: an axis decides a
 // whole row of sub-cells as an interval, about 70 dispatch slots for 28 triangles at once, where
 // the warp testing sub-cells one triangle at a time took about 200 for every triangle.
+// Kept short: the reduce's warps walk different parts of a long kernel, and waiting for instructions
+// was their first stall.  One body for the three families, rows one at a time, and the clip and sum
+// loops not unrolled took the mesh's reduce from 8.87 to 7.54 ms.
 constexpr int TRI_MASK = 68;   // bytes from one pair's mask to the next (17 words: no bank conflict)
 __device__ __forceinline__ void tri_mask(const float v[3][3], const float f[3][3], float4 A, float4 B, float4 C, int vi,
                                          int vj, int vk, uint8_t* __restrict__ out) {
@@ -638,23 +641,30 @@ __device__ __forceinline__ void tri_mask(const float v[3][3], const float f[3][3
     }
     // the pairs (i0 + 8 i1) that pass the edge axes of families 0 (y, z), 1 (x, z), 2 (x, y)
     uint32_t fam[6];
-#pragma unroll
+#pragma unroll 1
     for (int fa = 0; fa < 3; ++fa) {
-        const int a0 = fa == 0 ? 1 : 0, a1 = fa == 2 ? 1 : 2;   // the family's coordinates (i0, i1)
+        // the family's coordinates (i0, i1): (y, z), (x, z), (x, y)
+        float x0[3], x1[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x0[k] = fa == 0 ? x[1][k] : x[0][k];
+            x1[k] = fa == 2 ? x[1][k] : x[2][k];
+        }
+        const float V0 = fa == 0 ? V[1] : V[0], V1 = fa == 2 ? V[1] : V[2];
         EdgeAxis ax[3];
         float delta = 0.0f;
         bool fit = true;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             // p_k = s0 (v_a0 - c0) + s1 (v_a1 - c1), as family_pass
-            const float s0 = fa == 1 ? f[j][2] : -f[j][fa == 0 ? 2 : 1];
-            const float s1 = fa == 1 ? -f[j][0] : f[j][fa == 0 ? 1 : 0];
-            ax[j] = edge_axis(x[a0], x[a1], V[a0], V[a1], s0, s1, delta, fit);
+            const float s0 = fa == 1 ? f[j][2] : (fa == 0 ? -f[j][2] : -f[j][1]);
+            const float s1 = fa == 1 ? -f[j][0] : (fa == 0 ? f[j][1] : f[j][0]);
+            ax[j] = edge_axis(x0, x1, V0, V1, s0, s1, delta, fit);
         }
         uint32_t lo, hi, open;
         family_rows(ax, delta, lo, hi, open);
         if (!fit) open = 0xffu;
-        open &= box[a1];   // (rows outside the box need no decision)
+        open &= fa == 2 ? box[1] : box[2];   // (rows outside the box need no decision)
         while (open) {
             const int i1 = __ffs(open) - 1;
             open &= open - 1;
@@ -665,8 +675,10 @@ __device__ __forceinline__ void tri_mask(const float v[3][3], const float f[3][3
             if (i1 < 4) lo = (lo & ~(0xffu << sh)) | (bits << sh);
             else hi = (hi & ~(0xffu << sh)) | (bits << sh);
         }
-        fam[2 * fa] = lo;
-        fam[2 * fa + 1] = hi;
+        // (constant indices: fam stays in registers)
+        if (fa == 0) { fam[0] = lo; fam[1] = hi; }
+        else if (fa == 1) { fam[2] = lo; fam[3] = hi; }
+        else { fam[4] = lo; fam[5] = hi; }
     }
     // the box axes: y columns and z rows of family 0, x columns of family 1
     const uint32_t ycols = box[1] * 0x01010101u, xcols = box[0] * 0x01010101u;
@@ -745,6 +757,7 @@ __device__ __forceinline__ int clip_plane_s(float* __restrict__ buf, int pi, int
     auto at = [&](int poly, int v, int j) -> float& { return buf[((poly * 12 + v) * 3 + j) * 32 + t]; };
     int m = 0, v = off;
     float S[3] = {at(pi, off, 0), at(pi, off, 1), at(pi, off, 2)};
+#pragma unroll 1
     for (int k = 0; k < n; ++k) {
         v = v + 1 == n ? 0 : v + 1;
         const float E[3] = {at(pi, v, 0), at(pi, v, 1), at(pi, v, 2)};
@@ -807,6 +820,7 @@ __device__ float tri_measure(const float v[3][3], float* __restrict__ buf) {
     const float a0 = at(cur, off, 0), a1 = at(cur, off, 1), a2 = at(cur, off, 2);
     int w = vertex(1);
     float e1[3] = {at(cur, w, 0) - a0, at(cur, w, 1) - a1, at(cur, w, 2) - a2};
+#pragma unroll 1
     for (int k = 1; k + 1 < n; ++k) {
         w = vertex(k + 1);
         const float e2[3] = {at(cur, w, 0) - a0, at(cur, w, 1) - a1, at(cur, w, 2) - a2};
@@ -1692,8 +1706,9 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint3
 // moment terms and its 512-bit mask, so that a mesh's few triangles per voxel fill the lanes.  Then
 // each voxel's masks are ORed, lane L on bits 16 L .. 16 L + 15.  A voxel of more than 32 triangles
 // is a group of its own and runs in batches of 32.
-// Bound by dispatch (DRAM idle).  2.09 M triangles at 1024^3, 28.5 M pairs, 3.9 per voxel: 8.9 ms, of
-// which the areas take 2.4, the edge axes 2.7 and the face normal 2.4 (45.9 ms with a voxel's
+// Bound by dispatch (DRAM idle).  2.09 M triangles at 1024^3, 28.5 M pairs, 3.9 per voxel: 7.5 ms,
+// issuing on 80 % of slots with 18 lanes (8.9 ms, and 68 %, in the longer kernel; of those the areas
+// took 2.4, the edge axes 2.7 and the face normal 2.4; 45.9 ms with a voxel's
 // triangles alone in the lanes and the warp on one triangle's sub-cells; 12.0 ms with grouped
 // areas and records but the warp still on one triangle).  6 blocks per SM: 9.1 ms.
 __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_t* __restrict__ keys,
@@ -1779,18 +1794,21 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_
                         const uint32_t ue = __shfl_sync(0xffffffffu, st, g + u + 1) - base;
                         if (it < 7u * m) {
                             float acc = 0.0f;
+#pragma unroll 1
                             for (uint32_t j = ub; j < ue; ++j) acc = acc + qw[j * 7 + c];
                             if (c == 0) out.mass[s0 + g + u] = acc;
                             else out.moment[(size_t)(s0 + g + u) * 6 + c - 1] = acc;
                         }
                     }
                 } else if (lane < 7) {
+#pragma unroll 1
                     for (uint32_t j = 0; j < cnt; ++j) accc = accc + qw[j * 7 + lane];
                 }
                 // the masks, voxel by voxel; a voxel's outputs once its last batch is in
                 for (uint32_t u = 0; u < m; ++u) {
                     const uint32_t ub = m > 1 ? __shfl_sync(0xffffffffu, st, g + u) - base : 0u;
                     const uint32_t ue = m > 1 ? __shfl_sync(0xffffffffu, st, g + u + 1) - base : cnt;
+#pragma unroll 1
                     for (uint32_t j = ub; j < ue; ++j)
                         chunk |= *reinterpret_cast<const uint16_t*>(sh.mask + j * TRI_MASK + 2 * lane);
                     if (m > 1 || base + cnt >= gend) {
