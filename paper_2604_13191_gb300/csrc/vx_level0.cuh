@@ -1710,7 +1710,7 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint3
 // issuing on 80 % of slots with 18 lanes (8.9 ms, and 68 %, in the longer kernel; of those the areas
 // took 2.4, the edge axes 2.7 and the face normal 2.4; 45.9 ms with a voxel's
 // triangles alone in the lanes and the warp on one triangle's sub-cells; 12.0 ms with grouped
-// areas and records but the warp still on one triangle).  6 blocks per SM: 9.1 ms.
+// areas and records but the warp still on one triangle).  6 blocks per SM: 8.3 ms.
 __global__ void __launch_bounds__(RED_WARPS * 32, 5) k_reduce_tris(const uint32_t* __restrict__ keys,
                                                                 const uint32_t* __restrict__ prims,
                                                                 const uint32_t* __restrict__ starts,
