@@ -764,8 +764,9 @@ __global__ void __launch_bounds__(1024) k_pack_dirs(const float* __restrict__ d,
 }
 
 // The warp tier's residency: 5 blocks per SM (90 registers, no spill, two steps of the sample
-// loop in flight) cluster the 768k-capsule yarn in 7.1 ms; 6 blocks in 7.24, 4 blocks with four
-// steps in 8.0.  Before the compares by sign, the branch-free roots and the constant folded into
+// loop in flight) cluster the 768k-capsule yarn in 6.8 ms, the loops around the sampling
+// not unrolled: the warps wait for instructions otherwise (7.1 ms; 6 blocks 7.24, 4 blocks with four
+// steps 8.0 ms).  Before the compares by sign, the branch-free roots and the constant folded into
 // the terms: 7.79 ms.
 // One parent listed in `work` per group of G warps (G = 1: a warp per parent, for levels
 // with many parents; G = CL_BLOCK_WARPS: a block per parent, for the few coarse parents
@@ -817,13 +818,16 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
         // gather candidates in (child, lobe) order, with their statistics where the child
         // level kept them (alive = 2: not sampled yet)
         int n = 0;
+#pragma unroll 1
         for (uint32_t c = beg; c < end; ++c) {
             const int lc = in.lobe_count[c];
+#pragma unroll 1
             for (int l = tid; l < lc * 7; l += NT) {
                 const int li = l / 7, j = l % 7;
                 const float x = in.lobes[((size_t)c * in.K + li) * 7 + j];
                 if (j < 6) sm.S[(n + li) * 6 + j] = x; else sm.w[n + li] = x;
             }
+#pragma unroll 1
             for (int l = tid; l < lc; l += NT) {
                 bool have = false;
                 if (cst) {
@@ -841,9 +845,11 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
             }
             n += lc;
         }
+#pragma unroll 1
         for (int l = n + tid; l < slots; l += NT) sm.alive[l] = 0;
         gsync();
         int sampled = 0;
+#pragma unroll 1
         for (int l = 0; l < n; ++l) {
             if (sm.alive[l] != 2) continue;
             const LobeOwn st = sample_lobe<G>(sm.S + l * 6, dirs, N, unit, inv_n, red, turn++);
@@ -854,6 +860,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
             ++sampled;
         }
         gsync();
+#pragma unroll 1
         for (int l = tid; l < n; l += NT) sm.alive[l] = 1;
         gsync();
         int count = n, next = n;
@@ -861,6 +868,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
             // the alive slots in increasing order (count <= 8K <= 64 of them)
             if (tid < 32) {
                 int base = 0;
+#pragma unroll 1
                 for (int s0 = 0; s0 < next; s0 += 32) {
                     const int sl = s0 + tid;
                     const bool al = sl < next && sm.alive[sl];
@@ -874,6 +882,7 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
             // six histogram differences of at most N each, so it fits 32 bits
             unsigned long long best = ~0ull;
             const int npairs = count * (count - 1) / 2;
+#pragma unroll 1
             for (int q = tid; q < npairs; q += NT) {
                 const uint32_t ab = kPairTable.ab[q];
                 const int i = sm.list[ab >> 8], j = sm.list[ab & 0xffu];
@@ -921,12 +930,15 @@ __global__ void __launch_bounds__(G == 1 ? CL_WARPS * 32 : G * 32, G == 1 ? 5 : 
         // output: alive lobes by weight (descending), ties by creation index
         float* lo = out.lobes + (size_t)p * K * 7;
         float* co = out.compact + (size_t)p * K * 6;
+#pragma unroll 1
         for (int x = tid; x < next; x += NT) {
             if (!sm.alive[x]) continue;
             const float wx = sm.w[x];
             int rank = 0;
+#pragma unroll 1
             for (int y = 0; y < next; ++y)
                 if (sm.alive[y] && (sm.w[y] > wx || (sm.w[y] == wx && y < x))) ++rank;
+#pragma unroll 1
             for (int j = 0; j < 6; ++j) lo[rank * 7 + j] = sm.S[x * 6 + j];
             lo[rank * 7 + 6] = wx;
             compact_params(sm.S + x * 6, co + rank * 6);
