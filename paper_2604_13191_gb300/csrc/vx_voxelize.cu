@@ -844,6 +844,10 @@ __device__ __forceinline__ uint64_t voxel_key(uint32_t x, uint32_t y, uint32_t z
 }
 
 // A voxel of a primitive waiting for its gradient: the primitive's slot in the warp and the voxel.
+// A warp's entries wait in a ring of 64: fewer than 32 wait before a turn's pushes, so at most 63 do
+// after it, and a push never meets one that waits.  A push may take the slot of one that has been
+// read, so a __syncwarp stands between the reads and the next pushes.
+constexpr uint32_t ADJ_RING = 64;
 __device__ __forceinline__ uint64_t adj_entry(int slot, int x, int y, int z) {
     return ((uint64_t)slot << 36) | ((uint64_t)x << 24) | ((uint64_t)y << 12) | (uint64_t)z;
 }
@@ -937,7 +941,7 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4*
     struct Shared {
         double c[SEGC * 32];
         double acc[8 * 32];
-        uint64_t queue[64];
+        uint64_t queue[ADJ_RING];
     };
     __shared__ Shared shared[ADJ_WARPS];
     Shared& sh = shared[threadIdx.x >> 5];
@@ -957,18 +961,19 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4*
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) sh.acc[c * 32 + lane] = 0.0;
-        uint32_t qn = 0;
+        uint32_t qh = 0, qn = 0;   // the first waiting entry and their number
         for (;;) {
             const bool more = !walk.done;
             const uint32_t bal = __ballot_sync(0xffffffffu, more);
-            if (more) sh.queue[qn + __popc(bal & lt)] = walk.take(slot);
+            if (more) sh.queue[(qh + qn + __popc(bal & lt)) % ADJ_RING] = walk.take(slot);
             qn += __popc(bal);
             if (bal != 0u && qn < 32u) continue;
             if (qn == 0u) break;
             __syncwarp();
             // the gradients of up to 32 queued voxels
-            const bool on = (uint32_t)lane < min(qn, 32u);
-            const uint64_t e = sh.queue[lane];
+            const uint32_t taken = min(qn, 32u);
+            const bool on = (uint32_t)lane < taken;
+            const uint64_t e = on ? sh.queue[(qh + lane) % ADJ_RING] : 0ull;
             const int own = on ? (int)(e >> 36) : 32;
             bool hit = false;
             double g[8];
@@ -998,10 +1003,9 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4*
                 }
                 __syncwarp();
             }
-            const uint64_t rest = qn > 32u ? sh.queue[32 + lane] : 0ull;
-            __syncwarp();
-            if (qn > 32u) sh.queue[lane] = rest;
-            qn = qn > 32u ? qn - 32u : 0u;
+            __syncwarp();   // (also orders the reads of the entries before the next pushes)
+            qh += taken;
+            qn -= taken;
             if (bal == 0u && qn == 0u) break;
         }
         __syncwarp();
@@ -1280,7 +1284,7 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
                                                      float scale, float4* __restrict__ gverts, float* __restrict__ gw) {
     __shared__ double poly[ADJ_POLY];
     __shared__ double acc[10 * 32];
-    __shared__ uint64_t queue[64];
+    __shared__ uint64_t queue[ADJ_RING];
     const int lane = threadIdx.x, slots = 32 >> lg, slot = lane >> lg, sub = lane & ((1 << lg) - 1);
     const uint32_t lt = (1u << lane) - 1u;
     for (uint64_t p0 = (uint64_t)blockIdx.x * slots; p0 < np; p0 += (uint64_t)gridDim.x * slots) {
@@ -1298,7 +1302,7 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
         long long idx = sub;
 #pragma unroll
         for (int k = 0; k < 10; ++k) acc[k * 32 + lane] = 0.0;
-        uint32_t qn = 0;
+        uint32_t qh = 0, qn = 0;   // the first waiting entry and their number
         for (;;) {
             bool push = false;
             int x = 0, y = 0, z = 0;
@@ -1311,13 +1315,14 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
                 idx += 1 << lg;
             }
             const uint32_t bal = __ballot_sync(0xffffffffu, push);
-            if (push) queue[qn + __popc(bal & lt)] = adj_entry(slot, x, y, z);
+            if (push) queue[(qh + qn + __popc(bal & lt)) % ADJ_RING] = adj_entry(slot, x, y, z);
             qn += __popc(bal);
             if (more && qn < 32u) continue;
             if (qn == 0u) break;
             __syncwarp();
-            const bool on = (uint32_t)lane < min(qn, 32u);
-            const uint64_t e = queue[lane];
+            const uint32_t taken = min(qn, 32u);
+            const bool on = (uint32_t)lane < taken;
+            const uint64_t e = on ? queue[(qh + lane) % ADJ_RING] : 0ull;
             const int own = on ? (int)(e >> 36) : 32;
             double g[10];
             int ex = 0, ey = 0, ez = 0;
@@ -1344,10 +1349,9 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
                 }
                 __syncwarp();
             }
-            const uint64_t rest = qn > 32u ? queue[32 + lane] : 0ull;
-            __syncwarp();
-            if (qn > 32u) queue[lane] = rest;
-            qn = qn > 32u ? qn - 32u : 0u;
+            __syncwarp();   // (also orders the reads of the entries before the next pushes)
+            qh += taken;
+            qn -= taken;
             if (!more && qn == 0u) break;
         }
         __syncwarp();
