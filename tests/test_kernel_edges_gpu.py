@@ -246,3 +246,49 @@ def test_pair_sort_with_and_without_its_own_offsets(n):
     for f in ("keys", "mask", "mass", "moment", "occ", "proj", "lobes"):
         assert np.array_equal(np.asarray(whole[f]).view(np.uint8), np.asarray(parts[f]).view(np.uint8)), f
     ctx.close()
+
+
+@pytest.mark.parametrize("a,b,r", [
+    ((-4e19, -4e19, -4e19), (-4.1e19, -4e19, -4e19), 6e19),      # every sum of squares overflows
+    ((4e19, 0, 0), (4e19, 1e19, 0), 7e19),                       # the squares of one axis do
+    ((3, -4e19, -4e19), (5, -4e19, -4e19), 6e19),                # those of two
+    ((-4e19, 3, -4e19), (-4e19, 5, -4e19), 6e19),
+    ((-4e19, -4e19, 3), (4e19, 4e19, 3), 6e19),                  # the axis runs through the grid
+    ((1e19, 1e19, 1e19), (1e19, 1e19, 1.2e19), 2e19),            # only the radius does
+    ((2e19, 1e19, 1e19), (2e19, 1e19, 1e19), 3e19),              # without length
+])
+def test_capsule_radius_whose_square_overflows(a, b, r):
+    """r^2 is infinite in FP32: the comparisons of steps 1 and 2 hold against an infinite budget and against
+    none that is not a number, and step 3's minimum is at most r^2 whatever it is.  Stated here in
+    numpy's FP32, sub-cell by sub-cell."""
+    R, f32 = 8, np.float32
+    ctrl = np.array([[*a, r], [*b, r]], f32)
+    i = np.arange(R)
+    vox = np.stack(np.meshgrid(i, i, i, indexing="ij"), -1).reshape(-1, 3).astype(f32)
+    lo = np.arange(8).astype(f32) * f32(0.125)
+    hi = (np.arange(8) + 1).astype(f32) * f32(0.125)
+    with np.errstate(over="ignore", invalid="ignore"):
+        def squares(p, q):                                       # [voxel, axis, interval]
+            mn, mx = np.minimum(p, q)[..., None], np.maximum(p, q)[..., None]
+            g = np.maximum(np.maximum(lo - mx, mn - hi), f32(0))
+            return g * g
+        A, B = ctrl[0, :3] - vox, ctrl[1, :3] - vox
+        rr = f32(ctrl[0, 3] * ctrl[0, 3])
+        assert np.isinf(rr)
+        bits = np.zeros((R ** 3, 8, 8, 8), bool)                 # [voxel, sz, sy, sx]
+        for s in (squares(A, B), squares(A, A), squares(B, B)):
+            T = rr - (s[:, 1, None, :] + s[:, 2, :, None])       # [voxel, sz, sy]
+            bits |= s[:, 0, None, None, :] <= T[..., None]
+    words = np.packbits(bits.reshape(R ** 3, 512), axis=1, bitorder="little").view(np.uint64)
+    key = np.zeros(R ** 3, np.uint64)
+    for t in range(3):
+        for ax in range(3):
+            key |= ((vox[:, ax].astype(np.uint64) >> np.uint64(t)) & np.uint64(1)) << np.uint64(3 * t + ax)
+    order = np.argsort(key)
+    order = order[words[order].any(1)]
+    ctx = vx.Context(DEV)
+    got = ctx.voxelize(synth.Grid((0.0, 0.0, 0.0), 1.0, R), ctrl=torch.from_numpy(ctrl).to(DEV),
+                       fiber_offsets=torch.tensor([0, 2], device=DEV)).host()
+    assert np.array_equal(got["keys"].astype(np.uint64), key[order])
+    assert np.array_equal(got["mask"].view(np.uint64).reshape(-1, 8), words[order])
+    ctx.close()
