@@ -91,19 +91,38 @@ __global__ void k_bprep_tris(const float4* __restrict__ tv, const float* __restr
     inst_of[p] = (uint8_t)ii;
 }
 
-// count with the resolution of each primitive's instance (see k_count)
+// count with the resolution of each primitive's instance (see k_count); `go` (or NULL): nothing is done
+// unless it holds kCountLarge
 template <bool FIBER>
 __global__ void __launch_bounds__(COUNT_WARPS * 32) k_bcount(const float4* __restrict__ r0, const float4* __restrict__ r1,
                                                              const float4* __restrict__ r2, uint32_t np, int lg,
                                                              const BInst* __restrict__ inst,
-                                                             const uint8_t* __restrict__ inst_of,
+                                                             const uint8_t* __restrict__ inst_of, int least, int most,
                                                              uint32_t* __restrict__ counts,
-                                                             uint32_t* __restrict__ ballots) {
+                                                             uint32_t* __restrict__ ballots, uint32_t* __restrict__ flags,
+                                                             const uint32_t* __restrict__ go) {
     __shared__ CountRecords<FIBER> rec[COUNT_WARPS];
+    if (go && !(*go & kCountLarge)) return;
     const uint32_t groups = (uint32_t)(((uint64_t)np + (1u << lg) - 1) >> lg);
     for (uint32_t g = blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); g < groups; g += gridDim.x * COUNT_WARPS)
         count_group<FIBER>(rec[threadIdx.x >> 5], g << lg, lg, np, r0, r1, r2,
-                           [&](uint32_t p) { return full_window(inst[inst_of[p]].R); }, counts, ballots, CAND_BALLOTS);
+                           [&](uint32_t p) { return full_window(inst[inst_of[p]].R); }, least, most, counts, ballots,
+                           CAND_BALLOTS, flags);
+}
+
+// The grouped count and, where it may leave large ranges out, the launch that takes those: a graph
+// cannot leave it away, so its blocks (eight per SM) look at the flag first.  flags: a zeroed word.
+// Returns the number of launches.
+template <bool FIBER>
+int launch_bcount(const float4* r0, const float4* r1, const float4* r2, uint32_t np, const BInst* inst,
+                  const uint8_t* inst_of, uint32_t* counts, uint32_t* ballots, uint32_t* flags, cudaStream_t s) {
+    const int lg = count_lanes_log2(np);
+    k_bcount<FIBER><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
+        r0, r1, r2, np, lg, inst, inst_of, 0, lg > 0 ? kGroupRange : kAnyRange, counts, ballots, flags, nullptr);
+    if (lg == 0) return 1;
+    k_bcount<FIBER><<<std::min(count_blocks(np, 0), (unsigned)vx::kSMs * 8), COUNT_WARPS * 32, 0, s>>>(
+        r0, r1, r2, np, 0, inst, inst_of, kGroupRange + 1, kAnyRange, counts, ballots, nullptr, flags);
+    return 2;
 }
 
 // emit, clamped to the pair capacity (an overflow is reported by the count clamp); the ballots
@@ -276,7 +295,8 @@ enum {
     C_ERR = 0, C_SEGTOT, C_PAIRS_TOT, C_PAIRS, C_SEG_TOT, C_SEG, C_VOX_TOT, C_VOX,
     C_LVL = 8,  // C_LVL + l: parent count of level l (1..kMaxLevels); C_LVL + 16 + l: raw totals
     C_TAKE = 48, // work counter of the reduce kernel
-    C_CLUSTER = 50  // [50] parents listed for clustering, [51] their take counter
+    C_CLUSTER = 50, // [50] parents listed for clustering, [51] their take counter
+    C_COUNT = 52    // flags of the candidate count
 };
 
 // Buffers of the pair stages (candidate pairs, sort, segments, per-voxel temporaries and
@@ -467,14 +487,9 @@ vx_status instance_pairs(vx_batch* b, bool fiber, const vx_primitives* prims, co
             k_bprep_tris<<<gf(np, 256, 1u << 30), 256, 0, s>>>((const float4*)prims->tri_verts, prims->weights, np,
                                                                dinst, ninst, r0, r1, r2, inst_of, C + C_ERR);
         }
-        const int lg = count_lanes_log2(np);
         if (e == cudaSuccess) {
-            if (fiber)
-                k_bcount<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(r0, r1, r2, np, lg, dinst, inst_of, cnt,
-                                                                                 nullptr);
-            else
-                k_bcount<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(r0, r1, r2, np, lg, dinst, inst_of, cnt,
-                                                                                  nullptr);
+            if (fiber) launch_bcount<true>(r0, r1, r2, np, dinst, inst_of, cnt, nullptr, C + C_COUNT, s);
+            else launch_bcount<false>(r0, r1, r2, np, dinst, inst_of, cnt, nullptr, C + C_COUNT, s);
             k_inst_pair_totals<<<ninst, 256, 0, s>>>(cnt, dinst, tot);
             e = cudaGetLastError();
         }
@@ -529,15 +544,10 @@ vx_status enqueue(vx_batch* b, SubBatch& S, cudaStream_t s, bool plan, int64_t* 
     }
     // ---- candidates ----------------------------------------------------------------------
     const unsigned cblocks = (unsigned)std::min<size_t>((S.np + EMIT_WARPS - 1) / EMIT_WARPS, (size_t)vx::kSMs * 64);
-    const int lg = count_lanes_log2(S.np);
-    if (S.fiber)
-        k_bcount<true><<<count_blocks(S.np, lg), COUNT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, lg, S.dinst,
-                                                                           S.inst_of, S.cnt, S.ballots);
-    else
-        k_bcount<false><<<count_blocks(S.np, lg), COUNT_WARPS * 32, 0, s>>>(S.r0, S.r1, S.r2, S.np, lg, S.dinst,
-                                                                            S.inst_of, S.cnt, S.ballots);
+    *nl += S.fiber ? launch_bcount<true>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of, S.cnt, S.ballots, C + C_COUNT, s)
+                   : launch_bcount<false>(S.r0, S.r1, S.r2, S.np, S.dinst, S.inst_of, S.cnt, S.ballots, C + C_COUNT, s);
     if (vx_scan_u32_scratch(S.cnt, S.offs, S.np, C + C_PAIRS_TOT, S.part, s) != cudaSuccess) return VX_ERR_CUDA;
-    *nl += 4;
+    *nl += 3;
     if (plan) {
         const uint32_t err = readback(C_ERR);
         if (err) return VX_ERR_INVALID_ARG;

@@ -1236,27 +1236,48 @@ __device__ __forceinline__ int count_quick(const CountRecords<false>& cr, int i,
     return m > 1.0f ? 1 : (m < -1.0f ? -1 : 0);
 }
 
+// A warp takes its group's primitives one after the other, so one with a range of many voxels would
+// make its neighbours wait (and 32 of them in a row, a mesh's ground or walls, would all fall to one
+// warp).  A launch therefore takes only ranges of [least, most] voxels: the grouped launch leaves those
+// above kGroupRange to a second one with a warp each, made when it has raised kCountLarge.  The bound is
+// the most that a ballot store holds (64 words); a group of 32 such ranges is 0.25 ms for one warp.
+// 100,000 small triangles and 32 of 200 voxels' extent in a row: 82 ms, 287 ms in groups of any range.
+constexpr int kGroupRange = 2048, kAnyRange = 0x7fffffff;
+constexpr uint32_t kCountLarge = 1u;      // a range above `most` was left out (its count is 0)
+constexpr uint32_t kCountUnstored = 2u;   // a range has more voxels than its ballot words
+
 // floor of 0 <= x < 2^22, as a float
 __device__ __forceinline__ float floor_pos(float x) { return __fadd_rd(x, 8388608.0f) - 8388608.0f; }
 
 // Counts of 2^lg consecutive primitives from p0 (fewer at np) by a warp, and their ballots; win(p) is
-// the window of a primitive.
+// the window of a primitive.  Ranges below `least` are passed over, those above `most` count 0; flags
+// (or NULL) receives kCountLarge and kCountUnstored.
 template <bool FIBER, class Win>
 __device__ __forceinline__ void count_group(CountRecords<FIBER>& cr, uint32_t p0, int lg, uint32_t np,
                                             const float4* __restrict__ r0, const float4* __restrict__ r1,
-                                            const float4* __restrict__ r2, Win win, uint32_t* __restrict__ counts,
-                                            uint32_t* __restrict__ ballots, uint32_t stride) {
+                                            const float4* __restrict__ r2, Win win, int least, int most,
+                                            uint32_t* __restrict__ counts, uint32_t* __restrict__ ballots,
+                                            uint32_t stride, uint32_t* __restrict__ flags) {
     const int lane = threadIdx.x & 31;
     const uint32_t p = p0 + (uint32_t)lane;
     const int members = (int)min(1u << lg, np - p0);
+    uint32_t raise = 0;
+    bool write = false;
     if (lane < members) {
         float4 a, b, c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         const Range rg = prim_range<FIBER>(r0, r1, r2, p, win(p), a, b, c);
-        count_record(cr, lane, a, b, c, rg);
+        const bool below = rg.total < least, above = rg.total > most;
+        write = !below;
+        raise = (above ? kCountLarge : 0u) | (ballots && rg.total > 32ll * stride ? kCountUnstored : 0u);
+        if (!below && !above) count_record(cr, lane, a, b, c, rg);
         const float n0 = (float)rg.n[0], n1 = (float)rg.n[1];
         cr.r[0][lane] = make_float4(__frcp_rn(n0), n0, __frcp_rn(n1), n1);
         cr.r[1][lane] = make_float4(__int_as_float(rg.lo[0]), __int_as_float(rg.lo[1]), __int_as_float(rg.lo[2]),
-                                    __int_as_float((int)min(rg.total, (long long)kMaxFastRange + 1)));
+                                    __int_as_float(below || above ? 0 : (int)min(rg.total, (long long)kMaxFastRange + 1)));
+    }
+    if (flags && __any_sync(0xffffffffu, raise != 0u)) {
+        raise = __reduce_or_sync(0xffffffffu, raise);
+        if (lane == 0 && (raise & ~*(volatile uint32_t*)flags)) atomicOr(flags, raise);
     }
     __syncwarp();
     uint32_t mine = 0;
@@ -1291,7 +1312,7 @@ __device__ __forceinline__ void count_group(CountRecords<FIBER>& cr, uint32_t p0
         }
         if (lane == i) mine = n;
     }
-    if (lane < members) counts[p] = mine;
+    if (write) counts[p] = mine;
     __syncwarp();
 }
 
@@ -1309,13 +1330,14 @@ inline unsigned count_blocks(uint32_t np, int lg) {
 template <bool FIBER>
 __global__ void __launch_bounds__(COUNT_WARPS * 32, FIBER ? 7 : 5) k_count(const float4* __restrict__ r0, const float4* __restrict__ r1,
                                                             const float4* __restrict__ r2, uint32_t np, Window R, int lg,
-                                                            uint32_t* __restrict__ counts, uint32_t* __restrict__ ballots,
-                                                            uint32_t stride) {
+                                                            int least, int most, uint32_t* __restrict__ counts,
+                                                            uint32_t* __restrict__ ballots, uint32_t stride,
+                                                            uint32_t* __restrict__ flags) {
     __shared__ CountRecords<FIBER> rec[COUNT_WARPS];
     const uint32_t groups = (uint32_t)(((uint64_t)np + (1u << lg) - 1) >> lg);
     for (uint32_t g = blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); g < groups; g += gridDim.x * COUNT_WARPS)
-        count_group<FIBER>(rec[threadIdx.x >> 5], g << lg, lg, np, r0, r1, r2, [&](uint32_t) { return R; }, counts, ballots,
-                           stride);
+        count_group<FIBER>(rec[threadIdx.x >> 5], g << lg, lg, np, r0, r1, r2, [&](uint32_t) { return R; }, least, most,
+                           counts, ballots, stride, flags);
 }
 
 // Emit from the stored ballots.  A warp takes 32 consecutive primitives; their pairs are consecutive
@@ -1324,7 +1346,8 @@ __global__ void __launch_bounds__(COUNT_WARPS * 32, FIBER ? 7 : 5) k_count(const
 // (A warp per primitive left most of its lanes to the addresses of one word: 0.52 ms against
 // 0.22 ms for the 75 M pairs of the 768k-capsule yarn.)  Morton codes come from a table of one
 // coordinate's spread bits in shared memory.  A group with a primitive whose range was too large
-// to be stored is taken primitive by primitive, as k_candidates does.
+// to be stored is left to k_candidates, which the host launches for those when the count pass has
+// raised kCountUnstored: one warp on a whole group took up to 32 times as long.
 constexpr int STAGE_WARPS = 4;
 template <bool FIBER>
 __global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* __restrict__ r0,
@@ -1333,7 +1356,7 @@ __global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* 
                                                                   const uint32_t* __restrict__ offs,
                                                                   uint32_t* __restrict__ keys,
                                                                   uint32_t* __restrict__ vals,
-                                                                  uint32_t* __restrict__ ballots, uint32_t stride) {
+                                                                  const uint32_t* __restrict__ ballots, uint32_t stride) {
     __shared__ uint32_t spread[1024];
     __shared__ uint32_t stage_k[STAGE_WARPS][1024], stage_v[STAGE_WARPS][1024];
     const int lane = threadIdx.x & 31;
@@ -1352,14 +1375,7 @@ __global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* 
             float4 a, b, c;
             rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
         }
-        if (__any_sync(0xffffffffu, rg.total > 32ll * stride)) {
-            for (uint32_t q = p0; q < min(p0 + 32u, np); ++q) {
-                float4 a, b, c;
-                const Range rq = prim_range<FIBER>(r0, r1, r2, q, R, a, b, c);
-                candidates_of<FIBER, true>(q, a, b, c, rq, R, offs[q], keys, vals, ballots, stride);
-            }
-            continue;
-        }
+        if (__any_sync(0xffffffffu, rg.total > 32ll * stride)) continue;
         // ranges of at most 2048 voxels: i / n as the high word of i (2^32 / n + 1), exact for i n < 2^32
         const uint32_t tot = (uint32_t)rg.total, nw = (tot + 31u) / 32u;
         const uint32_t n0 = (uint32_t)max(rg.n[0], 1), n1 = (uint32_t)max(rg.n[1], 1);
@@ -1417,7 +1433,8 @@ __global__ void __launch_bounds__(STAGE_WARPS * 32) k_emit_stored(const float4* 
     }
 }
 
-// emit of a pass without stored ballots: a warp per primitive tests its range again
+// emit with a warp per primitive: of a pass without stored ballots, which tests the ranges again, or
+// (unstored_only) of the groups of 32 that k_emit_stored leaves
 template <bool FIBER>
 __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __restrict__ r0,
                                                                 const float4* __restrict__ r1,
@@ -1425,10 +1442,16 @@ __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __
                                                                 const uint32_t* __restrict__ offs,
                                                                 uint32_t* __restrict__ keys,
                                                                 uint32_t* __restrict__ vals,
-                                                                uint32_t* __restrict__ ballots, uint32_t stride) {
+                                                                uint32_t* __restrict__ ballots, uint32_t stride,
+                                                                bool unstored_only) {
     const uint32_t warps = gridDim.x * EMIT_WARPS;
     for (uint32_t p = blockIdx.x * EMIT_WARPS + (threadIdx.x >> 5); p < np; p += warps) {
         float4 a, b, c;
+        if (unstored_only) {
+            const uint32_t q = (p & ~31u) + (threadIdx.x & 31u);
+            if (!__any_sync(0xffffffffu, q < np && prim_range<FIBER>(r0, r1, r2, q, R, a, b, c).total > 32ll * stride))
+                continue;
+        }
         const Range rg = prim_range<FIBER>(r0, r1, r2, p, R, a, b, c);
         candidates_of<FIBER, true>(p, a, b, c, rg, R, offs[p], keys, vals, ballots, stride);
     }

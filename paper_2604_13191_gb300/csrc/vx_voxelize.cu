@@ -58,7 +58,7 @@ vx_status window_ballots(vx_context* ctx, uint32_t np, cudaStream_t s, uint32_t*
 
 // Candidate counts and offsets of the primitives over one window (WS_COUNT, WS_OFFS), and
 // the hit ballots of their ranges (WS_BALLOTS, see window_ballots); the exact total goes to
-// *total.  Synchronises the stream once.
+// *total.  Synchronises the stream once (twice when a range is too large for the grouped pass).
 vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& win, float4* r0, float4* r1,
                        float4* r2, uint32_t* misc, cudaStream_t s, uint64_t* total) {
     VX_TRY(vx_ws_ensure(ctx, WS_COUNT, (size_t)np * 4, s));
@@ -76,22 +76,31 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
         ctx->ballots_win[i] = win.lo[i];
         ctx->ballots_win[3 + i] = win.hi[i];
     }
-    const int lg = count_lanes_log2(np);
-    if (fiber)
-        VX_LAUNCH(ctx, ST_COUNT, s, k_count<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, lg, cnt, ballots, stride));
-    else
-        VX_LAUNCH(ctx, ST_COUNT, s, k_count<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
-                                        r0, r1, r2, np, win, lg, cnt, ballots, stride));
     unsigned long long* t64 = (unsigned long long*)(misc + 8);
-    bool done = false;
-    VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s, t64, vx_pin_of(ctx, misc, 12), &done));
-    if (!done) {   // no primitives
-        VX_CUDA_TRY(cudaMemsetAsync(t64, 0, 8, s));
-        VX_TRY(vx_readback_async(ctx, 0, misc, 48, s));
-    }
-    VX_CUDA_TRY(cudaStreamSynchronize(s));
-    if (((uint32_t*)ctx->host_pin)[0]) return VX_ERR_INVALID_ARG;
+    uint32_t* const flags = misc + 14;   // (zero but for a count pass that has raised some)
+    // ranges of [least, most] voxels, 2^lg primitives to a warp, then offsets and totals
+    auto pass = [&](int lg, int least, int most, uint32_t* raise) -> vx_status {
+        if (fiber)
+            VX_LAUNCH(ctx, ST_COUNT, s, k_count<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
+                                            r0, r1, r2, np, win, lg, least, most, cnt, ballots, stride, raise));
+        else
+            VX_LAUNCH(ctx, ST_COUNT, s, k_count<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
+                                            r0, r1, r2, np, win, lg, least, most, cnt, ballots, stride, raise));
+        bool done = false;
+        VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s, t64, vx_pin_of(ctx, misc, 16), &done));
+        if (!done) {   // no primitives
+            VX_CUDA_TRY(cudaMemsetAsync(t64, 0, 8, s));
+            VX_TRY(vx_readback_async(ctx, 0, misc, 64, s));
+        }
+        VX_CUDA_TRY(cudaStreamSynchronize(s));
+        return ((uint32_t*)ctx->host_pin)[0] ? VX_ERR_INVALID_ARG : VX_OK;
+    };
+    const int lg = count_lanes_log2(np);
+    VX_TRY(pass(lg, 0, lg > 0 ? kGroupRange : kAnyRange, flags));
+    const uint32_t raised = ((uint32_t*)ctx->host_pin)[14];
+    ctx->ballots_unstored = (raised & kCountUnstored) != 0;
+    if (raised) VX_CUDA_TRY(cudaMemsetAsync(flags, 0, 4, s));
+    if (raised & kCountLarge) VX_TRY(pass(0, kGroupRange + 1, kAnyRange, nullptr));
     *total = ((const uint64_t*)ctx->host_pin)[4];
     return VX_OK;
 }
@@ -148,12 +157,15 @@ vx_status window_segments(vx_context* ctx, bool fiber, uint32_t np, const Window
         else
             VX_LAUNCH(ctx, ST_EMIT, s, k_emit_stored<false><<<eblocks, STAGE_WARPS * 32, 0, s>>>(
                                            r0, r1, r2, np, win, offs, *k0, *v0, ctx->ballots, ctx->ballots_stride));
-    } else if (fiber) {
-        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, offs, *k0, *v0, nullptr, 0u));
-    } else {
-        VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
-                                       r0, r1, r2, np, win, offs, *k0, *v0, nullptr, 0u));
+    }
+    if (!same || ctx->ballots_unstored) {
+        uint32_t* const ballots = same ? ctx->ballots : nullptr;
+        if (fiber)
+            VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<true><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
+                                           r0, r1, r2, np, win, offs, *k0, *v0, ballots, ctx->ballots_stride, same));
+        else
+            VX_LAUNCH(ctx, ST_EMIT, s, k_candidates<false><<<cblocks, EMIT_WARPS * 32, 0, s>>>(
+                                           r0, r1, r2, np, win, offs, *k0, *v0, ballots, ctx->ballots_stride, same));
     }
     VX_CUDA_TRY(cudaGetLastError());
     VX_TRY(vx_radix_sort_u32(ctx, k0, v0, k1, v1, npairs, 3 * bits, s, misc));
@@ -283,7 +295,7 @@ vx_status prepare(vx_context* ctx, const vx_primitives* prims, const vx_grid* gr
     VX_TRY(vx_ws_ensure(ctx, WS_REC_B, (size_t)np * 16, s));
     if (!fiber) VX_TRY(vx_ws_ensure(ctx, WS_REC_C, (size_t)np * 16, s));
     VX_TRY(vx_ws_ensure(ctx, WS_MISC, 256, s));
-    uint32_t* misc = (uint32_t*)ctx->ws[WS_MISC].p;   // [0] err, [1] npairs, [2] nseg, [3] nvox, [4] segtotal
+    uint32_t* misc = (uint32_t*)ctx->ws[WS_MISC].p;   // [0] err, [1] npairs, [2] nseg, [3] nvox, [4] segtotal, [14] count flags
     VX_CUDA_TRY(cudaMemsetAsync(misc, 0, 64, s));
     float4* r0 = (float4*)ctx->ws[WS_REC_A].p;
     float4* r1 = (float4*)ctx->ws[WS_REC_B].p;
@@ -1575,17 +1587,23 @@ extern "C" vx_status vx_backward_noalloc(const vx_primitives* prims, const vx_gr
     k_prep_fibers<<<grid_for(np, 256), 256, 0, s>>>((const float4*)prims->ctrl, prims->num_ctrl, prims->fiber_offsets, fs, F, misc + 4,
                                                      prims->weights, np, g, r0, r1, misc);
     const int clg = count_lanes_log2(np);
-    k_count<true><<<count_blocks(np, clg), COUNT_WARPS * 32, 0, s>>>(r0, r1, nullptr, np, full_window((int)R), clg, cnt,
-                                                                     nullptr, 0u);
-    // the exact 64-bit total
-    k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
-        cnt, np, (unsigned long long*)(misc + 8));
-    uint32_t host[12] = {0};
-    NA_TRY(cudaMemcpyAsync(host, misc, 48, cudaMemcpyDeviceToHost, s));
-    NA_TRY(cudaStreamSynchronize(s));
-    if (host[0]) return VX_ERR_INVALID_ARG;
+    uint32_t host[16] = {0};
     uint64_t npairs64 = 0;
-    memcpy(&npairs64, host + 8, 8);
+    // (ranges too large for the grouped launch are counted by a second one)
+    for (int turn = 0; turn < 2; ++turn) {
+        k_count<true><<<count_blocks(np, turn ? 0 : clg), COUNT_WARPS * 32, 0, s>>>(
+            r0, r1, nullptr, np, full_window((int)R), turn ? 0 : clg, turn ? kGroupRange + 1 : 0,
+            turn || clg == 0 ? kAnyRange : kGroupRange, cnt, nullptr, 0u, misc + 14);
+        // the exact 64-bit total
+        NA_TRY(cudaMemsetAsync(misc + 8, 0, 8, s));
+        k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
+            cnt, np, (unsigned long long*)(misc + 8));
+        NA_TRY(cudaMemcpyAsync(host, misc, 64, cudaMemcpyDeviceToHost, s));
+        NA_TRY(cudaStreamSynchronize(s));
+        if (host[0]) return VX_ERR_INVALID_ARG;
+        memcpy(&npairs64, host + 8, 8);
+        if (!(host[14] & kCountLarge)) break;
+    }
     if (npairs64 > NA_MAX_PAIRS) return VX_ERR_CAPACITY;
     // the caller's outputs are written only once every limit has passed
     const int lg = adjoint_lanes_log2(np);
