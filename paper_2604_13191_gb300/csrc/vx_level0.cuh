@@ -1243,6 +1243,8 @@ __device__ __forceinline__ int count_quick(const CountRecords<false>& cr, int i,
 // the most that a ballot store holds (64 words); a group of 32 such ranges is 0.25 ms for one warp.
 // 100,000 small triangles and 32 of 200 voxels' extent in a row: 82 ms, 287 ms in groups of any range.
 constexpr int kGroupRange = 2048, kAnyRange = 0x7fffffff;
+// (a range of a 2048^3 grid can hold 2^33 voxels)
+__device__ __forceinline__ int capped_total(const Range& rg) { return (int)min(rg.total, (long long)kAnyRange); }
 constexpr uint32_t kCountLarge = 1u;      // a range above `most` was left out (its count is 0)
 constexpr uint32_t kCountUnstored = 2u;   // a range has more voxels than its ballot words
 
@@ -1266,14 +1268,15 @@ __device__ __forceinline__ void count_group(CountRecords<FIBER>& cr, uint32_t p0
     if (lane < members) {
         float4 a, b, c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         const Range rg = prim_range<FIBER>(r0, r1, r2, p, win(p), a, b, c);
-        const bool below = rg.total < least, above = rg.total > most;
+        const int tot = capped_total(rg);
+        const bool below = tot < least, above = tot > most;
         write = !below;
         raise = (above ? kCountLarge : 0u) | (ballots && rg.total > 32ll * stride ? kCountUnstored : 0u);
         if (!below && !above) count_record(cr, lane, a, b, c, rg);
         const float n0 = (float)rg.n[0], n1 = (float)rg.n[1];
         cr.r[0][lane] = make_float4(__frcp_rn(n0), n0, __frcp_rn(n1), n1);
         cr.r[1][lane] = make_float4(__int_as_float(rg.lo[0]), __int_as_float(rg.lo[1]), __int_as_float(rg.lo[2]),
-                                    __int_as_float(below || above ? 0 : (int)min(rg.total, (long long)kMaxFastRange + 1)));
+                                    __int_as_float(below || above ? 0 : min(tot, kMaxFastRange + 1)));
     }
     if (flags && __any_sync(0xffffffffu, raise != 0u)) {
         raise = __reduce_or_sync(0xffffffffu, raise);
