@@ -29,15 +29,6 @@
 
 namespace {
 
-// exact 64-bit total of the per-primitive candidate counts (the 32-bit scan total wraps)
-__global__ void k_sum_u64(const uint32_t* __restrict__ cnt, uint32_t n, unsigned long long* __restrict__ total) {
-    unsigned long long acc = 0;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) acc += cnt[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(total, acc);
-}
-
 // The count pass's ballot store (WS_BALLOTS) in *out and its words per primitive in *stride: 64 (ranges
 // of up to 2048 voxels, a capsule of 5 voxels' radius), 32 or 8, the most that takes at most 256 MB;
 // NULL when 8 take more (the emit pass then tests every voxel again).  A range's unused words
@@ -295,7 +286,7 @@ vx_status prepare(vx_context* ctx, const vx_primitives* prims, const vx_grid* gr
     VX_TRY(vx_ws_ensure(ctx, WS_REC_B, (size_t)np * 16, s));
     if (!fiber) VX_TRY(vx_ws_ensure(ctx, WS_REC_C, (size_t)np * 16, s));
     VX_TRY(vx_ws_ensure(ctx, WS_MISC, 256, s));
-    uint32_t* misc = (uint32_t*)ctx->ws[WS_MISC].p;   // [0] err, [1] npairs, [2] nseg, [3] nvox, [4] segtotal, [14] count flags
+    uint32_t* misc = (uint32_t*)ctx->ws[WS_MISC].p;   // [0] err, [1] npairs, [2] nseg, [3] nvox, [4] segtotal, [14] count flags, [15] large walks
     VX_CUDA_TRY(cudaMemsetAsync(misc, 0, 64, s));
     float4* r0 = (float4*)ctx->ws[WS_REC_A].p;
     float4* r1 = (float4*)ctx->ws[WS_REC_B].p;
@@ -903,22 +894,35 @@ struct SegWalk {
     static __device__ __forceinline__ int clampi(float f, int lo, int hi) {
         return f >= (float)hi ? hi : (f <= (float)lo ? lo : (f != f ? lo : (int)f));
     }
+    static __device__ __forceinline__ int longest(float4 a, float4 b) {
+        const float e0 = fabsf(b.x - a.x), e1 = fabsf(b.y - a.y), e2 = fabsf(b.z - a.z);
+        return e0 >= e1 && e0 >= e2 ? 0 : (e1 >= e2 ? 1 : 2);
+    }
+    // number of slabs of a segment, and the first
+    static __device__ __forceinline__ int slabs(float4 a, float4 b, int R, int m, int& first) {
+        const float am = sel3(m, a.x, a.y, a.z), bm = sel3(m, b.x, b.y, b.z);
+        first = clampi(floorf(fminf(am, bm)), 0, R);
+        return max(clampi(floorf(fmaxf(am, bm)), -1, R - 1) - first + 1, 0);
+    }
+    static __device__ __forceinline__ int slabs(float4 a, float4 b, int R) {
+        int first;
+        return slabs(a, b, R, longest(a, b), first);
+    }
     __device__ __forceinline__ void start(float4 a, float4 b, int R_, int sub, int step_) {
         R = R_;
         step = step_;
         A[0] = a.x; A[1] = a.y; A[2] = a.z;
         d[0] = b.x - a.x; d[1] = b.y - a.y; d[2] = b.z - a.z;
-        const float e0 = fabsf(d[0]), e1 = fabsf(d[1]), e2 = fabsf(d[2]);
-        m = e0 >= e1 && e0 >= e2 ? 0 : (e1 >= e2 ? 1 : 2);
+        m = longest(a, b);
         i1 = m == 0 ? 1 : 0;
         i2 = m == 2 ? 1 : 2;
         const float M = fmaxf(fmax3(fabsf(a.x), fabsf(a.y), fabsf(a.z)), fmax3(fabsf(b.x), fabsf(b.y), fabsf(b.z)));
         tol = 1e-6f * ((M + (float)R) + 1.0f);
         const float dm = sel3(m, d[0], d[1], d[2]);
         inv = dm != 0.0f ? 1.0f / dm : 0.0f;
-        const float am = sel3(m, a.x, a.y, a.z), bm = sel3(m, b.x, b.y, b.z);
-        s = clampi(floorf(fminf(am, bm)), 0, R) + sub;
-        s_end = clampi(floorf(fmaxf(am, bm)), -1, R - 1);
+        int first;
+        s_end = slabs(a, b, R, m, first) + first - 1;
+        s = first + sub;
         done = false;
         slab();
     }
@@ -940,12 +944,17 @@ struct SegWalk {
 // twenty, so the voxels come from the axis alone.  They go into a queue of the warp and are taken
 // 32 at a time, so that the FP64 work (the bound: 2 operations per clock and SM) runs with full
 // lanes whatever the segments' lengths; each segment's terms are added in the order of its walk.
+// A launch takes the segments of [least, most] slabs: with fewer than 32 lanes each, one of more than
+// kWalkSlabs would keep the others waiting, and goes to a second launch with a warp each (100,000
+// segments, 32 of them 200 voxels long: 0.7 ms, 1.9 ms on single lanes).
 // 768k segments at 256^3: 0.34 ms (0.44 with IEEE quotients and roots), against 9.8 ms for a warp per
 // segment over its candidate pairs (and 0.5 ms to count and emit those).
 constexpr int ADJ_WARPS = 4;
+constexpr int kWalkSlabs = 64;
 __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4* __restrict__ ra,
                                                                    const float4* __restrict__ rb, uint32_t np, int R,
-                                                                   int lg, const uint64_t* __restrict__ keys0,
+                                                                   int lg, int least, int most,
+                                                                   const uint64_t* __restrict__ keys0,
                                                                    uint32_t V0, const double* __restrict__ gm,
                                                                    const double* __restrict__ gM,
                                                                    double* __restrict__ seg_grad,
@@ -966,11 +975,18 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4*
         __syncwarp();
         SegWalk walk;
         walk.done = true;
+        bool mine = false;
         if (p < np) {
             const float4 a = ra[p], b = rb[p];
-            if (sub == 0) seg_constants(a, b, sh.c, slot);
-            walk.start(a, b, R, sub, 1 << lg);
+            const int n = SegWalk::slabs(a, b, R);
+            mine = n >= least && n <= most;
+            if (mine) {
+                if (sub == 0) seg_constants(a, b, sh.c, slot);
+                walk.start(a, b, R, sub, 1 << lg);
+            }
         }
+        const uint32_t owned = __ballot_sync(0xffffffffu, mine);
+        if (owned == 0u) continue;
 #pragma unroll
         for (int c = 0; c < 8; ++c) sh.acc[c * 32 + lane] = 0.0;
         uint32_t qh = 0, qn = 0;   // the first waiting entry and their number
@@ -1022,8 +1038,8 @@ __global__ void __launch_bounds__(ADJ_WARPS * 32) k_adjoint_fibers(const float4*
         }
         __syncwarp();
         for (int i = lane; i < slots * 8; i += 32)
-            if (p0 + (i >> 3) < np) seg_grad[p0 * 8 + i] = sh.acc[(i & 7) * 32 + (i >> 3)];
-        if (gw && lane < slots && p0 + lane < np) gw[p0 + lane] = (float)sh.acc[7 * 32 + lane];
+            if ((owned >> ((i >> 3) << lg)) & 1u) seg_grad[p0 * 8 + i] = sh.acc[(i & 7) * 32 + (i >> 3)];
+        if (gw && lane < slots && ((owned >> (lane << lg)) & 1u)) gw[p0 + lane] = (float)sh.acc[7 * 32 + lane];
     }
 }
 
@@ -1040,19 +1056,37 @@ inline unsigned adjoint_blocks(uint32_t np, int lg, int warps) {
     return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((w + warps - 1) / warps, (uint64_t)vx::kSMs * 64));
 }
 
-// Sum over the primitives of the voxels in their ranges (each at most 2^31): no window holds
-// more candidate pairs than that.
+// Sum over the primitives of their counts or, without counts, of the voxels in their ranges (each at
+// most 2^31): no window holds more candidate pairs than that.  *large is set when some primitive's walk
+// is too long for a share of a warp (see k_adjoint_fibers, k_adjoint_tris).
 template <bool FIBER>
 __global__ void k_range_bound(const float4* __restrict__ r0, const float4* __restrict__ r1, const float4* __restrict__ r2,
-                              uint32_t np, Window R, unsigned long long* __restrict__ total) {
+                              uint32_t np, Window R, const uint32_t* __restrict__ cnt,
+                              unsigned long long* __restrict__ total, uint32_t* __restrict__ large) {
     unsigned long long acc = 0;
+    bool any = false;
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < np; p += gridDim.x * blockDim.x) {
-        const Range rg = FIBER ? capsule_range(r0[p], r1[p], R) : tri_range(r0[p], r1[p], r2[p], R);
-        acc += (unsigned long long)min(rg.total, 0x80000000ll);
+        const float4 a = r0[p], b = r1[p];
+        const Range rg = FIBER ? capsule_range(a, b, R) : tri_range(a, b, r2[p], R);
+        acc += cnt ? (unsigned long long)cnt[p] : (unsigned long long)min(rg.total, 0x80000000ll);
+        any = any || (FIBER ? SegWalk::slabs(a, b, R.hi[0] + 1) > kWalkSlabs : rg.total > kGroupRange);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0 && acc) atomicAdd(total, acc);
+    if (any) *large = 1u;
+}
+
+// The gradients of all segments; `large`: some are left to a second launch.
+void adjoint_fibers(const float4* r0, const float4* r1, uint32_t np, int R, bool large, const uint64_t* keys0, uint32_t V0,
+                    const double* gm, const double* gM, double* seg_grad, float* gw, cudaStream_t s) {
+    const int lg = adjoint_lanes_log2(np);
+    const bool split = large && lg < 5;
+    k_adjoint_fibers<<<adjoint_blocks(np, lg, ADJ_WARPS), ADJ_WARPS * 32, 0, s>>>(
+        r0, r1, np, R, lg, 0, split ? kWalkSlabs : kAnyRange, keys0, V0, gm, gM, seg_grad, gw);
+    if (split)
+        k_adjoint_fibers<<<adjoint_blocks(np, 5, ADJ_WARPS), ADJ_WARPS * 32, 0, s>>>(
+            r0, r1, np, R, 5, kWalkSlabs + 1, kAnyRange, keys0, V0, gm, gM, seg_grad, gw);
 }
 
 // thread per control point: world-unit gradients from the segment before and after it
@@ -1284,14 +1318,17 @@ __device__ __forceinline__ bool tri_pair_grad(bool on, const float4 P0, const fl
 // Gradients of every triangle (world units, [T][3] float4 with w = 0, and the weights), 32 >> lg
 // triangles per block of one warp: lanes test the voxels of their triangle's box and queue its
 // candidates, which are taken 32 at a time so that the FP64 work runs with full lanes; each
-// triangle's terms are added in the order in which its lanes found them.  One warp per block: its
+// triangle's terms are added in the order in which its lanes found them.  A launch takes the triangles
+// whose boxes hold [least, most] voxels: with fewer than 32 lanes each, one of more than kGroupRange
+// would keep the others waiting, and goes to a second launch with a warp each (100,000 triangles, 32 of
+// them 150 voxels wide: 33 ms, 763 ms on single lanes).  One warp per block: its
 // polygons take 23 KB of shared memory, which leaves eight resident per SM, enough for the FP64
 // pipe that bounds the kernel (76 % busy).  178,802 triangles at 256^3: 1.1 ms; 1.6 ms with the
 // crossings inside a loop over the edges, 1.8 ms with each lane clipping at its own pace, 10.1 ms for
 // a warp per triangle (eight pairs in its lanes), six planes and polygons in local memory.
 __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ r0, const float4* __restrict__ r1,
                                                      const float4* __restrict__ r2, uint32_t np, Window R, int lg,
-                                                     const uint64_t* __restrict__ keys0, uint32_t V0,
+                                                     int least, int most, const uint64_t* __restrict__ keys0, uint32_t V0,
                                                      const double* __restrict__ gm, const double* __restrict__ gM,
                                                      float scale, float4* __restrict__ gverts, float* __restrict__ gw) {
     __shared__ double poly[ADJ_POLY];
@@ -1311,6 +1348,10 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
             c = r2[p];
             rg = tri_range(a, b, c, R);
         }
+        const bool mine = p < np && capped_total(rg) >= least && capped_total(rg) <= most;
+        const uint32_t owned = __ballot_sync(0xffffffffu, mine);
+        if (owned == 0u) continue;
+        if (!mine) rg.total = 0;
         long long idx = sub;
 #pragma unroll
         for (int k = 0; k < 10; ++k) acc[k * 32 + lane] = 0.0;
@@ -1369,12 +1410,12 @@ __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ 
         __syncwarp();
         for (int i = lane; i < slots * 3; i += 32) {
             const int t = i / 3, j = i - 3 * t;
-            if (p0 + t < np)
+            if ((owned >> (t << lg)) & 1u)
                 gverts[(p0 + t) * 3 + j] =
                     make_float4((float)(acc[(3 * j) * 32 + t] * (double)scale), (float)(acc[(3 * j + 1) * 32 + t] * (double)scale),
                                 (float)(acc[(3 * j + 2) * 32 + t] * (double)scale), 0.0f);
         }
-        if (gw && lane < slots && p0 + lane < np) gw[p0 + lane] = (float)acc[9 * 32 + lane];
+        if (gw && lane < slots && ((owned >> (lane << lg)) & 1u)) gw[p0 + lane] = (float)acc[9 * 32 + lane];
     }
 }
 
@@ -1441,13 +1482,16 @@ extern "C" vx_status vx_backward(vx_context* ctx, const vx_primitives* prims, co
     unsigned long long* t64 = (unsigned long long*)(misc + 8);
     const unsigned bblocks = (unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8);
     if (fiber)
-        VX_LAUNCH(ctx, ST_COUNT, s, k_range_bound<true><<<bblocks, 256, 0, s>>>(r0, r1, nullptr, np, full, t64));
+        VX_LAUNCH(ctx, ST_COUNT, s, k_range_bound<true><<<bblocks, 256, 0, s>>>(r0, r1, nullptr, np, full, nullptr, t64,
+                                                                              misc + 15));
     else
-        VX_LAUNCH(ctx, ST_COUNT, s, k_range_bound<false><<<bblocks, 256, 0, s>>>(r0, r1, r2, np, full, t64));
+        VX_LAUNCH(ctx, ST_COUNT, s, k_range_bound<false><<<bblocks, 256, 0, s>>>(r0, r1, r2, np, full, nullptr, t64,
+                                                                               misc + 15));
     VX_CUDA_TRY(cudaGetLastError());
-    VX_TRY(vx_readback_async(ctx, 0, misc, 48, s));
+    VX_TRY(vx_readback_async(ctx, 0, misc, 64, s));
     VX_CUDA_TRY(cudaStreamSynchronize(s));
     if (((uint32_t*)ctx->host_pin)[0]) return VX_ERR_INVALID_ARG;
+    const bool large = ((uint32_t*)ctx->host_pin)[15] != 0;
     if (((const uint64_t*)ctx->host_pin)[4] > (uint64_t)std::min<int64_t>(ctx->max_pairs, kMaxPassPairs)) {
         std::vector<Leaf> leaves;
         const int lo0[3] = {0, 0, 0};
@@ -1455,16 +1499,21 @@ extern "C" vx_status vx_backward(vx_context* ctx, const vx_primitives* prims, co
     }
     // ---- gradients ------------------------------------------------------------------------
     const int lg = adjoint_lanes_log2(np);
+    const bool split = large && lg < 5;
     if (!fiber) {
         // (no sharing between triangles: no scatter)
         VX_LAUNCH(ctx, ST_REDUCE_TRIS, s, k_adjoint_tris<<<adjoint_blocks(np, lg, 1), 32, 0, s>>>(
-                                              r0, r1, r2, np, full, lg, keys0, V0, gm, gM, g.s, (float4*)grad_ctrl,
-                                              grad_weights));
+                                              r0, r1, r2, np, full, lg, 0, split ? kGroupRange : kAnyRange, keys0, V0, gm,
+                                              gM, g.s, (float4*)grad_ctrl, grad_weights));
+        if (split)
+            VX_LAUNCH(ctx, ST_REDUCE_TRIS, s, k_adjoint_tris<<<adjoint_blocks(np, 5, 1), 32, 0, s>>>(
+                                                  r0, r1, r2, np, full, 5, kGroupRange + 1, kAnyRange, keys0, V0, gm, gM,
+                                                  g.s, (float4*)grad_ctrl, grad_weights));
         VX_CUDA_TRY(cudaGetLastError());
         return VX_OK;
     }
-    VX_LAUNCH(ctx, ST_REDUCE_FIBERS, s, k_adjoint_fibers<<<adjoint_blocks(np, lg, ADJ_WARPS), ADJ_WARPS * 32, 0, s>>>(
-                                            r0, r1, np, (int)R, lg, keys0, V0, gm, gM, pgrad, grad_weights));
+    VX_LAUNCH(ctx, ST_REDUCE_FIBERS, s, adjoint_fibers(r0, r1, np, (int)R, large, keys0, V0, gm, gM, pgrad, grad_weights, s));
+    if (split) ctx->launches[ST_REDUCE_FIBERS] += 1;   // (two kernels in one bracket)
     // per-segment gradients to control points
     uint32_t* fs = (uint32_t*)ctx->ws[WS_FIBER_START].p;
     VX_LAUNCH(ctx, ST_FINALIZE, s, k_adjoint_ctrl<<<grid_for((size_t)P, 256), 256, 0, s>>>(
@@ -1594,10 +1643,10 @@ extern "C" vx_status vx_backward_noalloc(const vx_primitives* prims, const vx_gr
         k_count<true><<<count_blocks(np, turn ? 0 : clg), COUNT_WARPS * 32, 0, s>>>(
             r0, r1, nullptr, np, full_window((int)R), turn ? 0 : clg, turn ? kGroupRange + 1 : 0,
             turn || clg == 0 ? kAnyRange : kGroupRange, cnt, nullptr, 0u, misc + 14);
-        // the exact 64-bit total
+        // the exact 64-bit total, and whether a walk is long
         NA_TRY(cudaMemsetAsync(misc + 8, 0, 8, s));
-        k_sum_u64<<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
-            cnt, np, (unsigned long long*)(misc + 8));
+        k_range_bound<true><<<(unsigned)std::min<size_t>(grid_for(np, 256), (size_t)vx::kSMs * 8), 256, 0, s>>>(
+            r0, r1, nullptr, np, full_window((int)R), cnt, (unsigned long long*)(misc + 8), misc + 15);
         NA_TRY(cudaMemcpyAsync(host, misc, 64, cudaMemcpyDeviceToHost, s));
         NA_TRY(cudaStreamSynchronize(s));
         if (host[0]) return VX_ERR_INVALID_ARG;
@@ -1606,9 +1655,7 @@ extern "C" vx_status vx_backward_noalloc(const vx_primitives* prims, const vx_gr
     }
     if (npairs64 > NA_MAX_PAIRS) return VX_ERR_CAPACITY;
     // the caller's outputs are written only once every limit has passed
-    const int lg = adjoint_lanes_log2(np);
-    k_adjoint_fibers<<<adjoint_blocks(np, lg, ADJ_WARPS), ADJ_WARPS * 32, 0, s>>>(r0, r1, np, (int)R, lg, keys0, V0, gm,
-                                                                                  gM, seg_grad, grad_weights);
+    adjoint_fibers(r0, r1, np, (int)R, host[15] != 0, keys0, V0, gm, gM, seg_grad, grad_weights, s);
     k_adjoint_ctrl<<<grid_for((size_t)P, 256), 256, 0, s>>>(prims->fiber_offsets, F, fs, P, seg_grad, g.s,
                                                              (float4*)grad_ctrl);
     NA_TRY(cudaGetLastError());

@@ -83,3 +83,78 @@ def test_one_lane_per_primitive(kind, n, R, size):
         assert bool(((got - ref).abs() <= 2.0 ** -23 * size).all())
         assert int((size > 0).sum()) > n // 2
     ctx.close()
+
+
+def _with_large(kind, n, R, rng, extent, count, at):
+    """Small primitives with `count` large ones (`extent` voxels long or wide) from place `at`."""
+    prims = _segments(n, R, rng, (0.1, 2.0)) if kind == "fibers" else _triangles(n, R, rng, (0.1, 2.0))
+    lo, hi = extent / 2 / R + 0.01, 1.0 - extent / 2 / R - 0.01
+    c = rng.uniform(lo, hi, (count, 3))
+    h = rng.uniform(-0.5, 0.5, (count, 3, 3)) * extent / R
+    h[:, 0], h[:, 1] = -0.5 * extent / R, 0.5 * extent / R
+    prims[at:at + count, :, :3] = c[:, None, :] + h[:, :prims.shape[1]]
+    return prims
+
+
+@pytest.mark.parametrize("kind,n,extent,count,at", [
+    ("fibers", 77824, 100.0, 40, 100),          # above 64 slabs, in a row, across two warps
+    ("fibers", 30000, 63.5, 33, 29967),         # about 64 slabs; the last, short group
+    ("triangles", 77824, 40.0, 40, 100),
+    ("triangles", 20000, 13.0, 33, 19967),      # about 2,048 voxels
+])
+def test_large_among_small(kind, n, extent, count, at):
+    """As above with primitives whose walk is left to a second launch."""
+    R = 128
+    rng = np.random.default_rng(n + 1)
+    prims = _with_large(kind, n, R, rng, extent, count, at)
+    weights = rng.uniform(0.5, 2.0, n).astype(np.float32)
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    ctx = vx.Context(DEV)
+    geom = _geom(kind, prims, weights)
+    keys = ctx.voxelize(grid, **geom).keys.clone()
+    gm, gM = _level_gradients(keys, 4, rng)
+    whole = _rows(kind, ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **geom))
+    for b in (at, max(0, at - 1900), 0):
+        part = _geom(kind, prims[b:b + 2000], weights[b:b + 2000])
+        ref = _rows(kind, ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **part))
+        for got, r in zip(whole, ref):
+            m = r.shape[0]
+            size = r.abs().reshape(m, -1).amax(1).reshape(m, *[1] * (r.dim() - 1))
+            assert bool(((got[b:b + m] - r).abs() <= 2.0 ** -23 * size).all())
+    ctx.close()
+
+
+def _time(call):
+    for _ in range(2):
+        call()
+    times = []
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        call()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return min(times)
+
+
+@pytest.mark.parametrize("kind,extent", [("fibers", 200.0), ("triangles", 100.0)])
+def test_large_ones_do_not_wait_for_one_lane(kind, extent):
+    """90,000 small primitives and 32 large ones take about as long as the two apart (one lane on a large
+    triangle took 32 times as long as its warp)."""
+    R, n, count = 256, 90000, 32
+    rng = np.random.default_rng(3)
+    prims = _with_large(kind, n, R, rng, extent, count, 500)
+    weights = np.ones(n, np.float32)
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    ctx = vx.Context(DEV)
+    geom = _geom(kind, prims, weights)
+    keys = ctx.voxelize(grid, **geom).keys.clone()
+    gm, gM = _level_gradients(keys, 0, rng)
+    few = slice(500, 500 + count)
+    rest = np.concatenate([prims[:500], prims[500 + count:]])
+    times = [_time(lambda g=g: ctx.backward(grid, keys0=keys, grad_mass=gm, grad_moment=gM, **g))
+             for g in (geom, _geom(kind, rest, weights[count:]), _geom(kind, prims[few], weights[few]))]
+    print(kind, times)
+    assert times[0] < 2.0 * (times[1] + times[2])
+    ctx.close()
