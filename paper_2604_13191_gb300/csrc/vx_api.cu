@@ -64,18 +64,30 @@ void vx_record_cuda_error(vx_context* ctx, cudaError_t e, const char* what) {
     snprintf(ctx->last_err, sizeof(ctx->last_err), "%s: %s", what, cudaGetErrorString(e));
 }
 
-void* vx_dev_alloc(vx_context* ctx, size_t bytes, cudaStream_t s) {
-    if (bytes == 0) bytes = 256;
+static void* dev_alloc_once(vx_context* ctx, size_t bytes, cudaStream_t s) {
     if (ctx->own_alloc) {
         void* p = nullptr;
         cudaError_t e = cudaMallocAsync(&p, bytes, s);
         if (e != cudaSuccess) {
             vx_record_cuda_error(ctx, e, "cudaMallocAsync");
+            cudaGetLastError();   // (a caller that goes on must not find it after its next launch)
             return nullptr;
         }
         return p;
     }
     return ctx->alloc.alloc(ctx->alloc.ctx, bytes, (void*)s);
+}
+
+void* vx_dev_alloc(vx_context* ctx, size_t bytes, cudaStream_t s) {
+    if (bytes == 0) bytes = 256;
+    void* p = dev_alloc_once(ctx, bytes, s);
+    if (p || !ctx->ws[WS_BALLOTS].p) return p;
+    // the ballots only spare the emit pass its tests: they give way (a launch that reads them is ahead
+    // on the stream)
+    vx_dev_free(ctx, ctx->ws[WS_BALLOTS].p, s);
+    ctx->ws[WS_BALLOTS] = vx::Buf();
+    ctx->ballots = nullptr;
+    return dev_alloc_once(ctx, bytes, s);
 }
 
 void vx_dev_free(vx_context* ctx, void* p, cudaStream_t s) {

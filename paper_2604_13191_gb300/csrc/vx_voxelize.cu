@@ -30,16 +30,18 @@
 namespace {
 
 // The count pass's ballot store (WS_BALLOTS) in *out and its words per primitive in *stride: 64 (ranges
-// of up to 2048 voxels, a capsule of 5 voxels' radius), 32 or 8, the most that takes at most 256 MB;
-// NULL when 8 take more (the emit pass then tests every voxel again).  A range's unused words
-// are never touched.  Errors: VX_ERR_OUT_OF_MEMORY, as for any workspace.
+// of up to 2048 voxels, a capsule of 5 voxels' radius), 32 or 8, the most that takes at most 256 MB and
+// that there is memory for; NULL when 8 take more than 256 MB (the emit pass then tests every voxel
+// again).  A range's unused words are never touched.  Errors: VX_ERR_OUT_OF_MEMORY without memory for 8.
 vx_status window_ballots(vx_context* ctx, uint32_t np, cudaStream_t s, uint32_t** out, uint32_t* stride) {
     *out = nullptr;
     *stride = 0;
     for (uint32_t words : {64u, 32u, 8u}) {
         const size_t bytes = (size_t)np * words * 4;
         if (bytes > ((size_t)256 << 20)) continue;
-        VX_TRY(vx_ws_ensure(ctx, WS_BALLOTS, bytes, s));
+        const vx_status st = vx_ws_ensure(ctx, WS_BALLOTS, bytes, s);
+        if (st == VX_ERR_OUT_OF_MEMORY && words > 8) continue;
+        VX_TRY(st);
         *out = (uint32_t*)ctx->ws[WS_BALLOTS].p;
         *stride = words;
         break;
@@ -73,10 +75,10 @@ vx_status count_window(vx_context* ctx, bool fiber, uint32_t np, const Window& w
     auto pass = [&](int lg, int least, int most, uint32_t* raise) -> vx_status {
         if (fiber)
             VX_LAUNCH(ctx, ST_COUNT, s, k_count<true><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
-                                            r0, r1, r2, np, win, lg, least, most, cnt, ballots, stride, raise));
+                                            r0, r1, r2, np, win, lg, least, most, cnt, ctx->ballots, stride, raise));
         else
             VX_LAUNCH(ctx, ST_COUNT, s, k_count<false><<<count_blocks(np, lg), COUNT_WARPS * 32, 0, s>>>(
-                                            r0, r1, r2, np, win, lg, least, most, cnt, ballots, stride, raise));
+                                            r0, r1, r2, np, win, lg, least, most, cnt, ctx->ballots, stride, raise));
         bool done = false;
         VX_TRY(vx_scan_u32(ctx, cnt, offs, np, misc + 1, s, t64, vx_pin_of(ctx, misc, 16), &done));
         if (!done) {   // no primitives

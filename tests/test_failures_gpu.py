@@ -133,3 +133,67 @@ def test_build_lod_events_rejects_bad_event_arguments():
         for k in ("keys", "mask", "mass", "moment", "occ", "proj", "lobe_count", "lobes"):
             assert np.array_equal(a[k], b[k]), k
     ctx.close()
+
+
+class LimitAllocator(api._TorchAllocator):
+    """torch's caching allocator behind a limit on the bytes held at one time, as a device's memory."""
+
+    def __init__(self, device, limit):
+        super().__init__(device)
+        self.limit, self.held, self.peak, self.sizes, self.refused = limit, 0, 0, {}, 0
+
+    def _alloc(self, ctx, nbytes, stream):
+        if self.held + int(nbytes) > self.limit:
+            self.refused += 1
+            return None
+        p = super()._alloc(ctx, nbytes, stream)
+        if p is not None:
+            self.sizes[p] = int(nbytes)
+            self.held += int(nbytes)
+            self.peak = max(self.peak, self.held)
+        return p
+
+    def _free(self, ctx, p, stream):
+        self.held -= self.sizes.pop(p, 0)
+        super()._free(ctx, p, stream)
+
+    def take(self, p):                 # a level handed to the caller, who drops it before the next call
+        self.held -= self.sizes.pop(p, 0)
+        return super().take(p)
+
+
+def _limit_context(limit):
+    ctx = vx.Context.__new__(vx.Context)
+    ctx.lib = vx.load()
+    ctx.device = DEV
+    ctx.alloc = LimitAllocator(DEV, limit)
+    h = C.c_void_p()
+    assert ctx.lib.vx_context_create(C.byref(ctx.alloc.struct), C.byref(h)) == 0
+    ctx.h = h
+    return ctx
+
+
+@pytest.mark.parametrize("kind,words", [("small", 64), ("small", 56), ("wide", 64), ("wide", 56)])
+def test_ballots_give_way_to_memory(kind, words):
+    """The count pass's ballots (up to 64 words per primitive) only spare the emit pass its tests: without
+    memory for them, or for what comes after them, they become fewer or none.  The limit is the call's
+    peak less `words` of them: 56 is what a store of 8 words needs.  `small` has little else to hold,
+    so that the 64 words are refused outright; `wide` holds most in the pairs that come later."""
+    R = 64
+    n = 200000 if kind == "small" else 20000
+    rng = np.random.default_rng(n)
+    v = rng.uniform(0.1, 0.9, (n, 1, 3)) + rng.uniform(-0.5, 0.5, (n, 3, 3)) * ((0.02 if kind == "small" else 5.0) / R)
+    tris = np.zeros((n, 3, 4), np.float32)
+    tris[..., :3] = v
+    geom = torch.from_numpy(tris).to(DEV)
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    probe = _limit_context(1 << 50)
+    ref = probe.voxelize(grid, tri_verts=geom).host()
+    ctx = _limit_context(probe.alloc.peak - int(n * words * 4))
+    for _ in range(2):
+        got = ctx.voxelize(grid, tri_verts=geom).host()
+        for f in ("keys", "mask", "mass", "moment", "occ", "proj", "lobes"):
+            assert np.array_equal(np.asarray(got[f]).view(np.uint8), np.asarray(ref[f]).view(np.uint8)), f
+    assert ctx.alloc.refused > 0
+    ctx.close()
+    probe.close()
