@@ -850,7 +850,9 @@ template <int RB>
 vx_status sort_pass(vx_context* ctx, uint32_t** keys, uint32_t** vals, uint32_t** keys_alt, uint32_t** vals_alt,
                     uint32_t n, int shift, uint32_t dmask, uint32_t nt, uint32_t* hist, cudaStream_t s,
                     uint32_t* err) {
-    static bool attr_set = false;   // dynamic shared memory of the scatter, once per process
+    // dynamic shared memory of the scatter: an attribute of the kernel on the device (and in the CUDA
+    // context) that this context lives in, so it is remembered here and not for the process
+    bool& attr_set = ctx->sort_smem_set[RB == 512];
     if (!attr_set) {
         VX_CUDA_TRY(cudaFuncSetAttribute(k_radix_scatter_pipe<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)pipe_smem(RB)));
