@@ -561,6 +561,8 @@ __device__ __noinline__ bool family_exact(float4 a, float4 b, float4 c, int vi, 
 //     of the bounds a bound is uncertain by less than delta = 20 u |inv| + 5 u (9 + 2 r) + 8 u.
 //   inv == 0 (alpha below 1e-4): the row passes or fails as a whole by the sign of half - |beta i1 +
 //     gamma|, times 1e9 in the place of r; uncertain when it is within near = 7 |alpha| + 23 u.
+// An edge parallel to the family's axis (s0 = s1 = 0; every edge of a box, two of three of a flat sheet)
+// never separates: T = 0 against a half of 1 passes every row.
 struct EdgeAxis {
     float inv, beta, gamma, half, r, scale, near;
 };
@@ -571,14 +573,15 @@ __device__ __forceinline__ EdgeAxis edge_axis(const float v0[3], const float v1[
 #pragma unroll
     for (int k = 0; k < 3; ++k) p[k] = s1 * (v1[k] - e) + s0 * (v0[k] - e);
     const float mn = fminf(fminf(p[0], p[1]), p[2]), mx = fmax3(p[0], p[1], p[2]);
-    const float B = fabsf(s0) * V0 + fabsf(s1) * V1;
-    fit = fit && B > 1e-30f && B < 1e30f;   // nothing overflows, underflows or is NaN
+    // (the 2e-30 makes the scaled half of a zero axis 1, and is below u^2 of any other that fits)
+    const float l1 = fabsf(s0) + fabsf(s1), B = __fmaf_rn(fabsf(s0), V0, __fmaf_rn(fabsf(s1), V1, 2e-30f));
+    fit = fit && (B > 1e-15f || l1 == 0.0f) && B < 1e30f;   // nothing overflows, underflows or is NaN
     const float q = vx_rcp(B);
     const float alpha = -0.125f * s0 * q;
     EdgeAxis a;
     a.beta = -0.125f * s1 * q;
     a.gamma = 0.5f * (mn + mx) * q;
-    a.half = (e * (fabsf(s0) + fabsf(s1)) + 0.5f * (mx - mn)) * q;
+    a.half = __fmaf_rn(e, l1, __fmaf_rn(0.5f, mx - mn, 2e-30f)) * q;
     const bool row = fabsf(alpha) < 1e-4f;
     a.inv = row ? 0.0f : vx_rcp(alpha);
     a.r = a.half * fabsf(a.inv);

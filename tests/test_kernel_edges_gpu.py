@@ -292,3 +292,58 @@ def test_capsule_radius_whose_square_overflows(a, b, r):
     assert np.array_equal(got["keys"].astype(np.uint64), key[order])
     assert np.array_equal(got["mask"].view(np.uint64).reshape(-1, 8), words[order])
     ctx.close()
+
+
+def _sheet(n, axis, level, lo, hi):
+    """n x n vertices of a plane sheet at right angles to `axis`, two triangles per cell."""
+    u = np.linspace(lo, hi, n)
+    P = np.full((n, n, 3), level)
+    P[..., (axis + 1) % 3], P[..., (axis + 2) % 3] = u[None, :], u[:, None]
+    a, b, c, d = P[:-1, :-1], P[:-1, 1:], P[1:, 1:], P[1:, :-1]
+    t = np.zeros((n - 1, n - 1, 2, 3, 4), np.float32)
+    t[..., 0, 0, :3], t[..., 0, 1, :3], t[..., 0, 2, :3] = a, b, c
+    t[..., 1, 0, :3], t[..., 1, 1, :3], t[..., 1, 2, :3] = a, c, d
+    return t.reshape(-1, 3, 4)
+
+
+@pytest.mark.parametrize("n,R,level,lo,hi", [
+    (30, 16, 0.3337, 0.06, 0.94),     # edges along two axes, nothing on a plane
+    (17, 16, 0.5, 0.0, 1.0),          # everything on voxel planes
+    (30, 16, 17 / 128, 0.06, 0.94),   # the sheets on sub-cell planes
+    (3, 32, 0.61, 0.1, 0.9),          # edges of many voxels
+])
+def test_edges_along_the_axes(n, R, level, lo, hi):
+    """A box's faces: edges parallel to an axis (their edge axis in that family is zero, and separates
+    nothing) and diagonals in the coordinate planes."""
+    tris = np.concatenate([_sheet(n, ax, z, lo, hi) for ax in range(3) for z in (level, 1.0 - level)])
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    ctx = vx.Context(DEV)
+    got = ctx.voxelize(grid, tri_verts=torch.from_numpy(tris).to(DEV))
+    _same_level0(got, oracle.voxelize(synth.Workload("box", "triangles", grid, tri_verts=tris, K=1)))
+    ctx.close()
+
+
+def test_edges_along_the_axes_cost_nothing():
+    """A flat sheet whose edges lie along the axes takes no longer than the same sheet turned a little (its
+    zero edge axes sent every row to the definition, and the sheet took 1.3 times as long)."""
+    n, R = 2048, 1024
+    flat = _sheet(n, 2, 0.50031, 0.05, 0.95)
+    turned = flat.copy()
+    turned[..., 0], turned[..., 1] = flat[..., 0] + 0.01 * flat[..., 1], flat[..., 1] - 0.01 * flat[..., 0]
+    turned[..., 2] += 0.01 * (flat[..., 0] - flat[..., 1])
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    ctx = vx.Context(DEV)
+    best = []
+    for t in (flat, turned):
+        geom = torch.from_numpy(t).to(DEV)
+        times = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ctx.voxelize(grid, tri_verts=geom)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        best.append(min(times))
+    assert best[0] < 1.15 * best[1], best
+    ctx.close()
