@@ -783,7 +783,7 @@ __device__ __forceinline__ int clip_plane_s(float* __restrict__ buf, int pi, int
         const bool ein = ge ? (Ea >= c) : (Ea <= c);
         if (sin_ != ein) {
             const float num = c - Sa, den = Ea - Sa;
-            const float sv = fabsf(num) >= 1e-24f && fabsf(den) <= 1e30f ? vx_div(num, den) : num / den;
+            const float sv = fabsf(num) >= 1e-24f && fabsf(den) <= 1e12f ? vx_div(num, den) : num / den;
 #pragma unroll
             for (int j = 0; j < 3; ++j) at(po, m, j) = (j == axis) ? c : S[j] + sv * (E[j] - S[j]);
             ++m;

@@ -407,7 +407,7 @@ __device__ bool sqrtm3(const float* S, float* Rm) {
             const float d = aqq - app, e = 2.0f * apq;
             const float dd = d * d + e * e;
             float t;
-            if (dd >= 1e-30f && dd <= 1e30f && fabsf(e) >= 1e-24f)
+            if (dd >= 1e-30f && dd <= 1e20f && fabsf(e) >= 1e-24f)
                 t = vx_div(e, fabsf(d) + vx_sqrt(dd));
             else
                 t = e / (fabsf(d) + sqrtf(dd));
