@@ -347,3 +347,23 @@ def test_edges_along_the_axes_cost_nothing():
         best.append(min(times))
     assert best[0] < 1.15 * best[1], best
     ctx.close()
+
+
+@pytest.mark.parametrize("kind,R", [("tri", 4), ("tri", 8), ("tri", 64), ("cap", 4), ("cap", 8), ("cap", 64)])
+def test_one_primitive_with_extent(kind, R):
+    """The smallest batch and the shortest group: one pair's lane, or one primitive in every voxel."""
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    if kind == "tri":
+        tris = np.array([[[1.2, 1.3, 1.25, 0.0], [1.9, 1.4, 1.8, 0.0], [1.3, 2.6, 1.6, 0.0]]], np.float32) / np.float32(R)
+        w = synth.Workload("one", "triangles", grid, tri_verts=tris, K=1)
+        geom = dict(tri_verts=torch.from_numpy(tris).to(DEV))
+    else:
+        ctrl = np.array([[1.3, 1.4, 1.6, 0.2], [1.7, 2.6, 1.4, 0.3]], np.float32) / np.float32(R)
+        off = np.array([0, 2], np.int64)
+        w = synth.Workload("one", "fibers", grid, ctrl=ctrl, fiber_offsets=off, K=1)
+        geom = dict(ctrl=torch.from_numpy(ctrl).to(DEV), fiber_offsets=torch.from_numpy(off).to(DEV))
+    ref = oracle.voxelize(w)
+    assert ref["keys"].shape[0] >= 2 and float(ref["mass"].min()) >= 0.0 and float(ref["mass"].sum()) > 0.1
+    ctx = vx.Context(DEV)
+    _same_level0(ctx.voxelize(grid, **geom), ref)
+    ctx.close()
