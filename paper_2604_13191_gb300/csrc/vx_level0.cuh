@@ -210,16 +210,10 @@ __device__ __forceinline__ CapsuleX capsule_x(float a, float b) {
 // A radius whose square overflows leaves r^2 = inf, and steps 1 and 2 then hold for a whole row when
 // its y and z terms have a finite sum (anything <= inf) and for none of it otherwise (inf - inf is not a
 // number, and no comparison with that holds).  capsule_row compares by the sign of a difference, which is
-// undefined for inf - inf, so such a slot gets the largest finite value in r^2's place, which no FP32
-// square rounds to, and x terms of zero: the budget is then at least zero in the one case and -inf in
-// the other.  Step 3 takes r^2 back (slot_rr).
+// undefined for inf - inf, so it takes at most the largest finite value for r^2, and such a capsule's x
+// terms are zero (capsule_x of two NaN): the budget is then at least zero in the one case and -inf in the
+// other.
 constexpr float kHugeRR = 3.402823466e38f;
-__device__ __forceinline__ void slot_overflow(CapsuleSlot& cs) {
-    const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    cs.c.a_rr.w = kHugeRR;
-    for (int h = 0; h < 2; ++h) cs.x.g2[h] = cs.x.ea2[h] = cs.x.eb2[h] = zero;
-}
-__device__ __forceinline__ float slot_rr(const CapsuleLocal& c) { return c.a_rr.w == kHugeRR ? INFINITY : c.a_rr.w; }
 
 // Steps 1-2 of the capsule test for one row of 8 sub-cells (sx = 0..7 at sy; tz: the z terms of
 // its slab).  `set` receives the sub-cells that step 2 decides set, `open` those that pass step 1.
@@ -232,7 +226,7 @@ __device__ __forceinline__ float slot_rr(const CapsuleLocal& c) { return c.a_rr.
 __device__ __forceinline__ void capsule_row(const CapsuleSlot& cs, const AxisTerms& tz, int sy, uint32_t& set,
                                             uint32_t& open) {
     const AxisTerms ty = axis_terms(cs.c.a_rr.y, cs.c.b_reta.y, sy);
-    const float rr = cs.c.a_rr.w;
+    const float rr = fminf(cs.c.a_rr.w, kHugeRR);
     const float TG = rr - (ty.g2 + tz.g2);
     const float TA = rr - (ty.ea2 + tz.ea2);
     const float TB = rr - (ty.eb2 + tz.eb2);
@@ -242,7 +236,7 @@ __device__ __forceinline__ void capsule_row(const CapsuleSlot& cs, const AxisTer
     const float xa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
     const float xb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
     // a comparison x <= T by the sign of T - x (the exact sign of the difference; T and x are not
-    // both infinite with one sign, see slot_overflow), shifted into a word: additions run on the FMA pipe, where compares and selects load the ALU pipe, the busier
+    // both infinite with one sign, see kHugeRR), shifted into a word: additions run on the FMA pipe, where compares and selects load the ALU pipe, the busier
     uint32_t out = 0, shut = 0;
 #pragma unroll
     for (int sx = 7; sx >= 0; --sx) {
@@ -426,7 +420,7 @@ __device__ __forceinline__ uint32_t capsule_step3_pool(CapsuleTasks& ct, int nta
         const CapsuleLocal& c = ct.slot[task >> 9].c;
         const int sx = id & 7, sy = (id >> 3) & 7, zz = id >> 6;
         if (seg_box_min(c.a_rr.x, c.a_rr.y, c.a_rr.z, c.d_idd.x, c.d_idd.y, c.d_idd.z, (float)sx * 0.125f,
-                        (float)sy * 0.125f, (float)zz * 0.125f, 0.125f) <= slot_rr(c))
+                        (float)sy * 0.125f, (float)zz * 0.125f, 0.125f) <= c.a_rr.w)
             atomicOr(&ct.mask[id >> 5], bit);
     }
     __syncwarp();
@@ -1697,8 +1691,8 @@ __global__ void __launch_bounds__(RED_WARPS * 32, 7) k_reduce_fibers(const uint3
                     if (live) {
                         const CapsuleLocal cl = capsule_local(a, b, A.w);
                         ct.slot[lane].c = cl;
-                        ct.slot[lane].x = capsule_x(a[0], b[0]);
-                        if (cl.a_rr.w > kHugeRR) slot_overflow(ct.slot[lane]);
+                        const bool huge = cl.a_rr.w > kHugeRR;
+                        ct.slot[lane].x = capsule_x(huge ? NAN : a[0], huge ? NAN : b[0]);
                         okey = capsule_order(cl);
                     }
                     // the voxel in the top bits (every key of a lane in use below the others')
