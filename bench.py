@@ -852,8 +852,8 @@ def roofline(prof, w, level_sizes, steps):
                 "launches_per_step": nl // steps, "units_per_launch": units_per_launch,
                 "ops_per_unit": ALU_OPS[stage], "issue_slots": issue,
                 "ops_note": "ops_per_unit counts the definition's FP32 operations (512 sub-cell tests of 10 "
-                            "operations per pair); the kernel skips most of them with exact group tests, so "
-                            "issue_slots says how busy the SM is",
+                            "operations per pair); the kernel skips most of them with exact group tests, so this "
+                            "fraction can pass 1, and issue_slots says how busy the SM is",
                 "peak_source": f"152 SMs x 128 FP32 lanes x {clk_mhz:.0f} MHz (max SM clock, MEASURED_PEAKS)"}
     per_unit = HBM_BYTES.get(stage)
     ach = None if per_unit is None else units_per_launch * per_unit / (avg_ms * 1e-3) / 1e9

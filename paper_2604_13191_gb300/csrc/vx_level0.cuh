@@ -1028,7 +1028,7 @@ __device__ __forceinline__ bool tri_voxel_candidate(float4 a, float4 b, float4 c
 }
 
 // ------------------------------------------------------------------------------------
-// count / emit: warp per primitive over its voxel range
+// count / emit: the candidate voxels of every primitive's range
 // ------------------------------------------------------------------------------------
 // With `ballots`, the count pass stores each primitive's hit ballots (one word per 32 voxels
 // of its range, ranges of at most 32 * stride voxels) and the emit pass of the same
@@ -1458,9 +1458,6 @@ __global__ void __launch_bounds__(EMIT_WARPS * 32) k_candidates(const float4* __
 }
 
 // ------------------------------------------------------------------------------------
-// segments
-// ------------------------------------------------------------------------------------
-// ------------------------------------------------------------------------------------
 // reduce: warp per candidate voxel
 // lane l owns sub-cells sz = l >> 2, sy = 2 (l & 3) + {0,1}, sx = 0..7 (16 bits)
 // ------------------------------------------------------------------------------------
@@ -1588,7 +1585,7 @@ __device__ __forceinline__ uint32_t voxel_mask(CapsuleTasks& ct, uint32_t okey, 
 // A voxel of more than 32 capsules is a group of its own and runs in batches of 32.  The setup
 // and the mask steps each have one call site, so that the kernel holds one copy of them.
 // Issue-bound (80 % of slots; DRAM at the definition's bytes).  768k capsules at 512^3, 75 M pairs:
-// 10.4 ms against 18.9 ms when every capsule ran steps 1-2 on every row; a yarn of 4-voxel
+// 9.8 ms against 18.9 ms when every capsule ran steps 1-2 on every row; a yarn of 4-voxel
 // radius at 1024^3, 107 M pairs, four of five voxels covered: 5.2 ms against 9.6 ms.  Of 46 M
 // capsules tested, 24 % reach a row and 40 rows per 100 run.  7 blocks per SM (72 registers,
 // 24 words spilled) ran the 1024^3 yarn in 5.2 ms, 6 blocks in 5.4 ms.

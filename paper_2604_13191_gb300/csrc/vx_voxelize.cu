@@ -3,9 +3,11 @@
 //
 // Pipeline (one stream):
 //   prep      per primitive: grid coordinates (Sec. 3.1, P_volume), weights
-//   count     warp per primitive: conservative voxel test over its bounding box
+//   count     up to 32 primitives per warp: conservative voxel test over their bounding boxes, by a
+//             record per primitive, its hits kept as ballots (large boxes: a warp each)
 //   scan      exclusive offsets of the per-primitive candidate counts
-//   emit      warp per primitive: (Morton key, primitive id) pairs, ballot-compacted
+//   emit      (Morton key, primitive id) pairs from the ballots, 32 primitives per warp (those without
+//             ballots: a warp each, tested again)
 //   sort      stable LSD radix sort by key (Sec. 3.3: samples ordered by block id)
 //   heads     segment starts where the key changes (Sec. 3.3)
 //   reduce    warp per voxel: exact sub-cell masks (OR over primitives), mass and
@@ -724,7 +726,8 @@ inline size_t adj_part_bytes(uint32_t n, int L) { return ((size_t)n / ADJ_TILE +
 
 // FP64 operations of the adjoint are few per clock (two lanes per SM), so what can run elsewhere
 // does: reciprocals and inverse roots start from the special-function unit's approximation and take
-// two Newton steps (relative error below 2^-51; no bit-exact contract here), and comparisons of
+// two steps of Newton's iteration (y + y (1 - x y) and y + y (1/2 - x y^2 / 2); relative error below
+// 2^-51; no bit-exact contract here), and comparisons of
 // doubles whose order is that of their bits as integers run as integers.
 __device__ __forceinline__ double d_rcp(double x) {
     double y;
