@@ -1160,7 +1160,7 @@ __device__ __forceinline__ bool tri_pair_grad(bool on, const float4 P0, const fl
         if (fminf(fminf(U[0][k], U[1][k]), U[2][k]) < (float)vox[k]) need |= 1u << (2 * k);
         if (fmaxf(fmaxf(U[0][k], U[1][k]), U[2][k]) > (float)(vox[k] + 1)) need |= 2u << (2 * k);
 #pragma unroll
-        for (int v = 0; v < 3; ++v) at(0, v, k) = (double)U[v][k] - vox[k];
+        for (int v = 0; v < 3; ++v) at(0, v, k) = (double)(U[v][k] + 0.0f) - vox[k];   // (-0 becomes +0)
     }
     at(0, 0, 3) = 0.0; at(0, 0, 4) = 0.0;
     at(0, 1, 3) = 1.0; at(0, 1, 4) = 0.0;
@@ -1174,7 +1174,8 @@ __device__ __forceinline__ bool tri_pair_grad(bool on, const float4 P0, const fl
         const int c = work ? __ffs(need) - 1 : 0, k = c >> 1;
         need &= need - 1u;
         const bool hi = c & 1;
-        // inside x >= 0 (x <= 1), on the bits as integers: the polygon holds no negative zero
+        // inside x >= 0 (x <= 1), on the bits as integers: the polygon holds no negative zero (the
+        // sums below give none from values that are none)
         uint32_t in = 0;
         if (work)
             for (int i = 0; i < n; ++i) {
