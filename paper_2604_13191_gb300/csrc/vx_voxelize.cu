@@ -909,10 +909,11 @@ struct SegWalk {
         const float e0 = fabsf(b.x - a.x), e1 = fabsf(b.y - a.y), e2 = fabsf(b.z - a.z);
         return e0 >= e1 && e0 >= e2 ? 0 : (e1 >= e2 ? 1 : 2);
     }
-    // number of slabs of a segment, and the first
+    // number of slabs of a segment, and the first: an end on a plane belongs to the slabs on both sides
+    // (the rounding of the clip decides which of them holds it)
     static __device__ __forceinline__ int slabs(float4 a, float4 b, int R, int m, int& first) {
         const float am = sel3(m, a.x, a.y, a.z), bm = sel3(m, b.x, b.y, b.z);
-        first = clampi(floorf(fminf(am, bm)), 0, R);
+        first = clampi(ceilf(fminf(am, bm)) - 1.0f, 0, R);
         return max(clampi(floorf(fmaxf(am, bm)), -1, R - 1) - first + 1, 0);
     }
     static __device__ __forceinline__ int slabs(float4 a, float4 b, int R) {

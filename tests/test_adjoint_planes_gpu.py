@@ -149,3 +149,49 @@ def test_triangles_on_the_grid(snap, lanes):
         assert np.abs(g[i] - ref * float(w[i]) * R).max() <= 2.0 ** -22 * (size * float(w[i]) * R) + 1e-12, i
         assert abs(gw[i] - val) <= 2.0 ** -22 * big + 1e-12, i
     ctx.close()
+
+
+@pytest.mark.parametrize("lanes", [5, 0])
+@pytest.mark.parametrize("snap", [0, 1, 8])
+def test_segment_ends_on_planes(snap, lanes):
+    """With one loss weight for every voxel the loss is that weight times pi r^2 |B - A| (times the segment's
+    weight), however the planes cut it: its gradients with respect to both ends, the radius and the weight.  Ends
+    lie on the planes of a box that cuts the segments off, or on multiples of 1 / snap.  FP64 sums of up to
+    50 pieces, whose sliding ends cancel from pieces up to 1 / 1e-3 larger: 1e-12 of the gradient, and the FP32
+    rounding (2^-24)."""
+    R, n = 16, (3000 if lanes == 5 else 80000)
+    rng = np.random.default_rng(snap + 7)
+    P = np.clip(rng.uniform(2, 14, (n, 1, 3)) + rng.uniform(-4, 4, (n, 2, 3)), 3, 13)
+    if snap:
+        P = np.round(P * snap) / snap
+    P = P.astype(np.float32)
+    # (a segment without length has no gradient; one in a voxel plane lies in the voxels on both sides)
+    flat = ((P[:, 0] == P[:, 1]) & (P[:, 0] == np.round(P[:, 0]))).any(1)
+    d = P[:, 1].astype(np.float64) - P[:, 0]
+    length = np.sqrt((d * d).sum(1))
+    # near-parallel to a plane: the pieces' sliding ends are large and cancel
+    steep = (np.abs(d) < 1e-3) & (d != 0)
+    use = ~flat & (length > 0.01) & ~steep.any(1)
+    assert use.sum() > n // 3
+    ctrl = np.zeros((n, 2, 4), np.float32)
+    ctrl[..., :3], ctrl[..., 3] = P / np.float32(R), np.float32(0.25 / R)
+    w = rng.uniform(0.5, 2.0, n).astype(np.float32)
+    grid = synth.Grid((0.0, 0.0, 0.0), 1.0 / R, R)
+    ctx = vx.Context(DEV)
+    geom = _geom("fibers", ctrl, w)
+    keys = ctx.voxelize(grid, **geom).keys.clone()
+    ones, none = torch.ones(keys.shape[0], device=DEV), torch.zeros(keys.shape[0], 6, device=DEV)
+    g, gw = ctx.backward(grid, keys0=keys, grad_mass=[ones], grad_moment=[none], **geom)
+    g, gw = g.cpu().numpy().reshape(n, 2, 4).astype(np.float64), gw.cpu().numpy().astype(np.float64)
+    r = 0.25
+    c = np.pi * r * r * w.astype(np.float64) * R
+    with np.errstate(invalid="ignore", divide="ignore"):
+        t = d / length[:, None]
+    for got, ref in ((g[:, 0, :3], -c[:, None] * t), (g[:, 1, :3], c[:, None] * t)):
+        assert np.abs(got - ref)[use].max(1).max() <= 2.0 ** -22 * c.max()
+    half = 0.5 * 2.0 * np.pi * r * length * w * R
+    for e in range(2):
+        assert (np.abs(g[:, e, 3] - half) <= 2.0 ** -22 * half + 1e-9)[use].all()
+    mass = np.pi * r * r * length
+    assert (np.abs(gw - mass) <= 2.0 ** -22 * mass + 1e-9)[use].all()
+    ctx.close()
