@@ -1150,7 +1150,8 @@ __global__ void k_adjoint_ctrl(const int64_t* __restrict__ off, int64_t F, const
 // themselves (1 - 3 * fl(1/3) = 0, a * b - b * a = 0), and a fused operation leaves a residue that moves
 // an edge from one of two planes to the other, or gives an empty piece an area and a normal: of 323
 // triangles with whole coordinates the derivatives of the area over all voxels then missed that of the
-// whole for 40 instead of 13.  The mesh below takes 1.26 ms instead of 1.20 for it.
+// whole for 40 instead of 13.  They cost 0.06 ms of the mesh's
+// 1.17 below.
 // Only the planes that some vertex of the triangle lies beyond are clipped against.
 // buf: the warp's two polygons, ADJ_POLY doubles (element (poly, vertex, coord) of lane t at
 // [((poly * ADJ_VERTS + vertex) * 5 + coord) * 32 + t]); a vertex carries x, y, z (exact for the
@@ -1349,7 +1350,7 @@ __device__ __forceinline__ bool tri_pair_grad(bool on, const float4 P0, const fl
 // would keep the others waiting, and goes to a second launch with a warp each (100,000 triangles, 32 of
 // them 150 voxels wide: 33 ms, 763 ms on single lanes).  One warp per block: its
 // polygons take 23 KB of shared memory, which leaves eight resident per SM, enough for the FP64
-// pipe that bounds the kernel (76 % busy).  178,802 triangles at 256^3: 1.1 ms; 1.6 ms with the
+// pipe that bounds the kernel (77 % busy).  178,802 triangles at 256^3: 1.17 ms; 1.6 ms with the
 // crossings inside a loop over the edges, 1.8 ms with each lane clipping at its own pace, 10.1 ms for
 // a warp per triangle (eight pairs in its lanes), six planes and polygons in local memory.
 __global__ void __launch_bounds__(32) k_adjoint_tris(const float4* __restrict__ r0, const float4* __restrict__ r1,
