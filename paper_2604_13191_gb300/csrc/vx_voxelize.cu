@@ -1150,8 +1150,7 @@ __global__ void k_adjoint_ctrl(const int64_t* __restrict__ off, int64_t F, const
 // themselves (1 - 3 * fl(1/3) = 0, a * b - b * a = 0), and a fused operation leaves a residue that moves
 // an edge from one of two planes to the other, or gives an empty piece an area and a normal: of 323
 // triangles with whole coordinates the derivatives of the area over all voxels then missed that of the
-// whole for 40 instead of 13.  They cost 0.06 ms of the mesh's
-// 1.17 below.
+// whole for 40 instead of 13.  They cost 0.06 ms of the 1.17 that the mesh below takes.
 // Only the planes that some vertex of the triangle lies beyond are clipped against.
 // buf: the warp's two polygons, ADJ_POLY doubles (element (poly, vertex, coord) of lane t at
 // [((poly * ADJ_VERTS + vertex) * 5 + coord) * 32 + t]); a vertex carries x, y, z (exact for the
